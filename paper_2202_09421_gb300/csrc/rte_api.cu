@@ -51,6 +51,8 @@ struct rte_ctx {
   // and the test-only request that the next march's first pass time out
   DevBuf err;
   bool inject_expire = false;
+  // item counters of the multi-step launches
+  DevBuf ctl;
   // photon balance of the last rte_forward (RTE_FLAG_PHOTON_BALANCE):
   // [G][n_steps][3] FP64 terms, block partials, per-group tickets, and the
   // FP64 cos / sin of the ordinates
@@ -249,6 +251,28 @@ double angdist(double a, double b) {
   return std::min(d, 2.0 * kPi - d);
 }
 
+// Checkpoint of the march state (u, L) before step s (a multiple of the
+// checkpoint interval).
+rte_status copy_checkpoint(rte_ctx* c, const float* u, DevBuf* L, int hl, int G, int s) {
+  const size_t gbytes = static_cast<size_t>(G) * c->plane * sizeof(float);
+  char* base = static_cast<char*>(c->ckpt.p) + static_cast<size_t>(s / c->par.ckpt_interval) * 4 * gbytes;
+  const void* src[4] = {u, L[hl].p, L[(hl + 1) % 3].p, L[(hl + 2) % 3].p};
+  for (int q = 0; q < 4; ++q)
+    RTE_TRY(cuda_status(cudaMemcpyAsync(base + q * gbytes, src[q], gbytes, cudaMemcpyDeviceToDevice, c->stream)));
+  return RTE_OK;
+}
+
+// Fluence of state u (after step s) into its snapshot slot.
+rte_status snapshot(rte_ctx* c, const float* u, int G, const std::vector<int>& snap_index, int s,
+                    float* fluence_out) {
+  const size_t per = static_cast<size_t>(c->nx) * c->ny;
+  const int n_snaps =
+      static_cast<int>(std::count_if(snap_index.begin(), snap_index.end(), [](int v) { return v >= 0; }));
+  return cuda_status(rte_kern::launch_fluence(u, fluence_out + static_cast<size_t>(snap_index[s]) * per,
+                                              per * n_snaps, c->nx, c->ny, c->M, G, c->plane,
+                                              static_cast<float>(2.0 * kPi / c->M), c->stream, &c->launches));
+}
+
 // Runs steps [s_begin, s_end) of the forward march on (U, R, L), starting
 // from whatever state they hold; records checkpoints/exitance/fluence when
 // asked.
@@ -264,17 +288,53 @@ rte_status march(rte_ctx* c, DevBuf& U, DevBuf& R, DevBuf* L, int& hl, int G, in
   const bool fused = a.x_variant == 3 && rte_kern::fused_supported(a);
   float* cur = F(U);
   float* oth = F(R);
+  // Multi-step launches: runs of steps between checkpoints and snapshots.
+  // Without slots the state alternates between U and R, so that it ends in U
+  // (an odd number of steps starts from a copy in R).  Not on the adjoint's
+  // recompute stream: a launch that keeps every SM for a whole segment leaves
+  // nothing to overlap with the passes of the other stream.
+  const bool overlapped = c->astream && c->stream == c->astream;
+  if (!fused && !balance_out && !c->timing && !overlapped && rte_kern::tc_march_supported(a)) {
+    if (!seg_out && ((s_end - s_begin) & 1)) {
+      RTE_TRY(cuda_status(cudaMemcpyAsync(oth, cur, gbytes, cudaMemcpyDeviceToDevice, c->stream)));
+      std::swap(cur, oth);
+    }
+    rte_kern::MarchArgs ma;
+    ma.a = a;
+    ma.b = b;
+    ma.slots = nullptr;
+    ma.slot_floats = 0;
+    ma.dstep = 1;
+    ma.ctl = static_cast<int*>(c->ctl.p);
+    for (int q = 0; q < 3; ++q) ma.L[q] = F(L[q]);
+    for (int s = s_begin; s < s_end;) {
+      if (save_ckpt && I > 0 && s % I == 0) RTE_TRY(copy_checkpoint(c, cur, L, hl, G, s));
+      int e = s + 1;                                   // the run [s, e)
+      while (e < s_end && !(save_ckpt && I > 0 && e % I == 0) && !(fluence_out && snap_index[e - 1] >= 0)) ++e;
+      ma.u0 = cur;
+      ma.u1 = oth;
+      ma.hl = hl;
+      ma.step0 = s;
+      ma.n_steps = e - s;
+      if (seg_out) {
+        ma.slots = (*seg_out)[s - s_begin];
+        ma.slot_floats = static_cast<size_t>(G) * c->plane;
+      }
+      RTE_TRY(cuda_status(rte_kern::launch_march_tc(ma, c->stream, &c->launches)));
+      hl = (hl + 2 * (e - s)) % 3;
+      if (seg_out) cur = (*seg_out)[e - 1 - s_begin];
+      else if ((e - s) & 1) std::swap(cur, oth);
+      if (fluence_out && snap_index[e - 1] >= 0)
+        RTE_TRY(snapshot(c, cur, G, snap_index, e - 1, fluence_out));
+      s = e;
+    }
+    return RTE_OK;
+  }
   for (int s = s_begin; s < s_end; ++s) {
     float* L1 = F(L[hl]);
     float* L2 = F(L[(hl + 1) % 3]);
     float* L3 = F(L[(hl + 2) % 3]);
-    if (save_ckpt && I > 0 && s % I == 0) {
-      char* base = static_cast<char*>(c->ckpt.p) + static_cast<size_t>(s / I) * 4 * gbytes;
-      const void* src[4] = {cur, L1, L2, L3};
-      for (int q = 0; q < 4; ++q)
-        RTE_TRY(cuda_status(cudaMemcpyAsync(base + q * gbytes, src[q], gbytes,
-                                            cudaMemcpyDeviceToDevice, c->stream)));
-    }
+    if (save_ckpt && I > 0 && s % I == 0) RTE_TRY(copy_checkpoint(c, cur, L, hl, G, s));
     cudaEvent_t* ev = nullptr;
     if (c->timing) {
       while (c->events.size() < 3 * (c->n_timed + 1)) {
@@ -294,15 +354,7 @@ rte_status march(rte_ctx* c, DevBuf& U, DevBuf& R, DevBuf* L, int& hl, int G, in
                                                 &c->launches, ev)));
     }
     hl = (hl + 2) % 3;
-    if (fluence_out && snap_index[s] >= 0) {
-      const size_t per = static_cast<size_t>(c->nx) * c->ny;
-      const int n_snaps = static_cast<int>(std::count_if(snap_index.begin(), snap_index.end(),
-                                                         [](int v) { return v >= 0; }));
-      RTE_TRY(cuda_status(rte_kern::launch_fluence(
-          cur, fluence_out + static_cast<size_t>(snap_index[s]) * per, per * n_snaps, c->nx,
-          c->ny, c->M, G, c->plane, static_cast<float>(2.0 * kPi / c->M), c->stream,
-          &c->launches)));
-    }
+    if (fluence_out && snap_index[s] >= 0) RTE_TRY(snapshot(c, cur, G, snap_index, s, fluence_out));
     if (seg_out)
       RTE_TRY(cuda_status(cudaMemcpyAsync((*seg_out)[s - s_begin], cur, gbytes,
                                           cudaMemcpyDeviceToDevice, c->stream)));
@@ -414,6 +466,7 @@ rte_status prepare_forward(rte_ctx* c, const rte_source_group* groups, int n_gro
   RTE_TRY(ensure(c->U, gbytes));
   RTE_TRY(ensure(c->R, gbytes));
   for (int q = 0; q < 3; ++q) RTE_TRY(ensure(c->L[q], gbytes));
+  RTE_TRY(ensure(c->ctl, rte_kern::tc_march_ctl_bytes(G)));
   RTE_TRY(ensure(c->ring, static_cast<size_t>(G) * n_steps * c->ring_len * sizeof(float)));
   const int I = c->par.ckpt_interval;
   c->n_ckpt = I > 0 ? (n_steps + I - 1) / I : 0;
@@ -463,12 +516,7 @@ rte_kern::BoundaryArgs forward_bargs(rte_ctx* c) {
 rte_status save_checkpoint(rte_ctx* c, int s, int hl) {
   const int I = c->par.ckpt_interval;
   if (I <= 0 || s % I != 0) return RTE_OK;
-  const size_t gbytes = static_cast<size_t>(c->G) * c->plane * sizeof(float);
-  char* base = static_cast<char*>(c->ckpt.p) + static_cast<size_t>(s / I) * 4 * gbytes;
-  const void* src[4] = {c->U.p, c->L[hl].p, c->L[(hl + 1) % 3].p, c->L[(hl + 2) % 3].p};
-  for (int q = 0; q < 4; ++q)
-    RTE_TRY(cuda_status(cudaMemcpyAsync(base + q * gbytes, src[q], gbytes, cudaMemcpyDeviceToDevice, c->stream)));
-  return RTE_OK;
+  return copy_checkpoint(c, F(c->U), c->L, hl, c->G, s);
 }
 
 // Runs `enqueue` (which puts the whole march on c->stream) directly, or, in
@@ -524,7 +572,7 @@ unsigned long long key_ptr(const void* p) { return static_cast<unsigned long lon
 // Key of the buffers a forward march of context c touches.
 void append_forward_key(const rte_ctx* c, std::vector<unsigned long long>& key) {
   const void* ptrs[] = {c->U.p, c->R.p, c->L[0].p, c->L[1].p, c->L[2].p, c->ring.p, c->S.p, c->A.p,
-                        c->T.p, c->ckpt.p, c->mua.p, c->mus.p};
+                        c->T.p, c->ckpt.p, c->mua.p, c->mus.p, c->ctl.p};
   key.push_back(static_cast<unsigned long long>(c->n_steps));
   key.push_back(static_cast<unsigned long long>(c->G));
   key.push_back(static_cast<unsigned long long>(c->kmax));
@@ -730,6 +778,7 @@ rte_status rte_destroy(rte_ctx* c) {
   release(c->batch_tab_adj);
   release(c->batch_jobs);
   release(c->err);
+  release(c->ctl);
   release(c->bal);
   release(c->bal_partial);
   release(c->bal_ticket);
@@ -1173,6 +1222,11 @@ static rte_status adjoint_impl(rte_ctx* c, const rte_detector* dets, int n_det, 
   float* moth = F(c->RA);
   int hl_adj = 0;
   std::vector<int> no_snaps(N, -1);
+  // Continuous form with multi-step launches: recompute, adjoint levels and
+  // gradient of a segment in turn on the context's stream, in one launch
+  // each.  The first segment buffer takes the forward levels, the second the
+  // adjoint's.
+  const bool marched = !discrete && !fused_adj && !c->timing && rte_kern::tc_march_supported(sa);
   // Levels needed: forward steps 0 .. N-2 (the adjoint vanishes at the last).
   const int last = N - 2;
   // Segments in reverse order.  The forward recompute of a segment (second
@@ -1191,7 +1245,7 @@ static rte_status adjoint_impl(rte_ctx* c, const rte_detector* dets, int n_det, 
   RTE_TRY(cuda_status(cudaStreamWaitEvent(c->astream, done_adj[0], 0)));
   auto seg_ptrs = [&](int k, int s0, int s_end) {
     std::vector<float*> segp(s_end - s0);
-    const size_t base = static_cast<size_t>(k % 2) * I * gfloats;
+    const size_t base = marched ? 0 : static_cast<size_t>(k % 2) * I * gfloats;
     for (int q = 0; q < s_end - s0; ++q) segp[q] = F(c->seg) + base + static_cast<size_t>(q) * gfloats;
     return segp;
   };
@@ -1199,7 +1253,7 @@ static rte_status adjoint_impl(rte_ctx* c, const rte_detector* dets, int n_det, 
     const int seg = segs[k];
     const int s0 = seg * I, s_end = std::min(s0 + I, last + 1);
     const cudaStream_t keep = c->stream;
-    c->stream = c->astream;
+    if (!marched) c->stream = c->astream;
     const bool keep_timing = c->timing;
     c->timing = false;
     // Restore the AB4 state of the checkpoint and recompute the segment.
@@ -1216,7 +1270,7 @@ static rte_status adjoint_impl(rte_ctx* c, const rte_detector* dets, int n_det, 
     c->timing = keep_timing;
     return st;
   };
-  if (!segs.empty()) RTE_TRY(recompute(0));
+  if (!segs.empty() && !marched) RTE_TRY(recompute(0));
   // Discrete form: the transposed step with src_step N-1 on the zero state
   // gives v^{N-1} = c dt chi0 BC^T(readout^T r^{N-1}), the field that the
   // gradient of level N-1 takes.
@@ -1227,6 +1281,33 @@ static rte_status adjoint_impl(rte_ctx* c, const rte_detector* dets, int n_det, 
   for (size_t k = 0; k < segs.size(); ++k) {
     const int seg = segs[k];
     const int s0 = seg * I, s_end = std::min(s0 + I, last + 1);
+    if (marched) {
+      const int n = s_end - s0;
+      RTE_TRY(recompute(static_cast<int>(k)));
+      rte_kern::MarchArgs ma;
+      ma.a = sa;
+      ma.b = ba;
+      ma.u0 = ma.u1 = mcur;
+      ma.slots = F(c->seg) + static_cast<size_t>(I) * gfloats;
+      ma.slot_floats = gfloats;
+      for (int q = 0; q < 3; ++q) ma.L[q] = F(c->LA[q]);
+      ma.hl = hl_adj;
+      ma.step0 = s_end - 1;
+      ma.dstep = -1;
+      ma.n_steps = n;
+      ma.ctl = static_cast<int*>(c->ctl.p);
+      RTE_TRY(cuda_status(rte_kern::launch_march_tc(ma, c->stream, &c->launches)));
+      hl_adj = (hl_adj + 2 * n) % 3;
+      // adjoint slot l is level s_end - 1 - l
+      const long long step = static_cast<long long>(gfloats);
+      RTE_TRY(cuda_status(rte_kern::launch_grad(
+          ma.slots, seg_ptrs(static_cast<int>(k), s0, s_end)[n - 1], F(c->PT), F(c->area), c->nx, c->ny, c->M, G,
+          c->plane, c->plane, scale, 1, {n, step, -step}, dJ_dmua ? D(c->grad_a) : nullptr,
+          dJ_dmus ? D(c->grad_b) : nullptr, c->stream, &c->launches)));
+      RTE_TRY(cuda_status(cudaMemcpyAsync(mcur, ma.slots + static_cast<size_t>(n - 1) * gfloats, gbytes,
+                                          cudaMemcpyDeviceToDevice, c->stream)));
+      continue;
+    }
     // next segment's recompute may start once the adjoint that read its
     // buffer (segment k - 1) is done
     if (k + 1 < segs.size()) {
@@ -1257,7 +1338,7 @@ static rte_status adjoint_impl(rte_ctx* c, const rte_detector* dets, int n_det, 
       }
       RTE_TRY(cuda_status(rte_kern::launch_grad(mcur, segp[lvl - s0], F(c->PT),
                                                 discrete ? nullptr : F(c->area), c->nx, c->ny, c->M, G,
-                                                c->plane, c->plane, discrete ? 1.0 : scale, discrete ? 0 : 1,
+                                                c->plane, c->plane, discrete ? 1.0 : scale, discrete ? 0 : 1, {1, 0, 0},
                                                 dJ_dmua ? D(c->grad_a) : nullptr,
                                                 dJ_dmus ? D(c->grad_b) : nullptr, c->stream,
                                                 &c->launches)));

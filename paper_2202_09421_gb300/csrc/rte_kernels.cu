@@ -436,33 +436,39 @@ template <int MM>
 __device__ __forceinline__ void grad_node(const float* __restrict__ MU, const float* __restrict__ Useg,
                                           const float* __restrict__ PT, const float* __restrict__ area,
                                           long long cell, int G, size_t plane, size_t useg_gs, double scale,
-                                          int flip, double* __restrict__ grad_a, double* __restrict__ grad_b) {
+                                          int flip, const GradLevels lv, double* __restrict__ grad_a,
+                                          double* __restrict__ grad_b) {
   float p[MM];
 #pragma unroll
   for (int d = 0; d < MM; ++d) p[d] = __ldg(PT + d);            // P~[0][d] = p_d (symmetric circulant)
-  float sa = 0.f, sb = 0.f;
-  for (int g = 0; g < G; ++g) {
-    const float* u = Useg + static_cast<size_t>(g) * useg_gs + static_cast<size_t>(cell) * MM;
-    const float* mu = MU + static_cast<size_t>(g) * plane + static_cast<size_t>(cell) * MM;
-    float uu[MM], lam[MM];
-#pragma unroll
-    for (int k = 0; k < MM / 8; ++k) {
-      ld32b(u + 8 * k, uu + 8 * k);
-      ld32b(mu + 8 * k, lam + 8 * k);
-    }
-#pragma unroll
-    for (int m = 0; m < MM; ++m) {
-      float pu = 0.f;
-#pragma unroll
-      for (int q = 0; q < MM; ++q) pu = fmaf(p[(m - q + MM) % MM], uu[q], pu);
-      const float l = flip ? lam[(m + MM / 2) % MM] : lam[m];
-      sa = fmaf(l, uu[m], sa);
-      sb = fmaf(l, uu[m] - pu, sb);
-    }
-  }
   const double k = area ? scale * static_cast<double>(area[cell]) : scale;
-  if (grad_a) grad_a[cell] -= k * static_cast<double>(sa);
-  if (grad_b) grad_b[cell] -= k * static_cast<double>(sb);
+  double da = grad_a ? grad_a[cell] : 0.0, db = grad_b ? grad_b[cell] : 0.0;
+  for (int l = 0; l < lv.n; ++l) {
+    float sa = 0.f, sb = 0.f;
+    for (int g = 0; g < G; ++g) {
+      const float* u = Useg + l * lv.u_step + static_cast<size_t>(g) * useg_gs + static_cast<size_t>(cell) * MM;
+      const float* mu = MU + l * lv.mu_step + static_cast<size_t>(g) * plane + static_cast<size_t>(cell) * MM;
+      float uu[MM], lam[MM];
+#pragma unroll
+      for (int q = 0; q < MM / 8; ++q) {
+        ld32b(u + 8 * q, uu + 8 * q);
+        ld32b(mu + 8 * q, lam + 8 * q);
+      }
+#pragma unroll
+      for (int m = 0; m < MM; ++m) {
+        float pu = 0.f;
+#pragma unroll
+        for (int q = 0; q < MM; ++q) pu = fmaf(p[(m - q + MM) % MM], uu[q], pu);
+        const float x = flip ? lam[(m + MM / 2) % MM] : lam[m];
+        sa = fmaf(x, uu[m], sa);
+        sb = fmaf(x, uu[m] - pu, sb);
+      }
+    }
+    da -= k * static_cast<double>(sa);
+    db -= k * static_cast<double>(sb);
+  }
+  if (grad_a) grad_a[cell] = da;
+  if (grad_b) grad_b[cell] = db;
 }
 
 // Any M: one warp per cell, the lanes over the ordinates, the row of P~ from
@@ -470,31 +476,34 @@ __device__ __forceinline__ void grad_node(const float* __restrict__ MU, const fl
 __device__ __forceinline__ void grad_cell(const float* __restrict__ MU, const float* __restrict__ Useg,
                                           const float* __restrict__ PT, const float* __restrict__ area,
                                           long long cell, int M, int G, size_t plane, size_t useg_gs,
-                                          double scale, int flip, double* __restrict__ grad_a,
-                                          double* __restrict__ grad_b) {
+                                          double scale, int flip, const GradLevels lv,
+                                          double* __restrict__ grad_a, double* __restrict__ grad_b) {
   __shared__ float ubuf[8][64];
   const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
-  float sa = 0.f, sb = 0.f;
-  for (int g = 0; g < G; ++g) {
-    const float* u = Useg + static_cast<size_t>(g) * useg_gs + static_cast<size_t>(cell) * M;
-    const float* mu = MU + static_cast<size_t>(g) * plane + static_cast<size_t>(cell) * M;
-    for (int m = lane; m < M; m += 32) ubuf[wl][m] = u[m];
-    __syncwarp();
-    for (int m = lane; m < M; m += 32) {
-      float pu = 0.f;
-      for (int q = 0; q < M; ++q) pu = fmaf(PT[q * M + m], ubuf[wl][q], pu);
-      const float lam = flip ? mu[(m + M / 2) % M] : mu[m];
-      sa = fmaf(lam, ubuf[wl][m], sa);
-      sb = fmaf(lam, ubuf[wl][m] - pu, sb);
+  const double k = area ? scale * static_cast<double>(area[cell]) : scale;
+  double da = grad_a ? grad_a[cell] : 0.0, db = grad_b ? grad_b[cell] : 0.0;
+  for (int l = 0; l < lv.n; ++l) {
+    float sa = 0.f, sb = 0.f;
+    for (int g = 0; g < G; ++g) {
+      const float* u = Useg + l * lv.u_step + static_cast<size_t>(g) * useg_gs + static_cast<size_t>(cell) * M;
+      const float* mu = MU + l * lv.mu_step + static_cast<size_t>(g) * plane + static_cast<size_t>(cell) * M;
+      for (int m = lane; m < M; m += 32) ubuf[wl][m] = u[m];
+      __syncwarp();
+      for (int m = lane; m < M; m += 32) {
+        float pu = 0.f;
+        for (int q = 0; q < M; ++q) pu = fmaf(PT[q * M + m], ubuf[wl][q], pu);
+        const float lam = flip ? mu[(m + M / 2) % M] : mu[m];
+        sa = fmaf(lam, ubuf[wl][m], sa);
+        sb = fmaf(lam, ubuf[wl][m] - pu, sb);
+      }
+      __syncwarp();
     }
-    __syncwarp();
+    da -= k * static_cast<double>(warp_sum(sa));
+    db -= k * static_cast<double>(warp_sum(sb));
   }
-  sa = warp_sum(sa);
-  sb = warp_sum(sb);
   if (lane == 0) {
-    const double k = area ? scale * static_cast<double>(area[cell]) : scale;
-    if (grad_a) grad_a[cell] -= k * static_cast<double>(sa);
-    if (grad_b) grad_b[cell] -= k * static_cast<double>(sb);
+    if (grad_a) grad_a[cell] = da;
+    if (grad_b) grad_b[cell] = db;
   }
 }
 
@@ -503,18 +512,18 @@ __device__ __forceinline__ bool grad_by_thread(int M) { return M == 16 || M == 3
 
 __global__ void grad_kernel(const float* __restrict__ MU, const float* __restrict__ Useg,
                             const float* __restrict__ PT, const float* __restrict__ area, int ncell,
-                            int M, int G, size_t plane, size_t useg_gs, double scale, int flip,
+                            int M, int G, size_t plane, size_t useg_gs, double scale, int flip, GradLevels lv,
                             double* __restrict__ grad_a, double* __restrict__ grad_b) {
   const long long t = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (grad_by_thread(M)) {
     if (t >= ncell) return;
-    if (M == 32) grad_node<32>(MU, Useg, PT, area, t, G, plane, useg_gs, scale, flip, grad_a, grad_b);
-    else grad_node<16>(MU, Useg, PT, area, t, G, plane, useg_gs, scale, flip, grad_a, grad_b);
+    if (M == 32) grad_node<32>(MU, Useg, PT, area, t, G, plane, useg_gs, scale, flip, lv, grad_a, grad_b);
+    else grad_node<16>(MU, Useg, PT, area, t, G, plane, useg_gs, scale, flip, lv, grad_a, grad_b);
     return;
   }
   const long long cell = t >> 5;
   if (cell >= ncell) return;   // whole warp exits together
-  grad_cell(MU, Useg, PT, area, cell, M, G, plane, useg_gs, scale, flip, grad_a, grad_b);
+  grad_cell(MU, Useg, PT, area, cell, M, G, plane, useg_gs, scale, flip, lv, grad_a, grad_b);
 }
 
 // Batched forms for media that march in lockstep: blockIdx.y picks the
@@ -524,15 +533,16 @@ __global__ void grad_batch_kernel(const GradJob* __restrict__ jobs, int slot, in
   const GradJob& j = jobs[blockIdx.y];
   const long long t = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   const float* useg = j.seg + static_cast<size_t>(slot) * j.slot_floats;
+  const GradLevels one{1, 0, 0};
   if (grad_by_thread(j.M)) {
     if (t >= j.ncell) return;
-    if (j.M == 32) grad_node<32>(j.MU, useg, j.PT, j.area, t, j.G, j.plane, j.plane, j.scale, flip, j.grad_a, j.grad_b);
-    else grad_node<16>(j.MU, useg, j.PT, j.area, t, j.G, j.plane, j.plane, j.scale, flip, j.grad_a, j.grad_b);
+    if (j.M == 32) grad_node<32>(j.MU, useg, j.PT, j.area, t, j.G, j.plane, j.plane, j.scale, flip, one, j.grad_a, j.grad_b);
+    else grad_node<16>(j.MU, useg, j.PT, j.area, t, j.G, j.plane, j.plane, j.scale, flip, one, j.grad_a, j.grad_b);
     return;
   }
   const long long cell = t >> 5;
   if (cell >= j.ncell) return;
-  grad_cell(j.MU, useg, j.PT, j.area, cell, j.M, j.G, j.plane, j.plane, j.scale, flip, j.grad_a, j.grad_b);
+  grad_cell(j.MU, useg, j.PT, j.area, cell, j.M, j.G, j.plane, j.plane, j.scale, flip, one, j.grad_a, j.grad_b);
 }
 
 __global__ void save_batch_kernel(const SaveJob* __restrict__ jobs, int slot) {
@@ -798,12 +808,12 @@ cudaError_t launch_balance(const float* U, size_t plane, int nx, int ny, int M, 
 
 cudaError_t launch_grad(const float* MU, const float* Useg, const float* PT, const float* area,
                         int nx, int ny, int M, int G, size_t plane, size_t useg_group_stride,
-                        double scale, int flip, double* grad_a, double* grad_b, cudaStream_t s,
-                        long long* launches) {
+                        double scale, int flip, GradLevels lv, double* grad_a, double* grad_b,
+                        cudaStream_t s, long long* launches) {
   const int ncell = nx * ny;
   const long long threads = (M == 16 || M == 32) ? ncell : 32LL * ncell;
   grad_kernel<<<static_cast<int>((threads + 255) / 256), 256, 0, s>>>(MU, Useg, PT, area, ncell, M, G, plane,
-                                                                      useg_group_stride, scale, flip, grad_a,
+                                                                      useg_group_stride, scale, flip, lv, grad_a,
                                                                       grad_b);
   if (launches) *launches += 1;
   return cudaGetLastError();

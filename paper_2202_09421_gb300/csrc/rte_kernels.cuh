@@ -129,6 +129,32 @@ void tc_batch_layout(BatchProblem* probs, int n, int* ctas_x, int* ctas_y);
 cudaError_t launch_step_tc_batched(const BatchProblem* probs, const BatchProblem* probs_dev, int n,
                                    int step, int hl, cudaStream_t s, long long* launches);
 
+// Several steps of every group in one launch (rte_tc_march.cu): schedule 1
+// with a line of more than 128 positions, without the tensor-core scattering
+// flag.  State buffers: u0 and u1
+// alternate (the state before step k of the launch is in u0 for even k, u1
+// for odd k), or, with slots, u^{k} of step k > 0 is written to slot k - 1
+// (slot_floats apart) and u0 holds the state before the first.  L[hl] is
+// L^{k-1} of the first step; the ring rotates by 2 (mod 3) per step.  Step k
+// takes the boundary data of step0 + k dstep.  ctl: tc_march_ctl_bytes(G)
+// bytes that no other launch in flight uses.
+struct MarchArgs {
+  StepArgs a;
+  BoundaryArgs b;
+  float* u0;
+  float* u1;
+  float* slots;
+  size_t slot_floats;
+  float* L[3];
+  int hl;
+  int step0, dstep, n_steps;
+  int rt, lag;                      // set by the launcher: 128-row output tiles per item, item order
+  int* ctl;
+};
+bool tc_march_supported(const StepArgs& a);
+size_t tc_march_ctl_bytes(int G);
+cudaError_t launch_march_tc(MarchArgs ma, cudaStream_t s, long long* launches);
+
 // Persistent warp-specialised passes (rte_tc_ws.cu): nx, ny <= 256, M in
 // {16, 32}, without the tensor-core scattering flag.
 bool tc_ws_supported(const StepArgs& a);
@@ -195,10 +221,16 @@ cudaError_t launch_rho(const float* resid, const float* Wn, int n_det, int ring_
 // grad_a[c] -= k sum_g sum_m lambda_m u_m; grad_b[c] -= k sum_g sum_m
 // lambda_m (u - P u)_m, with k = scale * area[c] (scale alone when area is
 // null) and lambda_m = mu_{m + M/2} when flip is set, mu_m otherwise.
+// Over lv.n levels in turn: level l has mu at MU + l mu_step, u at Useg + l
+// u_step (floats).
+struct GradLevels {
+  int n;
+  long long mu_step, u_step;
+};
 cudaError_t launch_grad(const float* MU, const float* Useg, const float* PT, const float* area,
                         int nx, int ny, int M, int G, size_t plane, size_t useg_group_stride,
-                        double scale, int flip, double* grad_a, double* grad_b, cudaStream_t s,
-                        long long* launches);
+                        double scale, int flip, GradLevels lv, double* grad_a, double* grad_b,
+                        cudaStream_t s, long long* launches);
 
 // Photon-balance sums of the post-BC state U (every group) for one step:
 // out[(g n_steps + step) 3 + k] = (photons int Phi / c, absorption int a Phi,

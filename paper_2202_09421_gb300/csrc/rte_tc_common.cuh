@@ -33,6 +33,25 @@ __device__ __forceinline__ float ab4_node(float cdt, float lk, float l1, float l
   return fmaf(cdt, fmaf(kAB3, l3, fmaf(kAB2, l2, fmaf(kAB1, l1, kAB0 * lk))), u);
 }
 
+// Exitance of one node, sum_m w_m v_m (eq. OpMed), in the order that every
+// y-pass schedule shares: four ordinates in order, then pairwise over the
+// groups of four (the order of a warp whose lanes hold four ordinates each).
+template <int M>
+__device__ __forceinline__ float exitance_sum_node(const float* w, const float* v) {
+  float p[M / 4];
+#pragma unroll
+  for (int k = 0; k < M / 4; ++k) {
+    p[k] = w[4 * k] * v[4 * k];
+#pragma unroll
+    for (int e = 1; e < 4; ++e) p[k] = fmaf(w[4 * k + e], v[4 * k + e], p[k]);
+  }
+#pragma unroll
+  for (int o = 1; o < M / 4; o <<= 1)
+#pragma unroll
+    for (int k = 0; k + o < M / 4; k += 2 * o) p[k] += p[k + o];
+  return p[0];
+}
+
 // Operand kinds of the precision modes (rte.h): 1 3xTF32, 2 TF32, 3 bf16x3,
 // 4 BF16.  KC = K positions per 128-byte row, GV = values per 16-byte group.
 template <int PREC>
@@ -78,6 +97,23 @@ __device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_
       "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
       "l"(src), "r"(bytes), "r"(bar)
       : "memory");
+}
+
+// The hi and (dst1 != 0) lo row ranges of an operator chunk, completing
+// together on bar.
+__device__ __forceinline__ void bulk_copy2(uint32_t dst0, const void* src0, uint32_t dst1, const void* src1,
+                                           uint32_t bytes, uint32_t bar) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(dst1 ? 2 * bytes : bytes)
+               : "memory");
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst0),
+      "l"(src0), "r"(bytes), "r"(bar)
+      : "memory");
+  if (dst1)
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst1),
+        "l"(src1), "r"(bytes), "r"(bar)
+        : "memory");
 }
 
 template <bool BF>
@@ -169,6 +205,15 @@ __device__ __forceinline__ float ld_hint(const float* ptr, uint64_t pol) {
   return v;
 }
 
+__device__ __forceinline__ float4 ld4_hint(const float* ptr, uint64_t pol) {
+  float4 v;
+  asm volatile("ld.global.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(ptr), "l"(pol)
+               : "memory");
+  return v;
+}
+
 // 32-byte global accesses (sm_100 and later): whole 32-byte sectors per
 // thread, so a warp that walks 32 nodes of 128 B leaves no half-written
 // sectors for L2 to merge.  Addresses are 32-byte aligned.
@@ -192,6 +237,19 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float v[8]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int t = 0; t < 8; ++t) v[t] = __uint_as_float(r[t]);
+}
+
+// The same in two parts: the values are there after tmem_ld8_wait.
+__device__ __forceinline__ void tmem_ld8_async(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld8_wait(uint32_t (&r)[8]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])
+               :
+               : "memory");
 }
 
 // x-pass epilogue at one node (Sec. 4.1, eq. RTEAB4L): acc[m] holds the

@@ -109,6 +109,21 @@ __host__ __device__ inline int stream_stages(int stage_bytes) {
   return s > kMaxStages ? kMaxStages : s;
 }
 
+// sum_m w_m v_m of a node whose M ordinates are adjacent lanes (w_m v_m of
+// ordinate m on lane m), in the order of the one-tile y-pass: four ordinates
+// in order, then pairwise.  The sum in the node's lanes with m % 4 == 0.
+template <int M>
+__device__ __forceinline__ float lane_exitance(float w, float v, int lane) {
+  const int q = lane & ~3;
+  float ex = __shfl_sync(0xffffffffu, w, q) * __shfl_sync(0xffffffffu, v, q);
+#pragma unroll
+  for (int e = 1; e < 4; ++e)
+    ex = fmaf(__shfl_sync(0xffffffffu, w, q + e), __shfl_sync(0xffffffffu, v, q + e), ex);
+#pragma unroll
+  for (int o = 4; o < M; o <<= 1) ex += __shfl_xor_sync(0xffffffffu, ex, o);
+  return ex;
+}
+
 // The y epilogue's rows per accumulator load: all loads of a chunk are
 // issued before any is used.
 constexpr int kRowsY = 16;
@@ -479,16 +494,12 @@ __global__ void __launch_bounds__(kStThreads, 1)
             if (ro) {
               if (__any_sync(kFull, bnd && (lf || rt))) {
                 const int F = lf ? 0 : 1;
-                float ex = 0.f;
-                for (int mm = 0; mm < M; ++mm)
-                  ex = fmaf(__ldg(b.wexit + F * M + mm), __shfl_sync(kFull, val, base + mm), ex);
+                const float ex = lane_exitance<M>(__ldg(b.wexit + F * M + m), val, lane);
                 if (bnd && (lf || rt) && m == 0) ro[lf ? j : ny + j] = ex;
               }
               if (__any_sync(kFull, bnd && (bt || tp))) {
                 const int F = bt ? 2 : 3;
-                float ex = 0.f;
-                for (int mm = 0; mm < M; ++mm)
-                  ex = fmaf(__ldg(b.wexit + F * M + mm), __shfl_sync(kFull, val, base + mm), ex);
+                const float ex = lane_exitance<M>(__ldg(b.wexit + F * M + m), val, lane);
                 if (bnd && (bt || tp) && m == 0) ro[bt ? 2 * ny + i : 2 * ny + nx + i] = ex;
               }
             }
