@@ -370,12 +370,13 @@ rte_status march(rte_ctx* c, DevBuf& U, DevBuf& R, DevBuf* L, int& hl, int G, in
 }
 
 // Uploads the operator E (row-major n x n, FP64) in the kernels' forms: the
-// SIMT array ET[k n + i] = E[i][k] and, in the tensor-core forms, the split,
+// padded SIMT array ET[k][i] = E[i][k] and, in the tensor-core forms, the split,
 // swizzled image (synchronises: the host vectors must outlive the copies).
 rte_status upload_operator(rte_ctx* c, const std::vector<double>& E, int n, DevBuf& simt, DevBuf& img) {
-  std::vector<float> T(static_cast<size_t>(n) * n);
+  const size_t ld = rte_kern::simt_ld(n);
+  std::vector<float> T(rte_kern::simt_rows(n) * ld, 0.f);
   for (int i = 0; i < n; ++i)
-    for (int k = 0; k < n; ++k) T[static_cast<size_t>(k) * n + i] = static_cast<float>(E[static_cast<size_t>(i) * n + k]);
+    for (int k = 0; k < n; ++k) T[k * ld + i] = static_cast<float>(E[static_cast<size_t>(i) * n + k]);
   RTE_TRY(upload(simt, T, c->stream));
   std::vector<float> im;
   std::vector<unsigned short> im16;

@@ -27,313 +27,482 @@ namespace {
 constexpr float kAB0 = 55.0f / 24.0f, kAB1 = -59.0f / 24.0f, kAB2 = 37.0f / 24.0f,
                 kAB3 = -9.0f / 24.0f;
 
-__host__ __device__ inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
-
-// Output rows of a tile are padded to 32 so that a block (8 x rows/8
-// threads) is a whole number of warps: the epilogue works warp by warp.
-constexpr int kRowPad = 32;
-
-// acc[r][c] += sum_k A[row0 + r][k] * B[k][col0 + c] over the whole K range,
-// with A given transposed in global memory (AT[k * n + row]) and staged in
-// shared memory chunk by chunk; B is the full slab already in shared memory.
-__device__ inline void gemm_rows(const float* __restrict__ AT, int n, int npad, int kpad,
-                                 const float* Bs, float* As, int row0, int col0,
-                                 float acc[kTM][kTN]) {
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-  const int nthr = blockDim.x * blockDim.y;
-  for (int k0 = 0; k0 < kpad; k0 += kKC) {
-    __syncthreads();
-    for (int idx = tid; idx < kKC * npad; idx += nthr) {
-      const int k = idx / npad, r = idx - k * npad;
-      const int kk = k0 + k;
-      As[idx] = (kk < n && r < n) ? __ldg(AT + static_cast<size_t>(kk) * n + r) : 0.0f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < kKC; ++k) {
-      const float4 a0 = *reinterpret_cast<const float4*>(As + k * npad + row0);
-      const float4 a1 = *reinterpret_cast<const float4*>(As + k * npad + row0 + 4);
-      const float4 b0 = *reinterpret_cast<const float4*>(Bs + (k0 + k) * kTileCols + col0);
-      const float4 b1 = *reinterpret_cast<const float4*>(Bs + (k0 + k) * kTileCols + col0 + 4);
-      const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-      for (int r = 0; r < kTM; ++r)
-#pragma unroll
-        for (int c = 0; c < kTN; ++c) acc[r][c] = fmaf(a[r], b[c], acc[r][c]);
-    }
-  }
-}
-
-__global__ void __launch_bounds__(512) xpass_kernel(StepArgs a, const float* __restrict__ U,
-                                                     float* __restrict__ R) {
-  extern __shared__ __align__(16) float smem[];
-  const int n = a.nx, M = a.M;
-  const int npad = round_up(n, kRowPad), kpad = round_up(n, kKC);
-  const int rows_per_tile = kTileCols / M;
-  float* Bs = smem;                                   // [kpad][64]
-  float* As = Bs + kpad * kTileCols;                  // [kKC][npad]
-  float* Ps = As + kKC * npad;                        // [M][M] (P~ transposed)
-  const int g = blockIdx.z;
-  const int j0 = blockIdx.x * rows_per_tile;
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-  const int nthr = blockDim.x * blockDim.y;
-  const float* Ug = U + static_cast<size_t>(g) * a.plane;
-
-  // Stage the rows' slab: Bs[i'][r*M + m] = u[j0 + r][i'][m].
-  for (int idx = tid; idx < kpad * (kTileCols / 4); idx += nthr) {
-    const int k = idx / (kTileCols / 4), c = (idx - k * (kTileCols / 4)) * 4;
-    const int r = c / M, m = c - r * M, j = j0 + r;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (k < n && r < rows_per_tile && j < a.ny)
-      v = __ldg(reinterpret_cast<const float4*>(Ug + (static_cast<size_t>(j) * n + k) * M + m));
-    *reinterpret_cast<float4*>(Bs + k * kTileCols + c) = v;
-  }
-  for (int idx = tid; idx < M * M; idx += nthr) Ps[idx] = __ldg(a.PT + idx);
-
-  const int row0 = threadIdx.y * kTM, col0 = threadIdx.x * kTN;
-  float acc[kTM][kTN];
-#pragma unroll
-  for (int r = 0; r < kTM; ++r)
-#pragma unroll
-    for (int c = 0; c < kTN; ++c) acc[r][c] = 0.f;
-  gemm_rows(a.DxT, n, npad, kpad, Bs, As, row0, col0, acc);
-
-  // Epilogue: node-local scattering and absorption, minus xi * d_x u.
-  // Columns past rows_per_tile * M (M not dividing 64) belong to no row of
-  // this tile.
-  const int r = col0 / M, mb = col0 - r * M, j = j0 + r;
-  if (r >= rows_per_tile || j >= a.ny) return;
-  float xi[kTN];
-#pragma unroll
-  for (int t = 0; t < kTN; ++t) xi[t] = __ldg(a.xi + mb + t);
-#pragma unroll
-  for (int ii = 0; ii < kTM; ++ii) {
-    const int i = row0 + ii;
-    if (i >= n) break;
-    const float* ucell = Bs + i * kTileCols + r * M;
-    float s[kTN];
-#pragma unroll
-    for (int t = 0; t < kTN; ++t) s[t] = 0.f;
-    for (int q = 0; q < M; ++q) {
-      const float uq = ucell[q];
-      const float4 p0 = *reinterpret_cast<const float4*>(Ps + q * M + mb);
-      const float4 p1 = *reinterpret_cast<const float4*>(Ps + q * M + mb + 4);
-      s[0] = fmaf(p0.x, uq, s[0]); s[1] = fmaf(p0.y, uq, s[1]);
-      s[2] = fmaf(p0.z, uq, s[2]); s[3] = fmaf(p0.w, uq, s[3]);
-      s[4] = fmaf(p1.x, uq, s[4]); s[5] = fmaf(p1.y, uq, s[5]);
-      s[6] = fmaf(p1.z, uq, s[6]); s[7] = fmaf(p1.w, uq, s[7]);
-    }
-    const float av = __ldg(a.mua + static_cast<size_t>(j) * n + i);
-    const float bv = __ldg(a.mus + static_cast<size_t>(j) * n + i);
-    float out[kTN];
-#pragma unroll
-    for (int t = 0; t < kTN; ++t)
-      out[t] = bv * s[t] - (av + bv) * ucell[mb + t] - xi[t] * acc[ii][t];
-    float* dst = R + static_cast<size_t>(g) * a.plane + (static_cast<size_t>(j) * n + i) * M + mb;
-    reinterpret_cast<float4*>(dst)[0] = make_float4(out[0], out[1], out[2], out[3]);
-    reinterpret_cast<float4*>(dst)[1] = make_float4(out[4], out[5], out[6], out[7]);
-  }
-}
-
 __device__ inline float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
 
-// TR: the transposed step of the discrete adjoint (BoundaryArgs::bct_src);
-// a separate instance, so that the forward step compiles without it.
-template <bool TR>
-__global__ void __launch_bounds__(512) ypass_kernel(StepArgs a, BoundaryArgs b, float* __restrict__ U,
-                                                     const float* __restrict__ R,
-                                                     const float* __restrict__ L1,
-                                                     const float* __restrict__ L2,
-                                                     float* __restrict__ L3, int src_step,
-                                                     int ring_step) {
+// ---------------------------------------------------------------- passes
+//
+// A pass is a GEMM of the n x n operator with the slab of a tile of lines,
+// n x BN (BN = lines per tile x M).  A CTA computes every row of its tile, so
+// that the y-pass may update U in place: its slab sits in shared memory from
+// the first read to the epilogue.  A thread has T x T outputs: blocks of four
+// rows, T / 4 of them, by T neighbouring columns of one node, so that the
+// epilogues move 16-byte pieces of whole lines.  The products are packed in
+// pairs of rows (fma.rn.f32x2: the same fused multiply-adds, two an
+// instruction, which leaves the issue slots for the shared-memory loads).
+//
+// Operator and slab arrive in chunks of kKC positions by cp.async, the
+// operator through a ring of kRing chunks; the operator array is padded with
+// zeros (simt_ld, simt_rows), so that a chunk is one contiguous run without
+// bounds checks.
+//
+// What bounds it: shared-memory reads (a 16-byte load returns 512 bytes a
+// warp; with 8 x 8 outputs the loads of a position take as long as its
+// multiply-adds) and the FP32 pipe (36.7 TFMA/s measured for independent
+// FFMA) together on large problems; on small ones the latency of the chunks,
+// the epilogue's loads and the launch.  Time per step before (one warp per
+// node in the y epilogue, a 64-column tile, bounds-checked operator loads)
+// and now: 256^2, M = 32, four groups 498 -> 215 us; 203 x 131, M = 24, three
+// groups 159 -> 62; 64^2, M = 16, one group 94 -> 12.
+struct TileShape {
+  int ntx, nty;                      // threads over columns and rows
+  int BN, per_tile;                  // columns and grid lines of the tile
+};
+
+constexpr int kSlabPad = 4;          // floats after a slab row (conflict-free column reads in the scattering)
+constexpr int kMaxThreads = 512;
+constexpr int kRing = 2;             // operator chunks in shared memory (four measured no faster and cost occupancy)
+
+// Column block tx and row block ty of a thread.  Eight neighbouring lanes
+// take four column blocks of two row blocks where the tile has them, so that
+// their 16-byte pieces of a slab row (T = 8: every other one) lie in
+// different banks.
+__device__ __forceinline__ void thread_place(const TileShape& ts, int& tx, int& ty) {
+  const int tid = threadIdx.x;
+  if ((ts.ntx & 3) == 0 && (ts.nty & 1) == 0) {
+    const int n4 = ts.ntx >> 2, q = tid >> 3;
+    tx = (tid & 3) + 4 * (q % n4);
+    ty = ((tid >> 2) & 1) + 2 * (q / n4);
+  } else {
+    tx = tid % ts.ntx;
+    ty = tid / ts.ntx;
+  }
+}
+
+// Boundary nodes of a y tile, at most: both x-faces and two y-face rows.
+__host__ __device__ inline int tile_nodes(int n, int M, int BN) { return (BN > M ? 2 : 1) * n + 2 * (BN / M); }
+
+size_t tile_smem(int n, int M, int BN, bool xpass) {
+  const size_t ld = simt_ld(n), rows = simt_rows(n);
+  size_t f = rows * (BN + kSlabPad) + static_cast<size_t>(kRing) * kKC * ld;
+  // P~, or the boundary tables and the boundary nodes' sources
+  f += xpass ? static_cast<size_t>(M) : static_cast<size_t>(8 * M) * 2 + 4 * M + 2 * tile_nodes(n, M, BN);
+  return f * sizeof(float);
+}
+
+__device__ __forceinline__ void cp_async16(float* dst, const float* src, bool valid) {
+  const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(valid ? 16 : 0) : "memory");
+}
+
+// acc[r][c] = sum_k AT[k][row(r)] slab[k][col(c)], k ascending.  copy_slab(k0)
+// starts the copies of slab rows k0 .. k0 + kKC - 1 (zeros past the line).
+template <int T, class CopySlab>
+__device__ __forceinline__ void tile_gemm(const float* __restrict__ AT, int n, const TileShape& ts, const float* Bs,
+                                          float* As, int tx, int ty, CopySlab&& copy_slab, float (&acc)[T][T]) {
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  const int ld = simt_ld(n), n_chunks = simt_rows(n) / kKC, ldb = ts.BN + kSlabPad;
+  const int chunk = kKC * ld;
+  auto fetch = [&](int c) {
+    if (c < n_chunks) {
+      const float* src = AT + static_cast<size_t>(c) * chunk;
+      float* dst = As + (c % kRing) * chunk;
+      for (int e = tid * 4; e < chunk; e += nthr * 4) cp_async16(dst + e, src + e, true);
+      copy_slab(c * kKC);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll
+  for (int c = 0; c < kRing - 1; ++c) fetch(c);
+  unsigned long long acc2[T / 2][T];                 // two rows each (fma.rn.f32x2)
+#pragma unroll
+  for (int r = 0; r < T / 2; ++r)
+#pragma unroll
+    for (int c = 0; c < T; ++c) acc2[r][c] = 0ull;
+  for (int c = 0; c < n_chunks; ++c) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kRing - 2) : "memory");
+    __syncthreads();                                 // chunk c is there; every thread is done with chunk c - 1
+    fetch(c + kRing - 1);
+    const float* ap = As + (c % kRing) * chunk + ty * 4;
+    const float* bp = Bs + c * kKC * ldb + tx * T;
+#pragma unroll
+    for (int k = 0; k < kKC; ++k) {
+      unsigned long long a2[T / 2];
+      float b[T];
+#pragma unroll
+      for (int v = 0; v < T / 4; ++v) {
+        const ulonglong2 x = *reinterpret_cast<const ulonglong2*>(ap + k * ld + v * 4 * ts.nty);
+        a2[2 * v] = x.x; a2[2 * v + 1] = x.y;
+      }
+#pragma unroll
+      for (int v = 0; v < T / 4; ++v) {
+        const float4 y = *reinterpret_cast<const float4*>(bp + k * ldb + v * 4);
+        b[4 * v] = y.x; b[4 * v + 1] = y.y; b[4 * v + 2] = y.z; b[4 * v + 3] = y.w;
+      }
+#pragma unroll
+      for (int q = 0; q < T; ++q) {
+        unsigned long long b2;
+        asm("mov.b64 %0, {%1, %1};" : "=l"(b2) : "f"(b[q]));
+#pragma unroll
+        for (int r = 0; r < T / 2; ++r)
+          asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc2[r][q]) : "l"(a2[r]), "l"(b2));
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < T / 2; ++r)
+#pragma unroll
+    for (int q = 0; q < T; ++q)
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[2 * r][q]), "=f"(acc[2 * r + 1][q]) : "l"(acc2[r][q]));
+}
+
+template <int T>
+__global__ void __launch_bounds__(kMaxThreads) xpass_kernel(StepArgs a, TileShape ts, const float* __restrict__ U,
+                                                            float* __restrict__ R) {
   extern __shared__ __align__(16) float smem[];
-  const int nx = a.nx, n = a.ny, M = a.M;
-  const int npad = round_up(n, kRowPad), kpad = round_up(n, kKC);
-  const int cols_per_tile = kTileCols / M;
-  float* Bs = smem;                                   // [kpad][64]
-  float* As = Bs + kpad * kTileCols;                  // [kKC][npad]
-  const int g = blockIdx.z;
-  const int i0 = blockIdx.x * cols_per_tile;
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-  const int nthr = blockDim.x * blockDim.y;
-  const size_t goff = static_cast<size_t>(g) * a.plane;
-  float* Ug = U + goff;
+  const int n = a.nx, M = a.M, ldb = ts.BN + kSlabPad;
+  float* Bs = smem;                                   // [rows][ldb]
+  float* As = Bs + simt_rows(n) * ldb;                // [kRing][kKC][ld]
+  float* Ps = As + kRing * kKC * simt_ld(n);              // [M]: p_d = P~[d][0], the circulant's first column
+  const int g = blockIdx.z, j0 = blockIdx.x * ts.per_tile;
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  int tx, ty;
+  thread_place(ts, tx, ty);
+  const float* Ug = U + static_cast<size_t>(g) * a.plane;
+  for (int e = tid; e < M; e += nthr) Ps[e] = __ldg(a.PT + e);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // slab row k: u[j0 + r][k][m] at column r M + m.  A thread copies the same
+  // 16 bytes of every nrow-th row.
+  const int cw = ts.BN / 4, ck = tid / cw, cc = (tid - ck * cw) * 4, nrow = nthr / cw;
+  const int cr = cc / M;
+  const bool c_ok = ck < nrow && j0 + cr < a.ny;
+  const float* csrc = Ug + static_cast<size_t>(c_ok ? j0 + cr : 0) * n * M + (cc - cr * M);
+  auto copy_slab = [&](int k0) {
+    if (ck < nrow)
+      for (int k = ck; k < kKC; k += nrow) {
+        const bool ok = c_ok && k0 + k < n;
+        cp_async16(Bs + (k0 + k) * ldb + cc, csrc + (ok ? static_cast<size_t>(k0 + k) * M : 0), ok);
+      }
+  };
+  float acc[T][T];
+  tile_gemm<T>(a.DxT, n, ts, Bs, As, tx, ty, copy_slab, acc);
+  asm volatile("griddepcontrol.launch_dependents;");
 
-  // Stage the columns' slab: Bs[j'][w*M + m] = u[j'][i0 + w][m] (contiguous).
-  const int valid_cols = min(cols_per_tile, nx - i0) * M;
-  for (int idx = tid; idx < kpad * (kTileCols / 4); idx += nthr) {
-    const int k = idx / (kTileCols / 4), c = (idx - k * (kTileCols / 4)) * 4;
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (k < n && c < valid_cols)
-      v = *reinterpret_cast<const float4*>(Ug + (static_cast<size_t>(k) * nx + i0) * M + c);
-    *reinterpret_cast<float4*>(Bs + k * kTileCols + c) = v;
-  }
-
-  const int row0 = threadIdx.y * kTM, col0 = threadIdx.x * kTN;
-  float acc[kTM][kTN];
+  // Epilogue: node-local scattering and absorption, minus xi * d_x u.  The
+  // thread's columns lie in one node per row.  P~[m][q] = p_{(m - q) mod M}:
+  // the T weights of ordinate q are those of q - 1 moved by one, so that T
+  // ordinates take 2 T weights, half of them from the T before; kHR rows at
+  // a time (registers).
+  constexpr int kHR = T == 4 ? 4 : 2;
+  const int c0 = tx * T, r = c0 / M, mb = c0 - r * M, j = j0 + r;
 #pragma unroll
-  for (int r = 0; r < kTM; ++r)
+  for (int h = 0; h < T / kHR; ++h) {
+    auto row_of = [&](int ii) { return ((h * kHR + ii) / 4) * 4 * ts.nty + ty * 4 + (h * kHR + ii) % 4; };
+    float s[kHR][T], w[2 * T];
 #pragma unroll
-    for (int c = 0; c < kTN; ++c) acc[r][c] = 0.f;
-  gemm_rows(a.DyT, n, npad, kpad, Bs, As, row0, col0, acc);
-
-  // AB4 update (eq. RTEAB4) for this thread's outputs.
-  const int w = col0 / M, mb = col0 - w * M, i = i0 + w;
-  const bool col_ok = w < cols_per_tile && i < nx;
-  float eta[kTN];
+    for (int ii = 0; ii < kHR; ++ii)
 #pragma unroll
-  for (int t = 0; t < kTN; ++t) eta[t] = __ldg(a.eta + mb + t);
+      for (int t = 0; t < T; ++t) s[ii][t] = 0.f;
+    // w[T + d] = p_{mb - q + d}, d in [-T, T)
+    auto load_w = [&](int k, float* dst) {             // p_k .. p_{k + T - 1}
+      k = k < 0 ? k + M : k;
 #pragma unroll
-  for (int jj = 0; jj < kTM; ++jj) {
-    const int j = row0 + jj;
-    if (!col_ok || j >= n) {
+      for (int v = 0; v < T / 4; ++v) {
+        const float4 p4 = *reinterpret_cast<const float4*>(Ps + k + 4 * v);
+        dst[4 * v] = p4.x; dst[4 * v + 1] = p4.y; dst[4 * v + 2] = p4.z; dst[4 * v + 3] = p4.w;
+      }
+    };
+    load_w(mb, w + T);
+    const float* ub[kHR];
 #pragma unroll
-      for (int t = 0; t < kTN; ++t) acc[jj][t] = 0.f;
-      continue;
-    }
-    const size_t base = goff + (static_cast<size_t>(j) * nx + i) * M + mb;
-    const float4 r0 = *reinterpret_cast<const float4*>(R + base);
-    const float4 r1 = *reinterpret_cast<const float4*>(R + base + 4);
-    const float4 p0 = *reinterpret_cast<const float4*>(L1 + base);
-    const float4 p1 = *reinterpret_cast<const float4*>(L1 + base + 4);
-    const float4 q0 = *reinterpret_cast<const float4*>(L2 + base);
-    const float4 q1 = *reinterpret_cast<const float4*>(L2 + base + 4);
-    const float4 s0 = *reinterpret_cast<const float4*>(L3 + base);
-    const float4 s1 = *reinterpret_cast<const float4*>(L3 + base + 4);
-    const float rv[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
-    const float l1[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
-    const float l2[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
-    const float l3[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
-    if constexpr (TR) {
-      // transposed step: ubar = w^{k+1} + L^T v (readout term and BC^T below)
+    for (int ii = 0; ii < kHR; ++ii) ub[ii] = Bs + row_of(ii) * ldb + r * M;
+    for (int q = 0; q < M; q += T) {
+      load_w(mb - q - T, w);
 #pragma unroll
-      for (int t = 0; t < kTN; ++t) acc[jj][t] = rv[t] - eta[t] * acc[jj][t] + l1[t];
-      continue;
-    }
-    float lk[8];
+      for (int q4 = 0; q4 < T / 4; ++q4) {
+        float u[kHR][4];
 #pragma unroll
-    for (int t = 0; t < kTN; ++t) {
-      lk[t] = rv[t] - eta[t] * acc[jj][t];
-      const float incr = kAB0 * lk[t] + kAB1 * l1[t] + kAB2 * l2[t] + kAB3 * l3[t];
-      acc[jj][t] = fmaf(a.cdt, incr, Bs[j * kTileCols + col0 + t]);   // u^{k+1}, pre-BC
-    }
-    reinterpret_cast<float4*>(L3 + base)[0] = make_float4(lk[0], lk[1], lk[2], lk[3]);
-    reinterpret_cast<float4*>(L3 + base)[1] = make_float4(lk[4], lk[5], lk[6], lk[7]);
-  }
-  __syncthreads();   // every thread has read u^k from Bs
-#pragma unroll
-  for (int jj = 0; jj < kTM; ++jj) {
-    const int j = row0 + jj;
-    if (j < kpad) {
-      *reinterpret_cast<float4*>(Bs + j * kTileCols + col0) =
-          make_float4(acc[jj][0], acc[jj][1], acc[jj][2], acc[jj][3]);
-      *reinterpret_cast<float4*>(Bs + j * kTileCols + col0 + 4) =
-          make_float4(acc[jj][4], acc[jj][5], acc[jj][6], acc[jj][7]);
-    }
-  }
-  __syncthreads();
-
-  // Boundary condition (eq. RTE third line) from the pre-BC values in Bs,
-  // store, and the exitance of eq. (OpMed) on boundary nodes.  One warp per
-  // grid node, lanes over ordinates.
-  const int lane = tid & 31, warp = tid >> 5, nwarps = nthr >> 5;
-  const int ncols = min(cols_per_tile, nx - i0);
-  const int ring_len = 2 * n + 2 * nx;
-  for (int cell = warp; cell < n * ncols; cell += nwarps) {
-    const int j = cell / ncols, wc = cell - j * ncols, ic = i0 + wc;
-    float* pre = Bs + j * kTileCols + wc * M;
-    const bool lf = ic == 0, rt = ic == nx - 1, bt = j == 0, tp = j == n - 1;
-    const bool bnd = lf || rt || bt || tp;
-    float* dst = Ug + (static_cast<size_t>(j) * nx + ic) * M;
-    if constexpr (TR) {
-      // Transposed step on this node: the readout transpose on the ring
-      // (every face the node lies on), w = BC^T ubar, then the transposed
-      // AB4 combination v' = c dt (chi0 w + chi1 w^{k+1} + chi2 w^{k+2} + chi3 w^{k+3}).
-      int tb = -1;
-      if (bnd) {
-        const float* eb = b.ebar + (static_cast<size_t>(g) * b.ebar_len + src_step) * ring_len;
-        for (int m = lane; m < M; m += 32) {
-          float v = pre[m];
-          if (lf || rt) v = fmaf(b.wexit[(lf ? 0 : 1) * M + m], eb[lf ? j : n + j], v);
-          if (bt || tp) v = fmaf(b.wexit[(bt ? 2 : 3) * M + m], eb[bt ? 2 * n + ic : 2 * n + nx + ic], v);
-          pre[m] = v;
+        for (int ii = 0; ii < kHR; ++ii) {
+          const float4 u4 = *reinterpret_cast<const float4*>(ub[ii] + q + 4 * q4);
+          u[ii][0] = u4.x; u[ii][1] = u4.y; u[ii][2] = u4.z; u[ii][3] = u4.w;
         }
-        __syncwarp();
-        tb = ((lf || rt) && (bt || tp)) ? 4 + (rt ? 1 : 0) + (tp ? 2 : 0) : (lf ? 0 : rt ? 1 : bt ? 2 : 3);
-      }
-      const size_t e0 = goff + (static_cast<size_t>(j) * nx + ic) * M;
-      for (int m = lane; m < M; m += 32) {
-        float wv = pre[m];
-        if (tb >= 0) {
-          const int* src = b.bct_src + (tb * M + m) * 4;
-          const float* cf = b.bct_f + (tb * M + m) * 4;
-          wv = 0.f;
 #pragma unroll
-          for (int q = 0; q < 4; ++q) wv = fmaf(cf[q], pre[src[q]], wv);
+        for (int t = 0; t < 4; ++t)
+#pragma unroll
+          for (int ii = 0; ii < kHR; ++ii)
+#pragma unroll
+            for (int e = 0; e < T; ++e) s[ii][e] = fmaf(w[T - (4 * q4 + t) + e], u[ii][t], s[ii][e]);
+      }
+#pragma unroll
+      for (int e = 0; e < T; ++e) w[T + e] = w[e];
+    }
+#pragma unroll
+    for (int ii = 0; ii < kHR; ++ii) {
+      const int i = row_of(ii);
+      if (i < n && j < a.ny) {
+        const size_t cell = static_cast<size_t>(j) * n + i;
+        const float av = __ldg(a.mua + cell), bv = __ldg(a.mus + cell);
+        float* dst = R + static_cast<size_t>(g) * a.plane + cell * M + mb;
+#pragma unroll
+        for (int v = 0; v < T / 4; ++v) {
+          const float4 u4 = *reinterpret_cast<const float4*>(Bs + i * ldb + c0 + 4 * v);
+          const float4 xi = __ldg(reinterpret_cast<const float4*>(a.xi + mb + 4 * v));
+          const float* ac = &acc[h * kHR + ii][4 * v];
+          const float* sv = &s[ii][4 * v];
+          *reinterpret_cast<float4*>(dst + 4 * v) =
+              make_float4(bv * sv[0] - (av + bv) * u4.x - xi.x * ac[0], bv * sv[1] - (av + bv) * u4.y - xi.y * ac[1],
+                          bv * sv[2] - (av + bv) * u4.z - xi.z * ac[2], bv * sv[3] - (av + bv) * u4.w - xi.w * ac[3]);
         }
-        const float incr = kAB0 * wv + kAB1 * L1[e0 + m] + kAB2 * L2[e0 + m] + kAB3 * L3[e0 + m];
-        L3[e0 + m] = wv;
-        dst[m] = a.cdt * incr;
-      }
-      continue;
-    }
-    if (!bnd) {
-      for (int m = lane; m < M; m += 32) dst[m] = pre[m];
-      continue;
-    }
-    const int* refl;
-    const float* fco;
-    const unsigned char* act;
-    if ((lf || rt) && (bt || tp)) {
-      const int c = (rt ? 1 : 0) + (tp ? 2 : 0);
-      refl = b.corner_refl + c * M; fco = b.corner_f + c * M; act = b.corner_act + c * M;
-    } else {
-      const int F = lf ? 0 : rt ? 1 : bt ? 2 : 3;
-      refl = b.face_refl + F * M; fco = b.face_f + F * M; act = b.face_act + F * M;
-    }
-    // ring node used for the source data (x-face index at corners)
-    const int node = lf ? j : rt ? n + j : bt ? 2 * n + ic : 2 * n + nx + ic;
-    float ex_x = 0.f, ex_y = 0.f;
-    for (int m = lane; m < M; m += 32) {
-      float v = pre[m];
-      if (act[m]) {
-        float q = 0.f;
-        for (int k = 0; k < b.kmax; ++k) {
-          const size_t gk = static_cast<size_t>(g) * b.kmax + k;
-          q = fmaf(b.S[gk * ring_len + node] * b.A[gk * M + m], b.T[gk * b.T_len + src_step], q);
-        }
-        if (b.rho)
-          q = fmaf(1.0f - fco[m], b.rho[(static_cast<size_t>(g) * b.rho_len + src_step) * ring_len + node], q);
-        v = fmaf(fco[m], pre[refl[m]], q);
-      }
-      dst[m] = v;
-      if (lf || rt) ex_x = fmaf(b.wexit[(lf ? 0 : 1) * M + m], v, ex_x);
-      if (bt || tp) ex_y = fmaf(b.wexit[(bt ? 2 : 3) * M + m], v, ex_y);
-    }
-    if (b.ring_out && ring_step >= 0) {
-      float* ro = b.ring_out + (static_cast<size_t>(g) * b.ring_steps + ring_step) * ring_len;
-      if (lf || rt) {
-        ex_x = warp_sum(ex_x);
-        if (lane == 0) ro[lf ? j : n + j] = ex_x;
-      }
-      if (bt || tp) {
-        ex_y = warp_sum(ex_y);
-        if (lane == 0) ro[bt ? 2 * n + ic : 2 * n + nx + ic] = ex_y;
       }
     }
   }
 }
 
-size_t pass_smem(int n, int M, bool xpass) {
-  const int npad = round_up(n, kRowPad), kpad = round_up(n, kKC);
-  size_t f = static_cast<size_t>(kpad) * kTileCols + static_cast<size_t>(kKC) * npad;
-  if (xpass) f += static_cast<size_t>(M) * M;
-  return f * sizeof(float);
+// TR: the transposed step of the discrete adjoint (BoundaryArgs::bct_src);
+// a separate instance, so that the forward step compiles without it.
+template <int T, bool TR>
+__global__ void __launch_bounds__(kMaxThreads) ypass_kernel(StepArgs a, BoundaryArgs b, TileShape ts,
+                                                            float* __restrict__ U, const float* __restrict__ R,
+                                                            const float* __restrict__ L1,
+                                                            const float* __restrict__ L2, float* __restrict__ L3,
+                                                            int src_step, int ring_step) {
+  extern __shared__ __align__(16) float smem[];
+  const int nx = a.nx, n = a.ny, M = a.M, ldb = ts.BN + kSlabPad;
+  float* Bs = smem;                                   // [rows][ldb]
+  float* As = Bs + simt_rows(n) * ldb;                // [kRing][kKC][ld]
+  // boundary tables: faces 0..3, corners 4..7; the factor and the reflected
+  // ordinate (its own with the sign bit set where nothing is imposed)
+  int2* bct = reinterpret_cast<int2*>(As + kRing * kKC * simt_ld(n));   // [8][M]
+  float* wexit = reinterpret_cast<float*>(bct + 8 * M);             // [4][M]
+  float* src0 = wexit + 4 * M;       // [node of the tile]: the first beam's S
+  float* srho = src0 + tile_nodes(n, M, ts.BN);                     // [node of the tile]: rho
+  // the tiles with an x-face, whose epilogue takes longest, start first
+  const int g = blockIdx.z;
+  const int tile = blockIdx.x == 0 ? 0 : blockIdx.x == 1 ? gridDim.x - 1 : blockIdx.x - 1;
+  const int i0 = tile * ts.per_tile;
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  int tx, ty;
+  thread_place(ts, tx, ty);
+  const size_t goff = static_cast<size_t>(g) * a.plane;
+  float* Ug = U + goff;
+  for (int e = tid; e < 8 * M; e += nthr) {
+    const bool face = e < 4 * M;
+    const int k = face ? e : e - 4 * M;
+    const bool act = (face ? b.face_act[k] : b.corner_act[k]) != 0;
+    bct[e] = make_int2(__float_as_int(face ? b.face_f[k] : b.corner_f[k]),
+                       act ? (face ? b.face_refl[k] : b.corner_refl[k]) : static_cast<int>(0x80000000u | (k % M)));
+    if (face) wexit[e] = b.wexit[k];
+  }
+  // Boundary nodes of the tile: the left face's, the right one's, the y-faces'
+  // (those that are not corners; false past the grid).  Their S and rho are
+  // asked for before the GEMM.
+  const int ring_len = 2 * n + 2 * nx;
+  const int n_l = i0 == 0 ? n : 0, n_r = i0 + ts.per_tile >= nx ? n : 0, n_nodes = n_l + n_r + 2 * ts.per_tile;
+  auto node_at = [&](int q, int& i, int& j) {
+    if (q < n_l + n_r) {
+      i = q < n_l ? 0 : nx - 1;
+      j = q < n_l ? q : q - n_l;
+      return true;
+    }
+    q -= n_l + n_r;
+    j = q < ts.per_tile ? 0 : n - 1;
+    i = i0 + (q < ts.per_tile ? q : q - ts.per_tile);
+    return i > 0 && i < nx - 1;
+  };
+  // ring node of the source data (x-face index at corners)
+  auto ring_node = [&](int i, int j) {
+    return i == 0 ? j : i == nx - 1 ? n + j : j == 0 ? 2 * n + i : 2 * n + nx + i;
+  };
+  if constexpr (!TR)
+    for (int q = tid; q < n_nodes; q += nthr) {
+      int i, j;
+      if (!node_at(q, i, j)) continue;
+      if (b.kmax > 0) src0[q] = __ldg(b.S + static_cast<size_t>(g) * b.kmax * ring_len + ring_node(i, j));
+      if (b.rho) srho[q] = __ldg(b.rho + (static_cast<size_t>(g) * b.rho_len + src_step) * ring_len + ring_node(i, j));
+    }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // slab row k: u[k][i0 + w][m] at column w M + m (contiguous)
+  const int cw = ts.BN / 4, ck = tid / cw, cc = (tid - ck * cw) * 4, nrow = nthr / cw;
+  const bool c_ok = ck < nrow && i0 + cc / M < nx;
+  const float* csrc = Ug + (c_ok ? static_cast<size_t>(i0) * M + cc : 0);
+  auto copy_slab = [&](int k0) {
+    if (ck < nrow)
+      for (int k = ck; k < kKC; k += nrow) {
+        const bool ok = c_ok && k0 + k < n;
+        cp_async16(Bs + (k0 + k) * ldb + cc, csrc + (ok ? static_cast<size_t>(k0 + k) * nx * M : 0), ok);
+      }
+  };
+  float acc[T][T];
+  tile_gemm<T>(a.DyT, n, ts, Bs, As, tx, ty, copy_slab, acc);
+  asm volatile("griddepcontrol.launch_dependents;");
+
+  // AB4 update (eq. RTEAB4); interior nodes are finished here, boundary nodes
+  // keep u^{k+1} before the boundary condition (TR: ubar) in acc.
+  auto row_of = [&](int jj) { return (jj / 4) * 4 * ts.nty + ty * 4 + jj % 4; };
+  auto is_bnd = [&](int i, int j) { return i == 0 || i == nx - 1 || j == 0 || j == n - 1; };
+  auto ld4 = [](const float* p) { return *reinterpret_cast<const float4*>(p); };
+#pragma unroll
+  for (int v = 0; v < T / 4; ++v) {
+    const int c0 = tx * T + 4 * v, w = c0 / M, mb = c0 - w * M, i = i0 + w;
+    const float4 eta = __ldg(reinterpret_cast<const float4*>(a.eta + mb));
+    const size_t base0 = goff + static_cast<size_t>(i) * M + mb;
+#pragma unroll
+    for (int jj = 0; jj < T; ++jj) {
+      const int j = row_of(jj);
+      if (i >= nx || j >= n) continue;
+      float* ac = &acc[jj][4 * v];
+      const size_t base = base0 + static_cast<size_t>(j) * nx * M;
+      const float4 r4 = ld4(R + base), p4 = ld4(L1 + base), q4 = ld4(L2 + base), s4 = ld4(L3 + base);
+      if constexpr (TR) {
+        // transposed step: ubar = w^{k+1} + L^T v
+        ac[0] = r4.x - eta.x * ac[0] + p4.x;
+        ac[1] = r4.y - eta.y * ac[1] + p4.y;
+        ac[2] = r4.z - eta.z * ac[2] + p4.z;
+        ac[3] = r4.w - eta.w * ac[3] + p4.w;
+        if (!is_bnd(i, j)) {
+          *reinterpret_cast<float4*>(U + base) =
+              make_float4(a.cdt * (kAB0 * ac[0] + kAB1 * p4.x + kAB2 * q4.x + kAB3 * s4.x),
+                          a.cdt * (kAB0 * ac[1] + kAB1 * p4.y + kAB2 * q4.y + kAB3 * s4.y),
+                          a.cdt * (kAB0 * ac[2] + kAB1 * p4.z + kAB2 * q4.z + kAB3 * s4.z),
+                          a.cdt * (kAB0 * ac[3] + kAB1 * p4.w + kAB2 * q4.w + kAB3 * s4.w));
+          *reinterpret_cast<float4*>(L3 + base) = make_float4(ac[0], ac[1], ac[2], ac[3]);
+        }
+      } else {
+        const float4 u4 = ld4(Bs + j * ldb + c0);
+        float4 lk;
+        lk.x = r4.x - eta.x * ac[0];
+        lk.y = r4.y - eta.y * ac[1];
+        lk.z = r4.z - eta.z * ac[2];
+        lk.w = r4.w - eta.w * ac[3];
+        ac[0] = fmaf(a.cdt, kAB0 * lk.x + kAB1 * p4.x + kAB2 * q4.x + kAB3 * s4.x, u4.x);
+        ac[1] = fmaf(a.cdt, kAB0 * lk.y + kAB1 * p4.y + kAB2 * q4.y + kAB3 * s4.y, u4.y);
+        ac[2] = fmaf(a.cdt, kAB0 * lk.z + kAB1 * p4.z + kAB2 * q4.z + kAB3 * s4.z, u4.z);
+        ac[3] = fmaf(a.cdt, kAB0 * lk.w + kAB1 * p4.w + kAB2 * q4.w + kAB3 * s4.w, u4.w);
+        *reinterpret_cast<float4*>(L3 + base) = lk;
+        if (!is_bnd(i, j)) *reinterpret_cast<float4*>(U + base) = make_float4(ac[0], ac[1], ac[2], ac[3]);
+      }
+    }
+  }
+
+  // Boundary nodes: the values before the boundary condition go to the slab's
+  // place, and all threads share the nodes, four ordinates each, in a rolled
+  // loop (unrolled over a thread's own outputs the code of this part did not
+  // fit the instruction cache).
+  __syncthreads();                                    // every thread has read u^k and the operator
+#pragma unroll
+  for (int v = 0; v < T / 4; ++v) {
+    const int c0 = tx * T + 4 * v, i = i0 + c0 / M;
+#pragma unroll
+    for (int jj = 0; jj < T; ++jj) {
+      const int j = row_of(jj);
+      const float* ac = &acc[jj][4 * v];
+      if (i < nx && j < n && is_bnd(i, j))
+        *reinterpret_cast<float4*>(Bs + j * ldb + c0) = make_float4(ac[0], ac[1], ac[2], ac[3]);
+    }
+  }
+  __syncthreads();
+  const int V = M / 4, n_items = n_nodes * V;         // four ordinates each
+  auto item = [&](int e, int& q, int& i, int& j, int& m) {
+    q = e / V;
+    m = (e - q * V) * 4;
+    return node_at(q, i, j);
+  };
+  if constexpr (TR) {                                 // the readout transpose on every face the node lies on
+    const float* eb = b.ebar + (static_cast<size_t>(g) * b.ebar_len + src_step) * ring_len;
+    for (int e = tid; e < n_items; e += nthr) {
+      int q, i, j, m;
+      if (!item(e, q, i, j, m)) continue;
+      float* pre = Bs + j * ldb + (i - i0) * M + m;
+      const float ex = i == 0 || i == nx - 1 ? __ldg(eb + (i == 0 ? j : n + j)) : 0.f;
+      const float ey = j == 0 || j == n - 1 ? __ldg(eb + (j == 0 ? 2 * n + i : 2 * n + nx + i)) : 0.f;
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        float x = pre[t];
+        if (i == 0 || i == nx - 1) x = fmaf(wexit[(i == 0 ? 0 : 1) * M + m + t], ex, x);
+        if (j == 0 || j == n - 1) x = fmaf(wexit[(j == 0 ? 2 : 3) * M + m + t], ey, x);
+        pre[t] = x;
+      }
+    }
+    __syncthreads();
+  }
+  // Boundary condition (eq. RTE third line), and the four ordinates' part of
+  // the exitance of eq. (OpMed): x-faces in px[j][column / 4], y-faces in
+  // py[face][column / 4], in the operator's place, which is large enough for
+  // tiles of up to 64 columns (kRing kKC ld >= ld BN / 4 + BN / 2).
+  const int cq = ts.BN / 4;
+  float* px = As;
+  float* py = As + simt_ld(n) * cq;
+  for (int e = tid; e < n_items; e += nthr) {
+    int nd, i, j, m;
+    if (!item(e, nd, i, j, m)) continue;
+    const int c0 = (i - i0) * M + m;
+    const bool lf = i == 0, rt = i == nx - 1, bt = j == 0, tp = j == n - 1;
+    const float* pre = Bs + j * ldb + (i - i0) * M;
+    const int tb = ((lf || rt) && (bt || tp)) ? 4 + (rt ? 1 : 0) + (tp ? 2 : 0) : (lf ? 0 : rt ? 1 : bt ? 2 : 3);
+    const size_t base = goff + (static_cast<size_t>(j) * nx + i) * M + m;
+    if constexpr (TR) {
+      // w = BC^T ubar, then v' = c dt (chi0 w + chi1 w^{k+1} + chi2 w^{k+2} + chi3 w^{k+3})
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int* src = b.bct_src + (tb * M + m + t) * 4;
+        const float* cf = b.bct_f + (tb * M + m + t) * 4;
+        float wv = 0.f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) wv = fmaf(__ldg(cf + q), pre[__ldg(src + q)], wv);
+        U[base + t] = a.cdt * (kAB0 * wv + kAB1 * L1[base + t] + kAB2 * L2[base + t] + kAB3 * L3[base + t]);
+        L3[base + t] = wv;
+      }
+    } else {
+      float q[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int k = 0; k < b.kmax; ++k) {
+        const size_t gk = static_cast<size_t>(g) * b.kmax + k;
+        const float sk = k == 0 ? src0[nd] : __ldg(b.S + gk * ring_len + ring_node(i, j));
+        const float tk = __ldg(b.T + gk * b.T_len + src_step);
+        const float4 ak = __ldg(reinterpret_cast<const float4*>(b.A + gk * M + m));
+        q[0] = fmaf(sk * ak.x, tk, q[0]);
+        q[1] = fmaf(sk * ak.y, tk, q[1]);
+        q[2] = fmaf(sk * ak.z, tk, q[2]);
+        q[3] = fmaf(sk * ak.w, tk, q[3]);
+      }
+      const float rho = b.rho ? srho[nd] : 0.f;
+      float x[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const int2 en = bct[tb * M + m + t];
+        const float fco = __int_as_float(en.x);
+        if (b.rho) q[t] = fmaf(1.0f - fco, rho, q[t]);
+        const float z = fmaf(fco, pre[en.y & 0x7fffffff], q[t]);
+        x[t] = en.y >= 0 ? z : pre[m + t];
+      }
+      *reinterpret_cast<float4*>(U + base) = make_float4(x[0], x[1], x[2], x[3]);
+      auto part = [&](int face) {
+        const float* we = wexit + face * M + m;
+        return fmaf(we[3], x[3], fmaf(we[2], x[2], fmaf(we[1], x[1], we[0] * x[0])));
+      };
+      if (lf || rt) px[j * cq + c0 / 4] = part(lf ? 0 : 1);
+      if (bt || tp) py[(bt ? 0 : cq) + c0 / 4] = part(bt ? 2 : 3);
+    }
+  }
+  if (TR || ring_step < 0) return;
+  __syncthreads();
+  // exitance of a boundary node: its M / 4 parts in order
+  float* ro = b.ring_out + (static_cast<size_t>(g) * b.ring_steps + ring_step) * ring_len;
+  auto node_sum = [&](const float* q) {
+    float e = q[0];
+    for (int k = 1; k < M / 4; ++k) e += q[k];
+    return e;
+  };
+  if (i0 == 0)
+    for (int j = tid; j < n; j += nthr) ro[j] = node_sum(px + j * cq);
+  if (i0 + ts.per_tile >= nx)
+    for (int j = tid; j < n; j += nthr) ro[n + j] = node_sum(px + j * cq + (nx - 1 - i0) * (M / 4));
+  for (int k = tid; k < 2 * ts.per_tile; k += nthr) {
+    const int face = k / ts.per_tile, w = k - face * ts.per_tile;
+    if (i0 + w < nx) ro[2 * n + face * nx + i0 + w] = node_sum(py + face * cq + w * (M / 4));
+  }
 }
 
 __global__ void fluence_kernel(const float* __restrict__ U, float* __restrict__ out,
@@ -699,35 +868,106 @@ __global__ void __launch_bounds__(kBalThreads)
 
 }  // namespace
 
+namespace {
+
+struct TilePlan {
+  TileShape ts;
+  int T, tiles;                      // outputs per thread T x T; tiles per group
+  size_t smem;
+};
+
+// Tile of a pass: n positions per line, `lines` lines per group.
+//
+// Eight by eight outputs a thread where that leaves every SM eight warps, in
+// tiles of 32 columns (256^2, M = 32, four groups: 215 us a step; 64 columns
+// 242; four by four 266).  Otherwise four by four, whose threads are four
+// times as many (64^2, M = 16, one group: 12 us against 26; 203 x 131, M =
+// 24, three groups: 62 against 85), in the widest tile of up to 64 columns
+// that still makes 128 CTAs (64^2, M = 32, four groups: 17 us with 64 columns
+// and 128 CTAs, 22 with 32 and 256), and otherwise in the narrowest of at
+// least four warps (64^2, M = 16, one group: 12.2 with 32, 13.3 with 64).
+TilePlan plan_tile(int n, int lines, int M, int G, bool xpass) {
+  constexpr int kSms = 152;
+  TilePlan p{};
+  const long long outputs = static_cast<long long>(n) * lines * M * G;
+  auto tiles = [&](int per) { return (lines + per - 1) / per; };
+  auto threads4 = [&](int per) { return simt_ld(n) / 4 * (per * M / 4); };
+  int per = 1;
+  if (outputs >= 64LL * 256 * kSms || threads4(1) > kMaxThreads) {
+    p.T = 8;
+    per = M < 32 ? 32 / M : 1;
+  } else {
+    p.T = 4;
+    const int last = M < 64 ? 64 / M : 1;
+    while (per < last && threads4(per) < 128) ++per;
+    for (int k = per + 1; k <= last && threads4(k) <= kMaxThreads && static_cast<long long>(tiles(k)) * G >= 128; ++k)
+      per = k;
+  }
+  p.ts.per_tile = per;
+  p.ts.BN = per * M;
+  p.ts.ntx = p.ts.BN / p.T;
+  p.ts.nty = simt_ld(n) / p.T;
+  p.tiles = tiles(per);
+  p.smem = tile_smem(n, M, p.ts.BN, xpass);
+  return p;
+}
+
+// Launches a pass with programmatic serialisation: the passes wait for the
+// launch before them (griddepcontrol.wait) after their prologue and let the
+// one behind them in after their GEMM, so that launch and prologue of a pass
+// overlap the epilogue of the pass before (64^2, M = 16: 16.6 us a step
+// without, 13.2 when let in at the start, 12 after the GEMM; let in at the
+// start, a grid that leaves SMs free is followed by CTAs that crowd on those).
+template <auto Kernel, class... A>
+cudaError_t launch_tile(const TilePlan& p, int G, cudaStream_t s, const A&... args) {
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+  if (attr != cudaSuccess) return attr;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(p.tiles, 1, G);
+  cfg.blockDim = dim3(p.ts.ntx * p.ts.nty);
+  cfg.dynamicSmemBytes = p.smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, Kernel, args...);
+}
+
+template <int T>
+cudaError_t launch_x(const TilePlan& p, const StepArgs& a, const float* U, float* R, cudaStream_t s) {
+  return launch_tile<xpass_kernel<T>>(p, a.G, s, a, p.ts, U, R);
+}
+
+template <int T, bool XT>
+cudaError_t launch_y(const TilePlan& p, const StepArgs& a, const BoundaryArgs& b, float* U, const float* R,
+                     const float* L1, const float* L2, float* L3, int step, cudaStream_t s) {
+  return launch_tile<ypass_kernel<T, XT>>(p, a.G, s, a, b, p.ts, U, R, L1, L2, L3, step, b.ring_out ? step : -1);
+}
+
+}  // namespace
+
 cudaError_t launch_step(const StepArgs& a, const BoundaryArgs& b, float* U, float* R,
                         const float* L1, const float* L2, float* L3, int step,
                         cudaStream_t s, long long* launches, cudaEvent_t* ev) {
   if (a.tc_mode != 0) return launch_step_tc(a, b, U, R, L1, L2, L3, step, s, launches, ev);
-  static bool attr_done = false;
-  const size_t smx = pass_smem(a.nx, a.M, true), smy = pass_smem(a.ny, a.M, false);
-  if (!attr_done) {
-    cudaFuncSetAttribute(xpass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-    cudaFuncSetAttribute(ypass_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-    cudaFuncSetAttribute(ypass_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-    attr_done = true;
-  }
-  const int per_tile = kTileCols / a.M;
-  // npad / kTM rows of threads: 8 x (multiple of 4) = whole warps.
-  dim3 bx(kTileCols / kTN, round_up(a.nx, kRowPad) / kTM);
-  dim3 gx((a.ny + per_tile - 1) / per_tile, 1, a.G);
+  const TilePlan px = plan_tile(a.nx, a.ny, a.M, a.G, true), py = plan_tile(a.ny, a.nx, a.M, a.G, false);
   if (ev) cudaEventRecord(ev[0], s);
-  xpass_kernel<<<gx, bx, smx, s>>>(a, U, R);
+  cudaError_t e = px.T == 8 ? launch_x<8>(px, a, U, R, s) : launch_x<4>(px, a, U, R, s);
   if (ev) cudaEventRecord(ev[1], s);
-  dim3 by(kTileCols / kTN, round_up(a.ny, kRowPad) / kTM);
-  dim3 gy((a.nx + per_tile - 1) / per_tile, 1, a.G);
-  const int ring_step = b.ring_out ? step : -1;
-  if (b.bct_src)
-    ypass_kernel<true><<<gy, by, smy, s>>>(a, b, U, R, L1, L2, L3, step, ring_step);
-  else
-    ypass_kernel<false><<<gy, by, smy, s>>>(a, b, U, R, L1, L2, L3, step, ring_step);
+  if (e == cudaSuccess) {
+    if (b.bct_src)
+      e = py.T == 8 ? launch_y<8, true>(py, a, b, U, R, L1, L2, L3, step, s)
+                    : launch_y<4, true>(py, a, b, U, R, L1, L2, L3, step, s);
+    else
+      e = py.T == 8 ? launch_y<8, false>(py, a, b, U, R, L1, L2, L3, step, s)
+                    : launch_y<4, false>(py, a, b, U, R, L1, L2, L3, step, s);
+  }
   if (ev) cudaEventRecord(ev[2], s);
   if (launches) *launches += 2;
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_fluence(const float* U, float* out, size_t out_group_stride, int nx, int ny,

@@ -4,9 +4,11 @@
 
 namespace rte_kern {
 
-// Columns of one pass tile: (rows or columns of the grid) x ordinates.
-constexpr int kTileCols = 64;
-constexpr int kTM = 8, kTN = 8, kKC = 16;
+// Operator array of the SIMT passes: E^T, padded with zeros to whole chunks
+// of kKC rows and rows of whole thread tiles.
+constexpr int kKC = 16;
+__host__ __device__ constexpr int simt_ld(int n) { return (n + 15) / 16 * 16; }
+__host__ __device__ constexpr int simt_rows(int n) { return (n + kKC - 1) / kKC * kKC; }
 
 // Boundary/source description shared by the y-pass epilogue.
 struct BoundaryArgs {
@@ -45,7 +47,7 @@ struct BoundaryArgs {
 struct StepArgs {
   int nx, ny, M, G;
   size_t plane;                     // ny*nx*M floats per group
-  const float* DxT;                 // [nx][nx], DxT[k*nx + i] = D_x[i][k]
+  const float* DxT;                 // [simt_rows(nx)][simt_ld(nx)], DxT[k][i] = D_x[i][k], zero-padded
   const float* DyT;
   const float* PT;                  // [M][M], PT[q*M + m] = P~[m][q]
   const float* xi;                  // [M]
