@@ -98,8 +98,6 @@ __device__ __forceinline__ void tc_pass_body(const StepArgs& a, const BoundaryAr
 
   // A launch after a timed-out one does nothing (the march reports the error).
   if (*static_cast<volatile int*>(a.err)) return;
-  // x-pass: the y-pass that follows may be scheduled as soon as CTAs leave.
-  if (XPASS) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   unsigned char* sm = smraw + ((1024 - (smem_u32(smraw) & 1023)) & 1023);
   unsigned char* Psm = sm + L.stage_bytes;    // P~ image (x-pass, TC scattering)
   const uint32_t bar_full = smem_u32(&bars[0]), bar_done = smem_u32(&bars[1]);
@@ -120,6 +118,7 @@ __device__ __forceinline__ void tc_pass_body(const StepArgs& a, const BoundaryAr
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = tmem_slot;
+  bool ok = true;
   // Failure injection (tests): one CTA waits on a barrier that nothing
   // arrives on, before this CTA has issued any copy or MMA, so that the
   // bounded wait runs out and sets the timeout word; the CTA then frees its
@@ -134,6 +133,18 @@ __device__ __forceinline__ void tc_pass_body(const StepArgs& a, const BoundaryAr
       return;
     }
   }
+  // Dependent launches.  An x-pass waits here for the y-pass before it (u^k)
+  // and then lets its y-pass in, whose main loop reads only u^k and D_y and
+  // so may overlap the x-pass; the y-pass waits for the x-pass before its
+  // epilogue, and has let the next x-pass in, which waits here.  Either lets
+  // its follower in with its tensor memory in hand: a CTA that waits for this
+  // launch never holds what this launch still has to allocate.
+  if (XPASS) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // a wait of the launch before that ran out meanwhile
+    if (*static_cast<volatile int*>(a.err)) ok = false;
+  }
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if constexpr (XPASS && SCAT_TC) {
     if (tid == 0) bulk_copy(smem_u32(Psm), a.PImg, kPBytes, bar_p);
   }
@@ -145,7 +156,6 @@ __device__ __forceinline__ void tc_pass_body(const StepArgs& a, const BoundaryAr
   const uint32_t idesc_base = (1u << 4) | (kFmt << 7) | (kFmt << 10) | (static_cast<uint32_t>(kMT >> 4) << 24);
   const uint32_t idesc_x = idesc_base | (static_cast<uint32_t>(kNC >> 3) << 17);
   const size_t chunk_bytes = static_cast<size_t>(2) * nrows_img * 128;   // hi + lo tiles of one K chunk
-  bool ok = true;
 
   // ---------------- main loop over K chunks ----------------
   // Slab^T chunk: S[c][kk] = -scale_m u(c, k0 + kk).  Each thread owns 4
@@ -743,8 +753,7 @@ cudaError_t launch_one(const StepArgs& a, const BoundaryArgs& b, float* U, float
                                                                           ring_step);
     return cudaGetLastError();
   }
-  // programmatic dependent launch: may start while the preceding x-pass's
-  // last CTAs run (see the wait before the y epilogue)
+  // programmatic dependent launch (see the waits in tc_pass_body)
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = dim3(kThreads);
@@ -804,11 +813,7 @@ cudaError_t launch_batched_one(const BatchProblem* probs, const BatchProblem* de
                          232448 - 2048);
     attr = true;
   }
-  if (XPASS) {
-    tc_pass_batched<XPASS, PREC, MM, SCAT_TC><<<ctas, kThreads, smem, s>>>(dev, n, step, hl);
-    return cudaGetLastError();
-  }
-  // the y-pass as a programmatic dependent of the batched x-pass before it
+  // programmatic dependent launches (see tc_pass_body)
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ctas);
   cfg.blockDim = dim3(kThreads);
@@ -899,7 +904,7 @@ cudaError_t launch_step_tc(const StepArgs& a, const BoundaryArgs& b, float* U, f
   const bool ystream = tma && a.x_variant == 5 && tc_ystream_supported(a);
   e = ws       ? launch_pass_ws(true, a, b, U, R, L1, L2, L3, step, ring_step, s)
       : stream ? launch_xpass_stream(a, b, U, R, s)
-               : launch_mode<true>(a, b, U, R, L1, L2, L3, step, ring_step, s);
+               : launch_mode<true>(a, b, U, R, L1, L2, L3, step, ring_step, s, !ev);
   if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[1], s);
   e = ws        ? launch_pass_ws(false, a, b, U, R, L1, L2, L3, step, ring_step, s)
