@@ -16,6 +16,7 @@
 // The same passes take the transposed step of the exact discrete adjoint
 // (BoundaryArgs::bct_src set): transposed D operators in the GEMMs and the
 // transposed AB4 / boundary / readout bookkeeping in the y-pass epilogue.
+#include <algorithm>
 #include <cstdint>
 
 #include "rte_kernels.cuh"
@@ -601,20 +602,29 @@ __device__ __forceinline__ void ld32b(const float* ptr, float* v) {
                : "l"(ptr));
 }
 
+// A cell's groups are shared by `split` neighbouring lanes (a power of two; the
+// FP32 sums of a lane's groups are added in FP64), so that small grids with
+// many groups fill the chip: 64^2, 16 groups, M = 32: 33 us with one lane per
+// cell, whose groups come one after another, 7 us with sixteen.
+constexpr long long kGradThreads = 152 * 256;
+
 template <int MM>
 __device__ __forceinline__ void grad_node(const float* __restrict__ MU, const float* __restrict__ Useg,
                                           const float* __restrict__ PT, const float* __restrict__ area,
-                                          long long cell, int G, size_t plane, size_t useg_gs, double scale,
-                                          int flip, const GradLevels lv, double* __restrict__ grad_a,
+                                          long long t, int ncell, int G, int split, size_t plane, size_t useg_gs,
+                                          double scale, int flip, const GradLevels lv, double* __restrict__ grad_a,
                                           double* __restrict__ grad_b) {
+  const int lane = static_cast<int>(t) & (split - 1);
+  const long long cell = t / split;
+  const bool valid = cell < ncell;
   float p[MM];
 #pragma unroll
   for (int d = 0; d < MM; ++d) p[d] = __ldg(PT + d);            // P~[0][d] = p_d (symmetric circulant)
-  const double k = area ? scale * static_cast<double>(area[cell]) : scale;
-  double da = grad_a ? grad_a[cell] : 0.0, db = grad_b ? grad_b[cell] : 0.0;
+  const double k = area && valid ? scale * static_cast<double>(area[cell]) : scale;
+  double ga = valid && grad_a ? grad_a[cell] : 0.0, gb = valid && grad_b ? grad_b[cell] : 0.0;
   for (int l = 0; l < lv.n; ++l) {
     float sa = 0.f, sb = 0.f;
-    for (int g = 0; g < G; ++g) {
+    for (int g = valid ? lane : G; g < G; g += split) {
       const float* u = Useg + l * lv.u_step + static_cast<size_t>(g) * useg_gs + static_cast<size_t>(cell) * MM;
       const float* mu = MU + l * lv.mu_step + static_cast<size_t>(g) * plane + static_cast<size_t>(cell) * MM;
       float uu[MM], lam[MM];
@@ -633,11 +643,24 @@ __device__ __forceinline__ void grad_node(const float* __restrict__ MU, const fl
         sb = fmaf(x, uu[m] - pu, sb);
       }
     }
-    da -= k * static_cast<double>(sa);
-    db -= k * static_cast<double>(sb);
+    double da = static_cast<double>(sa), db = static_cast<double>(sb);
+    for (int o = 1; o < split; o <<= 1) {
+      da += __shfl_xor_sync(0xffffffffu, da, o);
+      db += __shfl_xor_sync(0xffffffffu, db, o);
+    }
+    ga -= k * da;
+    gb -= k * db;
   }
-  if (grad_a) grad_a[cell] = da;
-  if (grad_b) grad_b[cell] = db;
+  if (!valid || lane != 0) return;
+  if (grad_a) grad_a[cell] = ga;
+  if (grad_b) grad_b[cell] = gb;
+}
+
+// Lanes per cell, until every SM has eight warps.
+__host__ __device__ inline int grad_split(long long ncell, int G) {
+  int split = 1;
+  while (2 * split <= G && split < 16 && ncell * split < kGradThreads) split *= 2;
+  return split;
 }
 
 // Any M: one warp per cell, the lanes over the ordinates, the row of P~ from
@@ -681,13 +704,13 @@ __device__ __forceinline__ bool grad_by_thread(int M) { return M == 16 || M == 3
 
 __global__ void grad_kernel(const float* __restrict__ MU, const float* __restrict__ Useg,
                             const float* __restrict__ PT, const float* __restrict__ area, int ncell,
-                            int M, int G, size_t plane, size_t useg_gs, double scale, int flip, GradLevels lv,
+                            int M, int G, int split, size_t plane, size_t useg_gs, double scale, int flip,
+                            GradLevels lv,
                             double* __restrict__ grad_a, double* __restrict__ grad_b) {
   const long long t = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (grad_by_thread(M)) {
-    if (t >= ncell) return;
-    if (M == 32) grad_node<32>(MU, Useg, PT, area, t, G, plane, useg_gs, scale, flip, lv, grad_a, grad_b);
-    else grad_node<16>(MU, Useg, PT, area, t, G, plane, useg_gs, scale, flip, lv, grad_a, grad_b);
+    if (M == 32) grad_node<32>(MU, Useg, PT, area, t, ncell, G, split, plane, useg_gs, scale, flip, lv, grad_a, grad_b);
+    else grad_node<16>(MU, Useg, PT, area, t, ncell, G, split, plane, useg_gs, scale, flip, lv, grad_a, grad_b);
     return;
   }
   const long long cell = t >> 5;
@@ -704,9 +727,11 @@ __global__ void grad_batch_kernel(const GradJob* __restrict__ jobs, int slot, in
   const float* useg = j.seg + static_cast<size_t>(slot) * j.slot_floats;
   const GradLevels one{1, 0, 0};
   if (grad_by_thread(j.M)) {
-    if (t >= j.ncell) return;
-    if (j.M == 32) grad_node<32>(j.MU, useg, j.PT, j.area, t, j.G, j.plane, j.plane, j.scale, flip, one, j.grad_a, j.grad_b);
-    else grad_node<16>(j.MU, useg, j.PT, j.area, t, j.G, j.plane, j.plane, j.scale, flip, one, j.grad_a, j.grad_b);
+    const int nc = static_cast<int>(j.ncell);
+    if (j.M == 32)
+      grad_node<32>(j.MU, useg, j.PT, j.area, t, nc, j.G, grad_split(nc, j.G), j.plane, j.plane, j.scale, flip, one, j.grad_a, j.grad_b);
+    else
+      grad_node<16>(j.MU, useg, j.PT, j.area, t, nc, j.G, grad_split(nc, j.G), j.plane, j.plane, j.scale, flip, one, j.grad_a, j.grad_b);
     return;
   }
   const long long cell = t >> 5;
@@ -1015,9 +1040,11 @@ cudaError_t launch_rho(const float* resid, const float* Wn, int n_det, int ring_
 
 cudaError_t launch_grad_batch(const GradJob* jobs_dev, int n_jobs, int max_ncell, int m_common, int slot,
                               int flip, cudaStream_t s, long long* launches) {
-  // one thread per cell for M in {16, 32} (every medium of a batch shares M)
   dim3 grid((max_ncell * 32 + 255) / 256, n_jobs);
-  if (m_common == 16 || m_common == 32) grid.x = (max_ncell + 255) / 256;
+  // M in {16, 32} (every medium of a batch shares M): grad_split lanes per
+  // cell, fewer than 2 kGradThreads where that is more than one
+  if (m_common == 16 || m_common == 32)
+    grid.x = static_cast<unsigned>((std::max<long long>(max_ncell, 2 * kGradThreads) + 255) / 256);
   grad_batch_kernel<<<grid, 256, 0, s>>>(jobs_dev, slot, flip);
   if (launches) *launches += 1;
   return cudaGetLastError();
@@ -1051,8 +1078,9 @@ cudaError_t launch_grad(const float* MU, const float* Useg, const float* PT, con
                         double scale, int flip, GradLevels lv, double* grad_a, double* grad_b,
                         cudaStream_t s, long long* launches) {
   const int ncell = nx * ny;
-  const long long threads = (M == 16 || M == 32) ? ncell : 32LL * ncell;
-  grad_kernel<<<static_cast<int>((threads + 255) / 256), 256, 0, s>>>(MU, Useg, PT, area, ncell, M, G, plane,
+  const int split = grad_split(ncell, G);
+  const long long threads = (M == 16 || M == 32) ? static_cast<long long>(ncell) * split : 32LL * ncell;
+  grad_kernel<<<static_cast<int>((threads + 127) / 128), 128, 0, s>>>(MU, Useg, PT, area, ncell, M, G, split, plane,
                                                                       useg_group_stride, scale, flip, lv, grad_a,
                                                                       grad_b);
   if (launches) *launches += 1;
