@@ -9,14 +9,14 @@
 // owned block plus a two-point halo: the "box".  Per step the CTA
 //   1. copies the box of u^k (owned + halo, from the input state buffer)
 //      into shared memory (cp.async);
-//   2. x-lines (row, m): lbuf = -xi_m D_x,seg u    (two lines per thread,
-//      sharing float4 operator loads, paired FP32 FMAs);
-//   3. y-lines (column, m): lbuf += -eta_m D_y,seg u;
-//   4. per node (one warp, or half a warp at M = 16, over the ordinates):
-//      L^k = lbuf + b P~u - (a + b) u, the AB4 update, the Fresnel boundary
-//      condition with beam or adjoint injection on physical boundary nodes
-//      (eq. RTE), the exitance ring (eq. OpMed); writes u^{k+1} to the output
-//      state buffer and L^k over the oldest history slot.
+//   2. x- and y-derivatives, side by side: half of the threads take x-lines
+//      (row, four ordinates), the other half y-lines (column, four
+//      ordinates); lbuf = -xi_m D_x,seg u, then lbuf += -eta_m D_y,seg u;
+//   3. per node and eight ordinates, a thread: L^k = lbuf + b P~u - (a + b) u,
+//      the AB4 update, the Fresnel boundary condition with beam or adjoint
+//      injection on physical boundary nodes (eq. RTE), the exitance ring (eq.
+//      OpMed); writes u^{k+1} to the output state buffer and L^k over the
+//      oldest history slot.
 // Neighbouring CTAs read this CTA's owned values as their halo during the
 // same step, so input and output states are different buffers.
 //
@@ -24,8 +24,16 @@
 // written: about 25 B against the two-pass form's 36 B, and 2 (s_x + s_y) +
 // 2 M flops of operator and scattering work instead of 2 (n_x + n_y) + 2 M.
 // The history is not staged in shared memory (that would leave one CTA per
-// SM): each warp streams it through registers one batch of nodes ahead, the
-// first batch while the derivatives are formed.
+// SM): a thread loads a node's while it works on the one before.
+//
+// What bounds it: shared-memory reads.  A 16-byte load returns 512 bytes a
+// warp, four cycles of the SM however few distinct words it asks for.  With
+// one ordinate per lane in the scattering (eight such loads for 32
+// multiply-adds a lane) and two lines per thread in the derivatives (4.5 for
+// 64) the loads took 16 k cycles of the SM per CTA against 4.6 k of FP32
+// multiply-adds.  Eight ordinates per thread share the node's u, with the
+// whole circulant in registers, and four lines share the operator: 6 k.
+// 256^2, M = 32, 16 groups, 16 x 16 parts: 279 -> 192 us a step.
 #include <cstdint>
 
 #include "rte_kernels.cuh"
@@ -49,12 +57,13 @@ __device__ __forceinline__ void cp16(float* dst, const float* src) {
 
 // Shared-memory layout (floats) of one CTA for MM ordinates and at most OM
 // owned points per axis; every region starts on a 16-byte boundary.  About
-// 88 KB at M = 32: two CTAs per SM.
+// 99 KB at M = 32: two CTAs per SM.
 template <int MM, int OM>
 struct FusedSmem {
   static constexpr int kBox = OM + 2 * kHalo;                      // box side (nodes)
-  static constexpr int kRow = kBox * MM + (MM == 16 ? 16 : 0);     // box row stride
-  static constexpr int kOwn = OM * OM * MM;                        // owned values
+  static constexpr int kN = MM + 4;                                // node stride: neighbours in different banks
+  static constexpr int kRow = kBox * kN;                           // box row stride
+  static constexpr int kOwn = OM * OM * kN;                        // owned values
   static constexpr int kBoxF = kBox * kRow;
   static constexpr int kOpF = (OM + 2 * kHalo) * OM;               // [k < seg][i < OM]
   static constexpr int kTotal = kBoxF + kOwn + 2 * kOpF + 2 * OM * OM;
@@ -69,9 +78,46 @@ __device__ __forceinline__ float group_sum(float v, int width) {
   return v;
 }
 
-// Node passes of the per-node phase whose history loads are in flight
-// together (a register pipeline one batch ahead; larger batches spill at
-// 128 registers).
+// 32 bytes of global memory (32-byte aligned: eight ordinates of a node).
+__device__ __forceinline__ void ld32(const float* p, float (&v)[8]) {
+  asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+               : "l"(p)
+               : "memory");
+}
+__device__ __forceinline__ void st32(float* p, const float (&v)[8]) {
+  asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+               "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+               : "memory");
+}
+
+// Derivative of four lines (neighbouring ordinates, u at line + k stride) at
+// kOut owned points: acc[q][t] holds points 2 q and 2 q + 1 of line t.  op:
+// [k][OM], the points in question first.
+template <int OM, int kOut>
+__device__ __forceinline__ void derive(const float* line, int stride, const float* op, int n_k,
+                                       float2 (&acc)[kOut / 2][4]) {
+#pragma unroll
+  for (int q = 0; q < kOut / 2; ++q)
+#pragma unroll
+    for (int t = 0; t < 4; ++t) acc[q][t] = make_float2(0.f, 0.f);
+#pragma unroll 4
+  for (int k = 0; k < n_k; ++k) {
+    const float4 u4 = *reinterpret_cast<const float4*>(line + k * stride);
+    const float2 uu[4] = {make_float2(u4.x, u4.x), make_float2(u4.y, u4.y), make_float2(u4.z, u4.z),
+                          make_float2(u4.w, u4.w)};
+    const float4* dk = reinterpret_cast<const float4*>(op + k * OM);
+#pragma unroll
+    for (int q = 0; q < kOut / 4; ++q) {
+      const float4 c = dk[q];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        acc[2 * q][t] = fma2(make_float2(c.x, c.y), uu[t], acc[2 * q][t]);
+        acc[2 * q + 1][t] = fma2(make_float2(c.z, c.w), uu[t], acc[2 * q + 1][t]);
+      }
+    }
+  }
+}
 
 template <int MM, int OM, bool EXACT>
 __global__ void __launch_bounds__(kFThreads, 2)
@@ -79,12 +125,9 @@ __global__ void __launch_bounds__(kFThreads, 2)
                       const float* __restrict__ L1, const float* __restrict__ L2, float* __restrict__ L3,
                       int src_step, int ring_step) {
   using S = FusedSmem<MM, OM>;
-  constexpr int kPerWarp = 32 / MM;                  // nodes per warp pass
-  constexpr int kWarps = kFThreads / 32;
-  constexpr int kBatch = 4;
   extern __shared__ __align__(16) float sm[];
   float* box = sm;                                  // [kBox][kRow]: node (x_lo-2+ib, y_lo-2+jb)
-  float* lbuf = box + S::kBoxF;                     // [ny_own][nx_own][MM]
+  float* lbuf = box + S::kBoxF;                     // [ny_own][nx_own][kN]
   float* dxs = lbuf + S::kOwn;                      // [k < sx][i < OM]
   float* dys = dxs + S::kOpF;                       // [k < sy][j < OM]
   float* abs_ = dys + S::kOpF;                      // [2][ny_own][nx_own]: a, b
@@ -98,11 +141,27 @@ __global__ void __launch_bounds__(kFThreads, 2)
   const int ox = EXACT ? OM : x_hi - x_lo, oy = EXACT ? OM : y_hi - y_lo;
   const int sx = x_shi - x_slo, sy = y_shi - y_slo;
   const int own = ox * oy;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int m = lane % MM, sub = lane / MM;
+  const int tid = threadIdx.x;
   const size_t goff = static_cast<size_t>(g) * a.plane;
   const float* Ug = Uin + goff;
 
+  // The part's history is asked for from L2 at once (lines of 32 floats): its
+  // loads come when the derivatives are done (256^2, 16 groups: 203 us a step
+  // without, 194 with; loaded into registers here instead, 245: spills).
+  {
+    const int per_row = ox * MM / 32;
+    for (int q = tid; q < oy * per_row; q += kFThreads) {
+      const int row = q / per_row, c = q - row * per_row;
+      const size_t at = goff + (static_cast<size_t>(y_lo + row) * nx + x_lo) * M + c * 32;
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(L1 + at));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(L2 + at));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(L3 + at));
+    }
+  }
+  // Dependent launches: a step waits here for the step before it, and lets
+  // the next one in when its derivatives are done (two groups: 33.5 us a step
+  // without, 31 with).
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   // 1. The box of u^k by cp.async: rows of the y-segment; owned rows span the
   //    x-segment, fringe rows the owned columns.
   {
@@ -113,39 +172,10 @@ __global__ void __launch_bounds__(kFThreads, 2)
       const int c0 = owned_row ? x_slo : x_lo, c1 = owned_row ? x_shi : x_hi;
       const int items = (c1 - c0) * V;
       const float* src = Ug + (static_cast<size_t>(gj) * nx + c0) * M;
-      float* dst = box + (gj - y_lo + kHalo) * S::kRow + (c0 - x_lo + kHalo) * MM;
-      for (int e = tid; e < items; e += kFThreads) cp16(dst + 4 * e, src + 4 * e);
+      float* dst = box + (gj - y_lo + kHalo) * S::kRow + (c0 - x_lo + kHalo) * S::kN;
+      for (int e = tid; e < items; e += kFThreads) cp16(dst + e / V * S::kN + e % V * 4, src + 4 * e);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
-  }
-  // Node passes of the per-node phase: warp w takes the owned rows
-  // w, w + kWarps, ..., each in ppr passes of kPerWarp nodes (lane group sub
-  // takes column pass * kPerWarp + sub).  A cursor (row, column) walks them
-  // without divisions; columns past the row end mirror node (0, 0).
-  const int ppr = (ox + kPerWarp - 1) / kPerWarp;
-  const int n_pass = (warp < oy ? (oy - warp + kWarps - 1) / kWarps : 0) * ppr;
-  auto advance = [&](int& jl, int& il) {
-    il += kPerWarp;
-    if (il >= ppr * kPerWarp) {
-      il = sub;
-      jl += kWarps;
-    }
-  };
-  auto hist_index = [&](int jl, int il) {
-    const bool ok = jl < oy && il < ox;
-    return goff + (static_cast<size_t>(y_lo + (ok ? jl : 0)) * nx + x_lo + (ok ? il : 0)) * M + m;
-  };
-  // History of this warp's first batch of passes, in flight while the
-  // derivatives are formed.
-  int pj = warp, pi = sub;                          // prefetch cursor
-  float h1[kBatch], h2[kBatch], h3[kBatch];
-#pragma unroll
-  for (int t = 0; t < kBatch; ++t) {
-    const size_t e = hist_index(pj, pi);
-    h1[t] = __ldg(L1 + e);
-    h2[t] = __ldg(L2 + e);
-    h3[t] = L3[e];
-    advance(pj, pi);
   }
   // Segment operators of this part (transposed: [k][i]), the phase matrix,
   // and the owned block of a and b.
@@ -166,211 +196,132 @@ __global__ void __launch_bounds__(kFThreads, 2)
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   __syncthreads();
 
-  // 2. x-lines: line l = (row jl, ordinate m); outputs i < ox.
+  // 2. The derivatives: threads 0 .. 127 the x-lines of (row, ordinates 4 mq
+  //    ..), the others the y-lines of (column, ...); with 16 ordinates two
+  //    threads share a line's owned points.
   {
-    const int nl = oy * MM;
-    const int xoff = (x_slo - x_lo + kHalo) * MM;
-    for (int l0 = tid; l0 < nl; l0 += 2 * kFThreads) {
-      const int l1 = l0 + kFThreads < nl ? l0 + kFThreads : l0;
-      const int j0 = l0 / MM, m0 = l0 - j0 * MM, j1 = l1 / MM, m1 = l1 - j1 * MM;
-      const float* r0 = box + (j0 + kHalo) * S::kRow + xoff + m0;
-      const float* r1 = box + (j1 + kHalo) * S::kRow + xoff + m1;
-      float2 acc0[OM / 2], acc1[OM / 2];
+    constexpr int kHalf = kFThreads / 2, MQ = MM / 4;
+    constexpr int kSplit = kHalf / (OM * MQ), kOut = OM / kSplit;
+    static_assert(kSplit * OM * MQ == kHalf, "one item per thread");
+    const bool xhalf = tid < kHalf;
+    const int ht = xhalf ? tid : tid - kHalf;
+    const int m0 = (ht % MQ) * 4, rest = ht / MQ, p0 = (rest % kSplit) * kOut, l = rest / kSplit;
+    const bool on = l < (xhalf ? oy : ox);
+    // interior parts have the full segment (owned range + two fringe points
+    // on each side): a fixed trip count
+    const int n_seg = xhalf ? sx : sy;
+    const int n_k = !on ? 0 : (EXACT && n_seg == OM + 2 * kHalo) ? OM + 2 * kHalo : n_seg;
+    const float* line = xhalf ? box + (l + kHalo) * S::kRow + (x_slo - x_lo + kHalo) * S::kN + m0
+                              : box + (y_slo - y_lo + kHalo) * S::kRow + (l + kHalo) * S::kN + m0;
+    float2 acc[kOut / 2][4];
+    derive<OM, kOut>(line, xhalf ? S::kN : S::kRow, (xhalf ? dxs : dys) + p0, n_k, acc);
+    const float4 w4 = __ldg(reinterpret_cast<const float4*>((xhalf ? a.xi : a.eta) + m0));
+    // point p of the line: node (row l, column p) or (row p, column l)
+    auto at = [&](int p) { return lbuf + (xhalf ? l * ox + p : p * ox + l) * S::kN + m0; };
+    if (on && xhalf) {
 #pragma unroll
-      for (int i = 0; i < OM / 2; ++i) acc0[i] = acc1[i] = make_float2(0.f, 0.f);
-      // interior parts have the full segment (owned range + two fringe
-      // points on each side): a fixed trip count
-      const int kx_n = (EXACT && sx == OM + 2 * kHalo) ? OM + 2 * kHalo : sx;
-#pragma unroll 4
-      for (int k = 0; k < kx_n; ++k) {
-        const float u0 = r0[k * MM], u1 = r1[k * MM];
-        const float2 uu0 = make_float2(u0, u0), uu1 = make_float2(u1, u1);
-        const float4* dk = reinterpret_cast<const float4*>(dxs + k * OM);
-#pragma unroll
-        for (int q = 0; q < OM / 4; ++q) {
-          if (4 * q < ox) {
-            const float4 c = dk[q];
-            const float2 clo = make_float2(c.x, c.y), chi = make_float2(c.z, c.w);
-            acc0[2 * q] = fma2(clo, uu0, acc0[2 * q]);
-            acc0[2 * q + 1] = fma2(chi, uu0, acc0[2 * q + 1]);
-            acc1[2 * q] = fma2(clo, uu1, acc1[2 * q]);
-            acc1[2 * q + 1] = fma2(chi, uu1, acc1[2 * q + 1]);
-          }
-        }
-      }
-      const float xi0 = -__ldg(a.xi + m0), xi1 = -__ldg(a.xi + m1);
-#pragma unroll
-      for (int i = 0; i < OM; ++i) {
-        if (i < ox) {
-          const float v0 = (i & 1) ? acc0[i / 2].y : acc0[i / 2].x;
-          const float v1 = (i & 1) ? acc1[i / 2].y : acc1[i / 2].x;
-          lbuf[(j0 * ox + i) * MM + m0] = xi0 * v0;
-          if (l1 != l0) lbuf[(j1 * ox + i) * MM + m1] = xi1 * v1;
-        }
+      for (int i = 0; i < kOut; ++i) {
+        if (p0 + i >= ox) continue;
+        auto v = [&](int t) { return (i & 1) ? acc[i / 2][t].y : acc[i / 2][t].x; };
+        *reinterpret_cast<float4*>(at(p0 + i)) = make_float4(-w4.x * v(0), -w4.y * v(1), -w4.z * v(2), -w4.w * v(3));
       }
     }
+    __syncthreads();
+    if (on && !xhalf) {
+#pragma unroll
+      for (int i = 0; i < kOut; ++i) {
+        if (p0 + i >= oy) continue;
+        auto v = [&](int t) { return (i & 1) ? acc[i / 2][t].y : acc[i / 2][t].x; };
+        float4* d = reinterpret_cast<float4*>(at(p0 + i));
+        const float4 x = *d;
+        *d = make_float4(fmaf(-w4.x, v(0), x.x), fmaf(-w4.y, v(1), x.y), fmaf(-w4.z, v(2), x.z),
+                         fmaf(-w4.w, v(3), x.w));
+      }
+    }
+    __syncthreads();
   }
-  __syncthreads();
 
-  // 3. y-lines: line l = (column il, ordinate m); outputs j < oy.
-  {
-    const int nl = ox * MM;
-    const int yoff = (y_slo - y_lo + kHalo) * S::kRow;
-    for (int l0 = tid; l0 < nl; l0 += 2 * kFThreads) {
-      const int l1 = l0 + kFThreads < nl ? l0 + kFThreads : l0;
-      const int i0 = l0 / MM, m0 = l0 - i0 * MM, i1 = l1 / MM, m1 = l1 - i1 * MM;
-      const float* c0 = box + yoff + (i0 + kHalo) * MM + m0;
-      const float* c1 = box + yoff + (i1 + kHalo) * MM + m1;
-      float2 acc0[OM / 2], acc1[OM / 2];
+  asm volatile("griddepcontrol.launch_dependents;");
+  // 3. Per node and eight ordinates mb .. mb + 7: scattering, L^k, AB4,
+  //    boundary condition, exitance.  P~[m][q] = p_{(m - q) mod M}: a thread
+  //    keeps p_{mb + k}, k = 0 .. M - 1.
+  constexpr int NB = MM / 8, kNodes = kFThreads / NB;          // threads per node, nodes per sweep
+  const int mb = (tid % NB) * 8;
+  float p[MM];
 #pragma unroll
-      for (int j = 0; j < OM / 2; ++j) acc0[j] = acc1[j] = make_float2(0.f, 0.f);
-      const int ky_n = (EXACT && sy == OM + 2 * kHalo) ? OM + 2 * kHalo : sy;
-#pragma unroll 4
-      for (int k = 0; k < ky_n; ++k) {
-        const float u0 = c0[k * S::kRow], u1 = c1[k * S::kRow];
-        const float2 uu0 = make_float2(u0, u0), uu1 = make_float2(u1, u1);
-        const float4* dk = reinterpret_cast<const float4*>(dys + k * OM);
+  for (int k = 0; k < MM; ++k) p[k] = __ldg(a.PT + (mb + k) % MM);
+  const int ring_len = 2 * ny + 2 * nx;
+  const bool interior = x_lo > 0 && x_hi < nx && y_lo > 0 && y_hi < ny;   // CTA-uniform: no boundary node
+  auto place = [&](int n, int& jl, int& il) {
+    const int nn = n < own ? n : 0;
+    jl = nn / ox;
+    il = nn - jl * ox;
+    return goff + (static_cast<size_t>(y_lo + jl) * nx + x_lo + il) * M + mb;
+  };
+  float h1[8], h2[8], h3[8];
+  int jl, il;
+  size_t e = place(tid / NB, jl, il);
+  ld32(L1 + e, h1);
+  ld32(L2 + e, h2);
+  ld32(L3 + e, h3);
+  for (int n0 = 0; n0 < own; n0 += kNodes) {
+    const int n = n0 + tid / NB;
+    const bool valid = n < own;
+    float g1[8], g2[8], g3[8];
+    int jn, in;
+    const size_t en = place(n + kNodes, jn, in);
+    const bool more = n + kNodes < own;
 #pragma unroll
-        for (int q = 0; q < OM / 4; ++q) {
-          if (4 * q < oy) {
-            const float4 c = dk[q];
-            const float2 clo = make_float2(c.x, c.y), chi = make_float2(c.z, c.w);
-            acc0[2 * q] = fma2(clo, uu0, acc0[2 * q]);
-            acc0[2 * q + 1] = fma2(chi, uu0, acc0[2 * q + 1]);
-            acc1[2 * q] = fma2(clo, uu1, acc1[2 * q]);
-            acc1[2 * q + 1] = fma2(chi, uu1, acc1[2 * q + 1]);
-          }
-        }
-      }
-      const float et0 = -__ldg(a.eta + m0), et1 = -__ldg(a.eta + m1);
+    for (int t = 0; t < 8; ++t) g1[t] = g2[t] = g3[t] = 0.f;
+    if (more) {
+      ld32(L1 + en, g1);
+      ld32(L2 + en, g2);
+      ld32(L3 + en, g3);
+    }
+    const float* un = box + (jl + kHalo) * S::kRow + (il + kHalo) * S::kN;
+    float s0[8], s1[8];                                        // even and odd q
 #pragma unroll
-      for (int j = 0; j < OM; ++j) {
-        if (j < oy) {
-          const float v0 = (j & 1) ? acc0[j / 2].y : acc0[j / 2].x;
-          const float v1 = (j & 1) ? acc1[j / 2].y : acc1[j / 2].x;
-          lbuf[(j * ox + i0) * MM + m0] = fmaf(et0, v0, lbuf[(j * ox + i0) * MM + m0]);
-          if (l1 != l0) lbuf[(j * ox + i1) * MM + m1] = fmaf(et1, v1, lbuf[(j * ox + i1) * MM + m1]);
-        }
+    for (int t = 0; t < 8; ++t) s0[t] = s1[t] = 0.f;
+#pragma unroll
+    for (int q = 0; q < MM; q += 4) {
+      const float4 v = *reinterpret_cast<const float4*>(un + q);
+#pragma unroll
+      for (int t = 0; t < 8; ++t) {
+        s0[t] = fmaf(p[(t - q + 2 * MM) % MM], v.x, s0[t]);
+        s1[t] = fmaf(p[(t - q - 1 + 2 * MM) % MM], v.y, s1[t]);
+        s0[t] = fmaf(p[(t - q - 2 + 2 * MM) % MM], v.z, s0[t]);
+        s1[t] = fmaf(p[(t - q - 3 + 2 * MM) % MM], v.w, s1[t]);
       }
     }
-  }
-  __syncthreads();
-
-  // 4. Per node: scattering, L^k, AB4, boundary condition, exitance; the
-  //    history of the next batch of passes is loaded while this one runs.
-  {
-    float prow[MM];
+    float* lb = lbuf + (jl * ox + il) * S::kN;
+    const float av = abs_[jl * ox + il], bv = abs_[OM * OM + jl * ox + il];
+    float lk[8], v[8];
 #pragma unroll
-    for (int q = 0; q < MM; ++q) prow[q] = __ldg(a.PT + q * MM + m);   // P~[m][q]: lanes read consecutive words
-    const int ring_len = 2 * ny + 2 * nx;
-    // An interior subdomain of the exact size has no node on the physical
-    // boundary, and its passes form a fixed grid (each warp's owned rows x the
-    // column passes), so every index below is a constant offset from the
-    // thread's bases.  Same arithmetic, in the same order, as the general
-    // loop that follows; the first batch's history (loaded before the
-    // derivatives) is for the same nodes.
-    const bool interior = EXACT && x_lo > 0 && x_hi < nx && y_lo > 0 && y_hi < ny;   // CTA-uniform
-    if (interior) {
-      constexpr int kRowsW = OM / kWarps;                        // owned rows per warp
-      constexpr int kColP = OM / kPerWarp;                       // column passes per row
-      constexpr int kPass = kRowsW * kColP;
-      const size_t hbase = goff + (static_cast<size_t>(y_lo + warp) * nx + x_lo + sub) * M + m;
-      const size_t hrow = static_cast<size_t>(kWarps) * nx * M;
-      auto hidx = [&](int pp) {
-        return hbase + static_cast<size_t>(pp / kColP) * hrow + static_cast<size_t>((pp % kColP) * kPerWarp) * M;
-      };
-      const float* unb = box + (warp + kHalo) * S::kRow + (sub + kHalo) * MM;
+    for (int w = 0; w < 2; ++w) {
+      const float4 l4 = *reinterpret_cast<const float4*>(lb + mb + 4 * w);
+      const float4 u4 = *reinterpret_cast<const float4*>(un + mb + 4 * w);
+      const float ll[4] = {l4.x, l4.y, l4.z, l4.w}, uu[4] = {u4.x, u4.y, u4.z, u4.w};
 #pragma unroll
-      for (int p0 = 0; p0 < kPass; p0 += kBatch) {
-        float g1[kBatch], g2[kBatch], g3[kBatch];
-#pragma unroll
-        for (int t = 0; t < kBatch; ++t) {
-          const int pp = p0 + kBatch + t;
-          g1[t] = g2[t] = g3[t] = 0.f;
-          if (pp < kPass) {
-            const size_t e = hidx(pp);
-            g1[t] = __ldg(L1 + e);
-            g2[t] = __ldg(L2 + e);
-            g3[t] = L3[e];
-          }
-        }
-#pragma unroll
-        for (int t = 0; t < kBatch; ++t) {
-          const int pp = p0 + t, rr = pp / kColP, cc = pp % kColP;
-          const float* un = unb + rr * kWarps * S::kRow + cc * kPerWarp * MM;
-          float2 s01 = make_float2(0.f, 0.f), s23 = make_float2(0.f, 0.f);
-#pragma unroll
-          for (int q = 0; q < MM; q += 4) {
-            const float4 v = *reinterpret_cast<const float4*>(un + q);
-            s01 = fma2(make_float2(prow[q], prow[q + 1]), make_float2(v.x, v.y), s01);
-            s23 = fma2(make_float2(prow[q + 2], prow[q + 3]), make_float2(v.z, v.w), s23);
-          }
-          const float sc = (s01.x + s01.y) + (s23.x + s23.y);
-          const float u = un[m];
-          const int n = (warp + kWarps * rr) * OM + sub + kPerWarp * cc;
-          const float av = abs_[n], bv = abs_[OM * OM + n];
-          const float lk = fmaf(bv, sc, lbuf[n * MM + m] - (av + bv) * u);
-          const float pre = fmaf(a.cdt, kAB0 * lk + kAB1 * h1[t] + kAB2 * h2[t] + kAB3 * h3[t], u);
-          const size_t e = hidx(pp);
-          L3[e] = lk;
-          Uout[e] = pre;
-        }
-#pragma unroll
-        for (int t = 0; t < kBatch; ++t) {
-          h1[t] = g1[t];
-          h2[t] = g2[t];
-          h3[t] = g3[t];
-        }
+      for (int r = 0; r < 4; ++r) {
+        const int t = 4 * w + r;
+        lk[t] = fmaf(bv, s0[t] + s1[t], ll[r] - (av + bv) * uu[r]);
+        v[t] = fmaf(a.cdt, kAB0 * lk[t] + kAB1 * h1[t] + kAB2 * h2[t] + kAB3 * h3[t], uu[r]);
       }
-      return;
     }
-    int cj = warp, ci = sub;                         // compute cursor
-    for (int t0 = 0; t0 < n_pass; t0 += kBatch) {
-      float g1[kBatch], g2[kBatch], g3[kBatch];
-      const bool more = t0 + kBatch < n_pass;
-#pragma unroll
-      for (int t = 0; t < kBatch; ++t) {
-        const size_t e = hist_index(pj, pi);
-        g1[t] = more ? __ldg(L1 + e) : 0.f;
-        g2[t] = more ? __ldg(L2 + e) : 0.f;
-        g3[t] = more ? L3[e] : 0.f;
-        advance(pj, pi);
-      }
-#pragma unroll
-      for (int t = 0; t < kBatch; ++t) {
-        if (t0 + t >= n_pass) break;                   // warp-uniform
-        const bool valid = ci < ox;
-        const int jl = valid ? cj : 0, il = valid ? ci : 0;
-        advance(cj, ci);
-        const int n = jl * ox + il;
-        const int gj = y_lo + jl, gi = x_lo + il;
-        const float* un = box + (jl + kHalo) * S::kRow + (il + kHalo) * MM;
-        float2 s01 = make_float2(0.f, 0.f), s23 = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int q = 0; q < MM; q += 4) {
-          const float4 v = *reinterpret_cast<const float4*>(un + q);
-          s01 = fma2(make_float2(prow[q], prow[q + 1]), make_float2(v.x, v.y), s01);
-          s23 = fma2(make_float2(prow[q + 2], prow[q + 3]), make_float2(v.z, v.w), s23);
+    if (valid) st32(L3 + e, lk);
+    if (!interior) {
+      const int gj = y_lo + jl, gi = x_lo + il;
+      const bool lf = gi == 0, rt = gi == nx - 1, bt = gj == 0, tp = gj == ny - 1;
+      const bool bnd = valid && (lf || rt || bt || tp);
+      if (__any_sync(0xffffffffu, bnd)) {
+        // pre-BC values through shared memory (this node's lbuf entries are
+        // no longer needed)
+        if (bnd) {
+          *reinterpret_cast<float4*>(lb + mb) = make_float4(v[0], v[1], v[2], v[3]);
+          *reinterpret_cast<float4*>(lb + mb + 4) = make_float4(v[4], v[5], v[6], v[7]);
         }
-        const float sc = (s01.x + s01.y) + (s23.x + s23.y);
-        const float u = un[m];
-        const float av = abs_[n], bv = abs_[OM * OM + n];
-        const int o = n * MM + m;
-        const float lk = fmaf(bv, sc, lbuf[o] - (av + bv) * u);
-        const float pre = fmaf(a.cdt, kAB0 * lk + kAB1 * h1[t] + kAB2 * h2[t] + kAB3 * h3[t], u);
-        const size_t e = goff + (static_cast<size_t>(gj) * nx + gi) * M + m;
-        const bool lf = gi == 0, rt = gi == nx - 1, bt = gj == 0, tp = gj == ny - 1;
-        const bool bnd = valid && (lf || rt || bt || tp);
-        if (valid) L3[e] = lk;
-        if (!__any_sync(0xffffffffu, bnd)) {
-          if (valid) Uout[e] = pre;
-          continue;
-        }
-        // Boundary nodes in this pass: pre-BC values through shared memory
-        // (this node's lbuf entries are no longer needed).
-        if (valid) lbuf[o] = pre;
         __syncwarp();
-        float v = pre;
+        float ex = 0.f, ey = 0.f;
         if (bnd) {
           const int* refl;
           const float* fco;
@@ -383,38 +334,47 @@ __global__ void __launch_bounds__(kFThreads, 2)
             refl = b.face_refl + F * M; fco = b.face_f + F * M; act = b.face_act + F * M;
           }
           const int node = lf ? gj : rt ? ny + gj : bt ? 2 * ny + gi : 2 * ny + nx + gi;
-          if (act[m]) {
-            float q = 0.f;
-            for (int k = 0; k < b.kmax; ++k) {
-              const size_t gk = static_cast<size_t>(g) * b.kmax + k;
-              q = fmaf(__ldg(b.S + gk * ring_len + node) * __ldg(b.A + gk * M + m),
-                       __ldg(b.T + gk * b.T_len + src_step), q);
+          float q[8];
+#pragma unroll
+          for (int t = 0; t < 8; ++t) q[t] = 0.f;
+          for (int k = 0; k < b.kmax; ++k) {
+            const size_t gk = static_cast<size_t>(g) * b.kmax + k;
+            const float sk = __ldg(b.S + gk * ring_len + node), tk = __ldg(b.T + gk * b.T_len + src_step);
+#pragma unroll
+            for (int t = 0; t < 8; ++t) q[t] = fmaf(sk * __ldg(b.A + gk * M + mb + t), tk, q[t]);
+          }
+          const float rho =
+              b.rho ? __ldg(b.rho + (static_cast<size_t>(g) * b.rho_len + src_step) * ring_len + node) : 0.f;
+#pragma unroll
+          for (int t = 0; t < 8; ++t) {
+            if (act[mb + t]) {
+              const float fc = __ldg(fco + mb + t);
+              if (b.rho) q[t] = fmaf(1.0f - fc, rho, q[t]);
+              v[t] = fmaf(fc, lb[__ldg(refl + mb + t)], q[t]);
             }
-            if (b.rho)
-              q = fmaf(1.0f - fco[m], __ldg(b.rho + (static_cast<size_t>(g) * b.rho_len + src_step) * ring_len + node), q);
-            v = fmaf(fco[m], lbuf[n * MM + refl[m]], q);
+            // exitance of the node's faces (eq. OpMed)
+            if (lf || rt) ex = fmaf(__ldg(b.wexit + (lf ? 0 : 1) * M + mb + t), v[t], ex);
+            if (bt || tp) ey = fmaf(__ldg(b.wexit + (bt ? 2 : 3) * M + mb + t), v[t], ey);
           }
         }
-        if (valid) Uout[e] = v;
-        // exitance of the node's faces (eq. OpMed), summed over its ordinates
-        float ex = 0.f, ey = 0.f;
-        if (bnd && (lf || rt)) ex = b.wexit[(lf ? 0 : 1) * M + m] * v;
-        if (bnd && (bt || tp)) ey = b.wexit[(bt ? 2 : 3) * M + m] * v;
-        ex = group_sum(ex, MM);
-        ey = group_sum(ey, MM);
-        if (bnd && m == 0 && b.ring_out && ring_step >= 0) {
+        ex = group_sum(ex, NB);
+        ey = group_sum(ey, NB);
+        if (bnd && mb == 0 && b.ring_out && ring_step >= 0) {
           float* ro = b.ring_out + (static_cast<size_t>(g) * b.ring_steps + ring_step) * ring_len;
           if (lf || rt) ro[lf ? gj : ny + gj] = ex;
           if (bt || tp) ro[bt ? 2 * ny + gi : 2 * ny + nx + gi] = ey;
         }
-        __syncwarp();
       }
+    }
+    if (valid) st32(Uout + e, v);
+    e = en;
+    jl = jn;
+    il = in;
 #pragma unroll
-      for (int t = 0; t < kBatch; ++t) {
-        h1[t] = g1[t];
-        h2[t] = g2[t];
-        h3[t] = g3[t];
-      }
+    for (int t = 0; t < 8; ++t) {
+      h1[t] = g1[t];
+      h2[t] = g2[t];
+      h3[t] = g3[t];
     }
   }
 }
@@ -431,10 +391,17 @@ cudaError_t launch_fused_t(const StepArgs& a, const BoundaryArgs& b, const float
     if (e != cudaSuccess) return e;
     attr_done = true;
   }
-  dim3 grid(a.px * a.py, a.G);
-  fused_step_kernel<MM, OM, EXACT><<<grid, kFThreads, S::kBytes, s>>>(a, b, Uin, Uout, L1, L2, L3, src_step,
-                                                                      ring_step);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(a.px * a.py, a.G);
+  cfg.blockDim = dim3(kFThreads);
+  cfg.dynamicSmemBytes = S::kBytes;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, fused_step_kernel<MM, OM, EXACT>, a, b, Uin, Uout, L1, L2, L3, src_step, ring_step);
 }
 
 template <int MM>

@@ -605,7 +605,7 @@ __device__ __forceinline__ void ld32b(const float* ptr, float* v) {
 // A cell's groups are shared by `split` neighbouring lanes (a power of two; the
 // FP32 sums of a lane's groups are added in FP64), so that small grids with
 // many groups fill the chip: 64^2, 16 groups, M = 32: 33 us with one lane per
-// cell, whose groups come one after another, 7 us with sixteen.
+// cell, whose groups come one after another, 9 us with sixteen.
 constexpr long long kGradThreads = 152 * 256;
 
 template <int MM>
