@@ -50,3 +50,35 @@ def test_multi_step_launch_matches_two_launches_per_step(nx, ny, M, groups, step
     # FP64 sums over bitwise equal recomputed states (their order may differ)
     for k in (3, 4):
         assert np.linalg.norm(a[k] - b[k]) <= 1e-7 * np.linalg.norm(b[k])
+
+
+@pytest.mark.parametrize("M,prec,steps,sizes", [
+    (32, TF32X3, 7, [(200, 140, 2), (48, 64, 1), (129, 40, 3), (300, 260, 1)]),
+    (16, BF16X3, 6, [(24, 260, 1), (257, 129, 2)]), (64, TF32, 5, [(140, 36, 1), (40, 300, 2)])])
+def test_batched_persistent_passes_match_each_medium_alone(M, prec, steps, sizes):
+    """Media with lines of more than 128 positions in one batch: the items of
+    all of them in one persistent launch per pass, states alternating between
+    two buffers (odd and even step counts, checkpoints from either)."""
+    from paper_2202_09421_gb300 import binding as B
+    from paper_2202_09421_gb300.solver import FCDOMSolver, adjoint_gradient_batch, forward_batch
+    dev = torch.device("cuda:0")
+    wls = [workload_custom(nx, ny, M, steps, 0.02, L=(nx - 1) / 66, mus=80.0 - 10 * k, n_groups=g, t_s=0.1,
+                           sigma_t=0.1, g=0.9 - 0.1 * k) for k, (nx, ny, g) in enumerate(sizes)]
+    ss = [FCDOMSolver(w.grid, w.optics, torch.tensor(w.mua, dtype=torch.float32, device=dev),
+                      torch.tensor(w.mus, dtype=torch.float32, device=dev), w.c, w.dt, precision=prec,
+                      ckpt_interval=3) for w in wls]
+    before = B.rte_kernel_launches(ss[0].ctx)
+    forward_batch(ss, [w.groups for w in wls], steps)
+    assert B.rte_kernel_launches(ss[0].ctx) - before == 2 * steps
+    curves = [s.readout(w.detectors) for s, w in zip(ss, wls)]
+    states = [[s.state(g).cpu().numpy() for g in range(len(w.groups))] for s, w in zip(ss, wls)]
+    grads = adjoint_gradient_batch(ss, [w.detectors for w in wls], [0.5 * c for c in curves])
+    for s, w, c, us, (J, ga, gb) in zip(ss, wls, curves, states, grads):
+        s.forward(w.groups, steps)
+        assert torch.equal(s.readout(w.detectors), c)
+        for g, u in enumerate(us):
+            assert np.abs(u).max() > 0 and np.array_equal(s.state(g).cpu().numpy(), u)
+        J1, ga1, gb1 = s.adjoint_gradient(w.detectors, 0.5 * c)
+        assert J == J1
+        assert torch.allclose(ga, ga1, rtol=1e-5, atol=0) and torch.allclose(gb, gb1, rtol=1e-5, atol=0)
+        s.close()
