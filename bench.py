@@ -59,20 +59,15 @@ NCU_TRAFFIC = {
     # the tomography workload's per-launch size (16 groups x 256^2 x 32),
     # keyed by the kernel and the sha256 prefix of its sources; an entry
     # whose sources changed since its capture no longer matches.
-    # TMA-fed x-pass (csrc/rte_tc_stream.cu + rte_tc_common.cuh) and the
-    # one-tile y-pass (csrc/rte_tc.cu + rte_tc_common.cuh), schedule 4:
-    # profiles/tc_stream_passes_tomo256_ncu.md
-    # TMA-fed x-pass (csrc/rte_tc_stream.cu + rte_tc_common.cuh) and the
-    # one-tile y-pass (csrc/rte_tc.cu + rte_tc_common.cuh), schedule 4:
-    # profiles/tc_stream_passes_tomo256_ncu.md
-    ("tc_pass_stream<x>", "1eb1154312966384"): 138.943232e6 + 90.579968e6,
-    ("tc_pass_kernel<y>", "5ad975b3d17dce21"): 687.169280e6 + 188.580352e6,
+    # multi-step march (csrc/rte_tc_march.cu + rte_tc_common.cuh), one launch
+    # of 8 steps, per step: profiles/march_tomo256_ncu.md
+    ("tc_march_kernel", "ef4a8deddf996317"): (6603.303680e6 + 3143.567616e6) / 8,
     # tile-local fused step (csrc/rte_fused.cu), 16 x 16 parts:
-    # profiles/fused_step_tomo256_ncu_full.md
-    ("fused_step_kernel", "09d63ccdc8189d08"): 538.545920e6 + 231.291136e6,
+    # profiles/fused_step_tomo256_ncu.md
+    ("fused_step_kernel", "0a3a711e2bec192f"): 539.476224e6 + 230.795264e6,
     # its tensor-core form (csrc/rte_fused_tc.cu + rte_tc_common.cuh):
     # profiles/fused_step_tc_tomo256_ncu.md
-    ("fused_step_tc_kernel", "36c1cad1904e669a"): 540.756736e6 + 231.811840e6,
+    ("fused_step_tc_kernel", "3bafd3fcf47785d7"): 539.331328e6 + 230.892800e6,
 }
 
 
@@ -82,6 +77,8 @@ def kernel_source_hash(name="tc_pass_ws"):
         srcs = ["rte_tc_ws.cu", "rte_tc_common.cuh"]
     elif name.startswith("tc_ypass_pipe"):
         srcs = ["rte_tc_pipe.cu", "rte_tc_common.cuh"]
+    elif name.startswith("tc_march"):
+        srcs = ["rte_tc_march.cu", "rte_tc_common.cuh"]
     elif name.startswith("tc_pass_stream"):
         srcs = ["rte_tc_stream.cu", "rte_tc_common.cuh"]
     elif name.startswith("tc_pass"):
@@ -367,16 +364,21 @@ def run_ours(args):
 
     # Rooflines.  The step: the method's algorithmic 24 B per update (read
     # u^k, L^{k-1..k-3}; write u^{k+1}, L^k) at the whole-step rate, against
-    # HBM.  The dominant pass: y-pass 28 B per update (read u, R, L1..L3;
-    # write u, L) against HBM; x-pass tensor-core flops (3 products x 2 flop
-    # x (n + M) per update) against the TF32 peak, and its 8 B per update
-    # against HBM.
+    # HBM.  Schedule 1 runs whole steps in one kernel (the multi-step march):
+    # 36 B per update (x: read u, write R; y: read u, R, L1..L3, write u, L)
+    # against HBM, and the tensor-core flops of both derivatives (3 products x
+    # 2 flop x (nx + ny) per update) against the TF32 peak.  The other
+    # schedules launch two passes per step, the dominant one being the y-pass,
+    # 28 B per update against HBM; x-pass tensor-core flops (3 products x 2
+    # flop x (n + M) per update) against the TF32 peak, and its 8 B per update
+    # against HBM.  (The library's per-pass events run schedule 1 as two
+    # passes too: pass times of that form.)
     ncell_m = g.nx * g.ny * g.M * len(wl.groups)
     step_gbs = 24.0 * updates / (ms_step / 1e3) / 1e9
     # the configuration timed: schedule = choice % 6 (0 persistent
-    # warp-specialised, 1 one tile per CTA, 2 pipelined y-pass, 4 TMA-fed
+    # warp-specialised, 1 multi-step march, 2 pipelined y-pass, 4 TMA-fed
     # persistent x-pass, 5 TMA-fed persistent x- and y-passes), choice >= 6
-    # tensor-core scattering
+    # tensor-core scattering (schedule 1: one tile per CTA)
     sched = tuned[0] % 6
     names = {0: ["tc_pass_ws<x>", "tc_pass_ws<y>"], 1: ["tc_pass_kernel<x>", "tc_pass_kernel<y>"],
              2: ["tc_pass_kernel<x>", "tc_ypass_pipe<y>"], 4: ["tc_pass_stream<x>", "tc_pass_kernel<y>"],
@@ -406,6 +408,19 @@ def run_ours(args):
                 "frac": dom_gbs / PEAKS["hbm_gbs"], "traffic": passes[names[dom]]["traffic"],
                 "kernel": names[dom], "peak_source": f"{PEAKS['source']} (MEASURED_PEAKS.json hbm_gbs)",
                 "passes": passes}
+    if tuned[0] == 1:
+        ms_k = ms_step / wl.n_steps
+        m_gbs = 36.0 * ncell_m / (ms_k / 1e3) / 1e9
+        m_tflops = 3 * 2 * (g.nx + g.ny) * ncell_m / (ms_k / 1e3) / 1e12
+        name = "tc_march_kernel"
+        traffic = NCU_TRAFFIC.get((name, kernel_source_hash(name)))
+        roofline.update({"achieved": m_gbs, "frac": m_gbs / PEAKS["hbm_gbs"], "traffic": traffic, "kernel": name,
+                         "march": {"ms_per_step": ms_k, "hbm": {"achieved": m_gbs, "bytes_per_update": 36,
+                                                                "frac": m_gbs / PEAKS["hbm_gbs"]},
+                                   "tensor": {"achieved": m_tflops, "unit": "TFLOP/s", "peak": tf32_peak,
+                                              "frac": m_tflops / tf32_peak,
+                                              "peak_source": "measured bf16 burst x 1/2 (tf32 nominal ratio)"},
+                                   "traffic": traffic}})
 
     # The other forms on the same workload: the plain FP32 SIMT form (the
     # metric's comparison) and the single-product TF32 reduced-precision form.

@@ -347,7 +347,7 @@ rte_status rte_host_segment_images(int n, double h, double alpha, double beta, i
 rte_status rte_host_bc_transpose(int M, double n_in, double n_out, int* src_out, double* f_out);
 
 /* Per-kernel timing with CUDA events on the context's stream.  While on,
- * every AB4 step records events around its two passes (x-pass: scattering
+ * every AB4 step runs as two launches, with events around its passes (x-pass: scattering
  * and x-derivative; y-pass: y-derivative, AB4, boundary condition,
  * exitance).  rte_kernel_times synchronises the stream, writes the summed
  * device time in ms of each pass (ms_out[2]) and the number of timed launches
@@ -371,7 +371,11 @@ long long rte_graph_captures(const rte_ctx* ctx);
  *   0  persistent warp-specialised x- and y-passes, one CTA per SM, where
  *      supported (tensor-core precisions; nx, ny <= 256, M in {16, 32}, no
  *      RTE_FLAG_TC_SCATTER);
- *   1  (default) one-tile-per-CTA passes;
+ *   1  (default) one-tile-per-CTA passes; in the tensor-core precisions,
+ *      without RTE_FLAG_TC_SCATTER and with a line of more than 128
+ *      positions, the same tiles as items of a persistent launch of up to
+ *      128 steps (between checkpoints and snapshots), bit for bit the same
+ *      results, also in the segments of rte_adjoint_gradient;
  *   2  one-tile-per-CTA x-pass and the pipelined persistent y-pass (the main
  *      loop of one tile and the epilogue of the previous one on two warp
  *      groups of one CTA per SM) where supported (tensor-core precisions,
@@ -395,7 +399,8 @@ long long rte_graph_captures(const rte_ctx* ctx);
  * Schedules 4 and 5 give the one-tile-per-CTA passes' results bit for bit.
  * rte_discrete_adjoint_gradient, rte_forward_batch and
  * rte_adjoint_gradient_batch run the one-tile-per-CTA passes under every
- * schedule.
+ * schedule (rte_forward_batch, with a line of more than 128 positions among
+ * the media, their tiles as items of one persistent launch per pass).
  * Unsupported sizes run the one-tile-per-CTA passes (the plain FP32 passes
  * in RTE_PREC_FP32).  Errors: INVALID_ARG. */
 rte_status rte_set_pass_variant(rte_ctx* ctx, int variant);

@@ -279,6 +279,10 @@ rte_status snapshot(rte_ctx* c, const float* u, int G, const std::vector<int>& s
                                               static_cast<float>(2.0 * kPi / c->M), c->stream, &c->launches));
 }
 
+// Steps of a multi-step launch, at most: 36 ms at 16 groups of 256^2, so that
+// work on other streams gets its turn (a launch costs about 0.1 ms of ramp).
+constexpr int kMarchSteps = 128;
+
 // Runs steps [s_begin, s_end) of the forward march on (U, R, L), starting
 // from whatever state they hold; records checkpoints/exitance/fluence when
 // asked.
@@ -316,7 +320,7 @@ rte_status march(rte_ctx* c, DevBuf& U, DevBuf& R, DevBuf* L, int& hl, int G, in
     for (int s = s_begin; s < s_end;) {
       if (save_ckpt && I > 0 && s % I == 0) RTE_TRY(copy_checkpoint(c, cur, L, hl, G, s));
       int e = s + 1;                                   // the run [s, e)
-      while (e < s_end && !(save_ckpt && I > 0 && e % I == 0) && !(fluence_out && snap_index[e - 1] >= 0)) ++e;
+      while (e < s_end && e - s < kMarchSteps && !(save_ckpt && I > 0 && e % I == 0) && !(fluence_out && snap_index[e - 1] >= 0)) ++e;
       ma.u0 = cur;
       ma.u1 = oth;
       ma.hl = hl;
@@ -1308,24 +1312,27 @@ static rte_status adjoint_impl(rte_ctx* c, const rte_detector* dets, int n_det, 
       rte_kern::MarchArgs ma;
       ma.a = sa;
       ma.b = ba;
-      ma.u0 = ma.u1 = mcur;
-      ma.slots = F(c->seg) + static_cast<size_t>(I) * gfloats;
-      ma.slot_floats = gfloats;
       for (int q = 0; q < 3; ++q) ma.L[q] = F(c->LA[q]);
-      ma.hl = hl_adj;
-      ma.step0 = s_end - 1;
       ma.dstep = -1;
-      ma.n_steps = n;
       ma.ctl = static_cast<int*>(c->ctl.p);
-      RTE_TRY(cuda_status(rte_kern::launch_march_tc(ma, c->stream, &c->launches)));
-      hl_adj = (hl_adj + 2 * n) % 3;
+      ma.slot_floats = gfloats;
+      float* mslots = F(c->seg) + static_cast<size_t>(I) * gfloats;
+      for (int o = 0; o < n; o += kMarchSteps) {
+        ma.slots = mslots + static_cast<size_t>(o) * gfloats;
+        ma.u0 = ma.u1 = o == 0 ? mcur : ma.slots - gfloats;
+        ma.hl = hl_adj;
+        ma.step0 = s_end - 1 - o;
+        ma.n_steps = std::min(kMarchSteps, n - o);
+        RTE_TRY(cuda_status(rte_kern::launch_march_tc(ma, c->stream, &c->launches)));
+        hl_adj = (hl_adj + 2 * ma.n_steps) % 3;
+      }
       // adjoint slot l is level s_end - 1 - l
       const long long step = static_cast<long long>(gfloats);
       RTE_TRY(cuda_status(rte_kern::launch_grad(
-          ma.slots, seg_ptrs(static_cast<int>(k), s0, s_end)[n - 1], F(c->PT), F(c->area), c->nx, c->ny, c->M, G,
+          mslots, seg_ptrs(static_cast<int>(k), s0, s_end)[n - 1], F(c->PT), F(c->area), c->nx, c->ny, c->M, G,
           c->plane, c->plane, scale, 1, {n, step, -step}, dJ_dmua ? D(c->grad_a) : nullptr,
           dJ_dmus ? D(c->grad_b) : nullptr, c->stream, &c->launches)));
-      RTE_TRY(cuda_status(cudaMemcpyAsync(mcur, ma.slots + static_cast<size_t>(n - 1) * gfloats, gbytes,
+      RTE_TRY(cuda_status(cudaMemcpyAsync(mcur, mslots + static_cast<size_t>(n - 1) * gfloats, gbytes,
                                           cudaMemcpyDeviceToDevice, c->stream)));
       continue;
     }
