@@ -53,6 +53,7 @@ struct rte_ctx {
   bool inject_expire = false;
   // item counters of the multi-step launches
   DevBuf ctl;
+  DevBuf mseg;                       // adjoint levels of one launch (kDualSteps at most)
   // photon balance of the last rte_forward (RTE_FLAG_PHOTON_BALANCE):
   // [G][n_steps][3] FP64 terms, block partials, per-group tickets, and the
   // FP64 cos / sin of the ordinates
@@ -282,6 +283,9 @@ rte_status snapshot(rte_ctx* c, const float* u, int G, const std::vector<int>& s
 // Steps of a multi-step launch, at most: 36 ms at 16 groups of 256^2, so that
 // work on other streams gets its turn (a launch costs about 0.1 ms of ramp).
 constexpr int kMarchSteps = 128;
+// The same for the adjoint beside a recompute: the adjoint levels of a launch
+// are kept for its gradient terms.
+constexpr int kDualSteps = 32;
 
 // Runs steps [s_begin, s_end) of the forward march on (U, R, L), starting
 // from whatever state they hold; records checkpoints/exitance/fluence when
@@ -309,7 +313,7 @@ rte_status march(rte_ctx* c, DevBuf& U, DevBuf& R, DevBuf* L, int& hl, int G, in
       RTE_TRY(cuda_status(cudaMemcpyAsync(oth, cur, gbytes, cudaMemcpyDeviceToDevice, c->stream)));
       std::swap(cur, oth);
     }
-    rte_kern::MarchArgs ma;
+    rte_kern::MarchArgs ma{};
     ma.a = a;
     ma.b = b;
     ma.slots = nullptr;
@@ -477,7 +481,7 @@ rte_status prepare_forward(rte_ctx* c, const rte_source_group* groups, int n_gro
   RTE_TRY(ensure(c->U, gbytes));
   RTE_TRY(ensure(c->R, gbytes));
   for (int q = 0; q < 3; ++q) RTE_TRY(ensure(c->L[q], gbytes));
-  RTE_TRY(ensure(c->ctl, rte_kern::tc_march_ctl_bytes(G)));
+  RTE_TRY(ensure(c->ctl, rte_kern::tc_march_ctl_bytes(2 * G)));
   RTE_TRY(ensure(c->ring, static_cast<size_t>(G) * n_steps * c->ring_len * sizeof(float)));
   const int I = c->par.ckpt_interval;
   c->n_ckpt = I > 0 ? (n_steps + I - 1) / I : 0;
@@ -790,6 +794,7 @@ rte_status rte_destroy(rte_ctx* c) {
   release(c->batch_jobs);
   release(c->err);
   release(c->ctl);
+  release(c->mseg);
   release(c->bal);
   release(c->bal_partial);
   release(c->bal_ticket);
@@ -1247,11 +1252,17 @@ static rte_status adjoint_impl(rte_ctx* c, const rte_detector* dets, int n_det, 
   float* moth = F(c->RA);
   int hl_adj = 0;
   std::vector<int> no_snaps(N, -1);
-  // Continuous form with multi-step launches: recompute, adjoint levels and
-  // gradient of a segment in turn on the context's stream, in one launch
-  // each.  The first segment buffer takes the forward levels, the second the
-  // adjoint's.
+  // Continuous form with multi-step launches, all on the context's stream.
+  // With few groups (tc_march_dual) the adjoint levels of a segment march
+  // beside the recompute of the next one, in launches of up to kDualSteps
+  // levels of both, each followed by its gradient terms; the adjoint levels
+  // of a launch take a buffer of their own.  With more groups, or without
+  // the memory for that buffer, recompute, adjoint and gradient of a segment
+  // follow one another, with the adjoint levels in the second segment buffer.
   const bool marched = !discrete && !fused_adj && !c->timing && rte_kern::tc_march_supported(sa);
+  const int chunk = std::min(I, kDualSteps);
+  const bool dual = marched && rte_kern::tc_march_dual(sa) &&
+                    ensure(c->mseg, static_cast<size_t>(chunk) * gbytes) == RTE_OK;
   // Levels needed: forward steps 0 .. N-2 (the adjoint vanishes at the last).
   const int last = N - 2;
   // Segments in reverse order.  The forward recompute of a segment (second
@@ -1270,9 +1281,18 @@ static rte_status adjoint_impl(rte_ctx* c, const rte_detector* dets, int n_det, 
   RTE_TRY(cuda_status(cudaStreamWaitEvent(c->astream, done_adj[0], 0)));
   auto seg_ptrs = [&](int k, int s0, int s_end) {
     std::vector<float*> segp(s_end - s0);
-    const size_t base = marched ? 0 : static_cast<size_t>(k % 2) * I * gfloats;
+    const size_t base = marched && !dual ? 0 : static_cast<size_t>(k % 2) * I * gfloats;
     for (int q = 0; q < s_end - s0; ++q) segp[q] = F(c->seg) + base + static_cast<size_t>(q) * gfloats;
     return segp;
+  };
+  // AB4 state of a checkpoint into U and L (history order from L[0])
+  auto restore = [&](int seg) -> rte_status {
+    const char* base = static_cast<const char*>(c->ckpt.p) + static_cast<size_t>(seg) * 4 * gbytes;
+    rte_status st = cuda_status(cudaMemcpyAsync(c->U.p, base, gbytes, cudaMemcpyDeviceToDevice, c->stream));
+    for (int q = 0; q < 3 && st == RTE_OK; ++q)
+      st = cuda_status(cudaMemcpyAsync(c->L[q].p, base + (q + 1) * gbytes, gbytes, cudaMemcpyDeviceToDevice,
+                                       c->stream));
+    return st;
   };
   auto recompute = [&](int k) -> rte_status {
     const int seg = segs[k];
@@ -1282,11 +1302,7 @@ static rte_status adjoint_impl(rte_ctx* c, const rte_detector* dets, int n_det, 
     const bool keep_timing = c->timing;
     c->timing = false;
     // Restore the AB4 state of the checkpoint and recompute the segment.
-    const char* base = static_cast<const char*>(c->ckpt.p) + static_cast<size_t>(seg) * 4 * gbytes;
-    rte_status st = cuda_status(cudaMemcpyAsync(c->U.p, base, gbytes, cudaMemcpyDeviceToDevice, c->stream));
-    for (int q = 0; q < 3 && st == RTE_OK; ++q)
-      st = cuda_status(cudaMemcpyAsync(c->L[q].p, base + (q + 1) * gbytes, gbytes, cudaMemcpyDeviceToDevice,
-                                       c->stream));
+    rte_status st = restore(seg);
     int hl = 0;
     std::vector<float*> segp = seg_ptrs(k, s0, s_end);
     if (st == RTE_OK) st = march(c, c->U, c->R, c->L, hl, G, s0, s_end, bf, false, no_snaps, nullptr, &segp);
@@ -1295,7 +1311,7 @@ static rte_status adjoint_impl(rte_ctx* c, const rte_detector* dets, int n_det, 
     c->timing = keep_timing;
     return st;
   };
-  if (!segs.empty() && !marched) RTE_TRY(recompute(0));
+  if (!segs.empty() && (!marched || dual)) RTE_TRY(recompute(0));
   // Discrete form: the transposed step with src_step N-1 on the zero state
   // gives v^{N-1} = c dt chi0 BC^T(readout^T r^{N-1}), the field that the
   // gradient of level N-1 takes.
@@ -1306,10 +1322,74 @@ static rte_status adjoint_impl(rte_ctx* c, const rte_detector* dets, int n_det, 
   for (size_t k = 0; k < segs.size(); ++k) {
     const int seg = segs[k];
     const int s0 = seg * I, s_end = std::min(s0 + I, last + 1);
+    if (dual) {
+      const bool more = k + 1 < segs.size();
+      const int t0 = more ? segs[k + 1] * I : 0, n = s_end - s0, n2 = more ? std::min(t0 + I, last + 1) - t0 : 0;
+      if (more) RTE_TRY(restore(segs[k + 1]));
+      float* fwd = F(c->seg) + static_cast<size_t>(k % 2) * I * gfloats;          // this segment's levels
+      float* nxt = F(c->seg) + static_cast<size_t>((k + 1) % 2) * I * gfloats;    // the next one's
+      const long long step = static_cast<long long>(gfloats);
+      int hl_fwd = 0;
+      for (int d = 0, d2 = 0; d < n || d2 < n2;) {
+        rte_kern::MarchArgs ma{};
+        ma.a = sa;
+        ma.ctl = static_cast<int*>(c->ctl.p);
+        // adjoint levels s_end - 1 - d .., recomputed levels t0 + d2 ..
+        rte_kern::MarchSide adj{}, rec{};
+        adj.b = ba;
+        adj.u0 = adj.u1 = mcur;
+        adj.slots = F(c->mseg);
+        adj.hl = hl_adj;
+        adj.step0 = s_end - 1 - d;
+        adj.dstep = -1;
+        rec.b = bf;
+        rec.slots = nxt + static_cast<size_t>(d2) * gfloats;
+        rec.u0 = rec.u1 = d2 == 0 ? F(c->U) : rec.slots - gfloats;
+        rec.hl = hl_fwd;
+        rec.step0 = t0 + d2;
+        rec.dstep = 1;
+        adj.slot_floats = rec.slot_floats = gfloats;
+        for (int q = 0; q < 3; ++q) {
+          adj.L[q] = F(c->LA[q]);
+          rec.L[q] = F(c->L[q]);
+        }
+        const bool has_adj = d < n, has_rec = d2 < n2;
+        ma.n_steps = std::min(has_adj ? std::min(chunk, n - d) : kMarchSteps, has_rec ? n2 - d2 : n);
+        ma.dual = has_adj && has_rec ? 1 : 0;
+        const rte_kern::MarchSide& one = has_adj ? adj : rec;
+        ma.b = one.b;
+        ma.u0 = one.u0;
+        ma.u1 = one.u1;
+        ma.slots = one.slots;
+        ma.slot_floats = gfloats;
+        for (int q = 0; q < 3; ++q) ma.L[q] = one.L[q];
+        ma.hl = one.hl;
+        ma.step0 = one.step0;
+        ma.dstep = one.dstep;
+        ma.two = rec;
+        RTE_TRY(cuda_status(rte_kern::launch_march_tc(ma, c->stream, &c->launches)));
+        const int m = ma.n_steps;
+        if (has_rec) {
+          hl_fwd = (hl_fwd + 2 * m) % 3;
+          d2 += m;
+        }
+        if (!has_adj) continue;
+        hl_adj = (hl_adj + 2 * m) % 3;
+        // slot l of the launch is level s_end - 1 - d - l
+        RTE_TRY(cuda_status(rte_kern::launch_grad(
+            adj.slots, fwd + static_cast<size_t>(n - 1 - d) * gfloats, F(c->PT), F(c->area), c->nx, c->ny, c->M, G,
+            c->plane, c->plane, scale, 1, {m, step, -step}, dJ_dmua ? D(c->grad_a) : nullptr,
+            dJ_dmus ? D(c->grad_b) : nullptr, c->stream, &c->launches)));
+        RTE_TRY(cuda_status(cudaMemcpyAsync(mcur, adj.slots + static_cast<size_t>(m - 1) * gfloats, gbytes,
+                                            cudaMemcpyDeviceToDevice, c->stream)));
+        d += m;
+      }
+      continue;
+    }
     if (marched) {
       const int n = s_end - s0;
       RTE_TRY(recompute(static_cast<int>(k)));
-      rte_kern::MarchArgs ma;
+      rte_kern::MarchArgs ma{};
       ma.a = sa;
       ma.b = ba;
       for (int q = 0; q < 3; ++q) ma.L[q] = F(c->LA[q]);

@@ -140,7 +140,16 @@ cudaError_t launch_step_tc_batched(const BatchProblem* probs, const BatchProblem
 // (slot_floats apart) and u0 holds the state before the first.  L[hl] is
 // L^{k-1} of the first step; the ring rotates by 2 (mod 3) per step.  Step k
 // takes the boundary data of step0 + k dstep.  ctl: tc_march_ctl_bytes(G)
-// bytes that no other launch in flight uses.
+// bytes (dual: 2 G) that no other launch in flight uses.
+struct MarchSide {                  // of a second march, as the fields of MarchArgs
+  BoundaryArgs b;
+  float* u0;
+  float* u1;
+  float* slots;
+  size_t slot_floats;
+  float* L[3];
+  int hl, step0, dstep;
+};
 struct MarchArgs {
   StepArgs a;
   BoundaryArgs b;
@@ -153,11 +162,17 @@ struct MarchArgs {
   int step0, dstep, n_steps;
   int rt, lag;                      // set by the launcher: 128-row output tiles per item, item order
   int* ctl;
+  // Two marches of the same medium at once (dual): the groups of a second one
+  // beside those of the first, on the same steps of the launch.
+  int dual;
+  MarchSide two;
   // batched form (launch_step_batch_march)
   const BatchProblem* probs;        // device
   int n_probs, xpass, items, flip;
 };
 bool tc_march_supported(const StepArgs& a);
+// Whether two marches of a.G groups are faster side by side than in turn.
+bool tc_march_dual(const StepArgs& a);
 size_t tc_march_ctl_bytes(int G);
 cudaError_t launch_march_tc(MarchArgs ma, cudaStream_t s, long long* launches);
 

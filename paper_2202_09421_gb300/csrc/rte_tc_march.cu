@@ -63,6 +63,9 @@ constexpr int kItemRing = 16;
 // groups: 278 us a step with 5, 280 with 3, 295 with 1).
 constexpr int kMarchLag = 5;
 
+// Forms of the kernel.
+enum { kSingle, kBatch, kDual };
+
 constexpr int kMaxM = 64;
 constexpr int kMaxD = 4;                                       // ring slots, at most
 // y-pass epilogue: per warp a ring of two pairs of rows of 5 arrays, per CTA
@@ -571,7 +574,7 @@ struct MarchShared {
   int abort_flag;
   float pcs[kMaxM];
   StepArgs pa;                       // batched form: of the epilogue's problem
-  BoundaryArgs pb;
+  BoundaryArgs pb, pb2;              // (dual: of the two marches)
 };
 
 // Bounded wait on an mbarrier; false when it, or any other wait of the CTA,
@@ -642,12 +645,15 @@ struct MarchRing {
   static constexpr int kStage = (ND + NS) * kUnit;            // 128 KB
 };
 
-// BATCH: one pass of one step of several media (launch_step_batch_march): the
+// DUAL: two marches of one medium, a.G counting the groups of both, which
+// alternate.  BATCH: one pass of one step of several media
+// (launch_step_batch_march): the
 // items are dealt out in order, no item waits for another, and the epilogue
 // warps take a problem's arguments and tables into shared memory when they
 // come to its first item.
-template <int PREC, int MM, bool BATCH>
+template <int PREC, int MM, int MODE>
 __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma) {
+  constexpr bool BATCH = MODE == kBatch, DUAL = MODE == kDual;
   using K = Kind<PREC>;
   constexpr bool X3 = K::X3, BF = K::BF;
   constexpr int KC = K::KC, GV = K::GV, M = MM;
@@ -660,7 +666,7 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
   // A launch after a timed-out one does nothing (the march reports the error;
   // BATCH: the items of the medium whose word is set).
   if (!BATCH && *static_cast<volatile int*>(a.err)) return;
-  const MarchItems it(a, ma.rt, ma.lag);
+  const MarchItems it(a, ma.rt, ma.lag);         // (DUAL: a.G is doubled by the launcher)
   const int total = BATCH ? ma.items : it.per_step() * ma.n_steps;
   auto item_of = [&](int t) {
     if constexpr (BATCH) return Item(ma.probs, ma.n_probs, ma.xpass != 0, ma.rt, KC, t);
@@ -696,6 +702,12 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
     sh.abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if constexpr (DUAL) {
+    if (tid == 0) {
+      sh.pb = ma.b;
+      sh.pb2 = ma.two.b;
+    }
+  }
   if constexpr (!BATCH) {
     for (int k = tid; k < M; k += kMarchThreads) sh.pcs[k] = __ldg(a.PT + k);
     BcTables(sm_epi, M).fill(ma.b, M, tid, kMarchThreads);
@@ -717,7 +729,16 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
   volatile int* abrt = &sh.abort_flag;
   int* xdone = ma.ctl + 32;                    // [G]
   int* ydone = xdone + it.G;
-  auto ubuf = [&](int k) {
+  // side and group of an item's group (DUAL)
+  auto side_of = [&](int gg) { return DUAL ? gg & 1 : 0; };
+  auto group_of = [&](int gg) { return DUAL ? gg >> 1 : gg; };
+  auto ubuf = [&](int gg, int k) {
+    if constexpr (DUAL) {
+      if (side_of(gg)) {
+        if (ma.two.slots) return k == 0 ? ma.two.u0 : ma.two.slots + static_cast<size_t>(k - 1) * ma.two.slot_floats;
+        return (k & 1) ? ma.two.u1 : ma.two.u0;
+      }
+    }
     if (ma.slots) return k == 0 ? ma.u0 : ma.slots + static_cast<size_t>(k - 1) * ma.slot_floats;
     return (k & 1) ? ma.u1 : ma.u0;
   };
@@ -850,11 +871,11 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
       const int line = im.tile * per_tile + c0 / M;
       const StepArgs& ca = args_of(im);
       if constexpr (BATCH) load_scales(ca);
-      const float* u_in = ubuf(im.s);
+      const float* u_in = ubuf(im.g, im.s);
       if constexpr (BATCH) u_in = ma.flip ? ma.probs[im.p].R : ma.probs[im.p].U;
       const bool col_ok = line < (im.xpass ? ca.ny : ca.nx);
       const size_t kstride = im.xpass ? M : static_cast<size_t>(ca.nx) * M;
-      const float* src = u_in + static_cast<size_t>(im.g) * ca.plane +
+      const float* src = u_in + static_cast<size_t>(group_of(im.g)) * ca.plane +
                          static_cast<size_t>(line) * (im.xpass ? static_cast<size_t>(ca.nx) * M : M) + m;
       float sc[4];
 #pragma unroll
@@ -936,6 +957,10 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
       if constexpr (BATCH) return sh.pb;
       else return ma.b;
     };
+    auto epi_side = [&](int side) -> const BoundaryArgs& {
+      if constexpr (DUAL) return side ? sh.pb2 : sh.pb;
+      else return epi_bargs();
+    };
     for (int k = 0;; ++k) {
       const int t = __shfl_sync(0xffffffffu, next_item(k), 0);
       if (!epi_all(t >= 0)) break;
@@ -958,10 +983,11 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
         }
       }
       const StepArgs& ea = epi_args();
-      const BoundaryArgs& eb = epi_bargs();
-      const size_t goff = static_cast<size_t>(im.g) * ea.plane;
-      const float* U = ubuf(im.s);
-      float* R = ubuf(im.s + 1);
+      const int side = side_of(im.g), lg = group_of(im.g);
+      const BoundaryArgs& eb = epi_side(side);
+      const size_t goff = static_cast<size_t>(lg) * ea.plane;
+      const float* U = ubuf(im.g, im.s);
+      float* R = ubuf(im.g, im.s + 1);
       if constexpr (BATCH) {
         const BatchProblem* P = ma.probs + im.p;
         U = ma.flip ? P->R : P->U;
@@ -969,9 +995,10 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
       }
       const uint32_t acc = tmem + b2 * acc_cols;
       const int t0 = im.tile * per_tile, row0 = im.rt0 * kMT;
-      const int hl = (ma.hl + 2 * im.s) % 3;
+      const int hl = ((DUAL && side ? ma.two.hl : ma.hl) + 2 * im.s) % 3;
       auto hist = [&](int q) {
         if constexpr (BATCH) return ma.probs[im.p].L[q];
+        else if constexpr (DUAL) return side ? ma.two.L[q] : ma.L[q];
         else return ma.L[q];
       };
       const float *L1 = hist(hl), *L2 = hist((hl + 1) % 3);
@@ -992,7 +1019,8 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
       } else if (im.xpass) {
         x_epilogue<MM>(ea, U, R, goff, t0, row0, im.nrt, sh.pcs, acc, sm_epi, warp, lane, released);
       } else {
-        y_epilogue<MM>(ea, eb, U, R, L1, L2, L3, goff, ma.step0 + im.s * ma.dstep, im.g, t0, row0, im.nrt, acc,
+        const int step = DUAL && side ? ma.two.step0 + im.s * ma.two.dstep : ma.step0 + im.s * ma.dstep;
+        y_epilogue<MM>(ea, eb, U, R, L1, L2, L3, goff, step, lg, t0, row0, im.nrt, acc,
                        sm_epi, warp, lane, [] { asm volatile("bar.sync 1, 256;" ::: "memory"); }, released);
       }
       if constexpr (!BATCH) {
@@ -1009,14 +1037,14 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols));
 }
 
-template <int PREC, int MM, bool BATCH>
+template <int PREC, int MM, int MODE>
 cudaError_t launch_march_t(const MarchArgs& ma, int sms, cudaStream_t s) {
   constexpr size_t smem = 1024 + MarchRing<Kind<PREC>::X3>::kStage + kEpiBytes;
   static const cudaError_t attr = cudaFuncSetAttribute(
-      tc_march_kernel<PREC, MM, BATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+      tc_march_kernel<PREC, MM, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (attr != cudaSuccess) return attr;
   const long long items =
-      BATCH ? ma.items : static_cast<long long>(MarchItems(ma.a, ma.rt, ma.lag).per_step()) * ma.n_steps;
+      MODE == kBatch ? ma.items : static_cast<long long>(MarchItems(ma.a, ma.rt, ma.lag).per_step()) * ma.n_steps;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(items < sms ? static_cast<unsigned>(items) : static_cast<unsigned>(sms));
   cfg.blockDim = dim3(kMarchThreads);
@@ -1026,26 +1054,26 @@ cudaError_t launch_march_t(const MarchArgs& ma, int sms, cudaStream_t s) {
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
-  cfg.numAttrs = BATCH ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, tc_march_kernel<PREC, MM, BATCH>, ma);
+  cfg.numAttrs = MODE == kBatch ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, tc_march_kernel<PREC, MM, MODE>, ma);
 }
 
-template <int PREC, bool BATCH>
+template <int PREC, int MODE>
 cudaError_t launch_march_m(const MarchArgs& ma, int sms, cudaStream_t s) {
   switch (ma.a.M) {
-    case 16: return launch_march_t<PREC, 16, BATCH>(ma, sms, s);
-    case 32: return launch_march_t<PREC, 32, BATCH>(ma, sms, s);
-    default: return launch_march_t<PREC, 64, BATCH>(ma, sms, s);
+    case 16: return launch_march_t<PREC, 16, MODE>(ma, sms, s);
+    case 32: return launch_march_t<PREC, 32, MODE>(ma, sms, s);
+    default: return launch_march_t<PREC, 64, MODE>(ma, sms, s);
   }
 }
 
-template <bool BATCH>
+template <int MODE>
 cudaError_t launch_march_p(const MarchArgs& ma, int sms, cudaStream_t s) {
   switch (ma.a.tc_mode) {
-    case 1: return launch_march_m<1, BATCH>(ma, sms, s);
-    case 2: return launch_march_m<2, BATCH>(ma, sms, s);
-    case 3: return launch_march_m<3, BATCH>(ma, sms, s);
-    default: return launch_march_m<4, BATCH>(ma, sms, s);
+    case 1: return launch_march_m<1, MODE>(ma, sms, s);
+    case 2: return launch_march_m<2, MODE>(ma, sms, s);
+    case 3: return launch_march_m<3, MODE>(ma, sms, s);
+    default: return launch_march_m<4, MODE>(ma, sms, s);
   }
 }
 
@@ -1071,10 +1099,21 @@ bool tc_march_supported(const StepArgs& a) {
   return rows && a.tc_mode != 0 && a.tc_scatter == 0 && a.x_variant == 1 && !a.test_expire;
 }
 
+bool tc_march_dual(const StepArgs& a) {
+  // Where one march leaves SMs without an item now and then, fewer than two
+  // items of a pass for each.  256^2, M = 32, a gradient's step (forward,
+  // recompute and adjoint) side by side against in turn: one group 125 us
+  // against 134, two 188 against 208, four 302 against 316, eight 472 against
+  // 448, sixteen 925 against 878 (twice the state between two uses in L2).
+  const MarchItems it(a, 2, 0);
+  return a.G * static_cast<long long>(it.nxi > it.nyi ? it.nxi : it.nyi) < 2 * sm_count();
+}
+
 size_t tc_march_ctl_bytes(int G) { return (32 + 2 * static_cast<size_t>(G)) * sizeof(int); }
 
 cudaError_t launch_march_tc(MarchArgs ma, cudaStream_t s, long long* launches) {
   const int sms = sm_count();
+  if (ma.dual) ma.a.G *= 2;
   // Row tiles per item: two output tiles share a conversion of the slab, one
   // makes twice the items.  One where a pass has no more items than SMs that
   // way (256^2, M = 32, 3xTF32: one group 46 us a step against 60; four
@@ -1085,7 +1124,7 @@ cudaError_t launch_march_tc(MarchArgs ma, cudaStream_t s, long long* launches) {
   if (ma.a.G * static_cast<long long>(one.nxi > one.nyi ? one.nxi : one.nyi) > sms) ma.rt = 2;
   cudaError_t e = cudaMemsetAsync(ma.ctl, 0, tc_march_ctl_bytes(ma.a.G), s);
   if (e != cudaSuccess) return e;
-  e = launch_march_p<false>(ma, sms, s);
+  e = ma.dual ? launch_march_p<kDual>(ma, sms, s) : launch_march_p<kSingle>(ma, sms, s);
   if (launches) *launches += 1;
   return e;
 }
@@ -1126,11 +1165,11 @@ cudaError_t launch_step_batch_march(const BatchProblem* probs, const BatchProble
   const MarchItems it(last.a, 2, 0);
   ma.xpass = 1;
   ma.items = last.item0_x + last.a.G * it.nxi;
-  cudaError_t e = launch_march_p<true>(ma, sm_count(), s);
+  cudaError_t e = launch_march_p<kBatch>(ma, sm_count(), s);
   if (e != cudaSuccess) return e;
   ma.xpass = 0;
   ma.items = last.item0_y + last.a.G * it.nyi;
-  e = launch_march_p<true>(ma, sm_count(), s);
+  e = launch_march_p<kBatch>(ma, sm_count(), s);
   if (launches) *launches += 2;
   return e;
 }

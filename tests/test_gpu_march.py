@@ -15,11 +15,12 @@ TF32X3, TF32, BF16X3, BF16 = 1, 2, 3, 4
 
 # sizes: one and two row tiles, ragged ends, a short other axis (items of a
 # single unit), two lines per tile (M = 64), more items than SMs; odd and even
-# step counts; snapshots and checkpoints that cut the march into runs
+# step counts; snapshots and checkpoints that cut the march into runs; segments
+# longer than one launch of the reverse sweep
 @pytest.mark.parametrize("nx,ny,M,groups,steps,prec", [
     (129, 129, 32, 1, 7, TF32X3), (256, 256, 32, 7, 9, TF32X3), (203, 131, 16, 2, 12, TF32),
     (256, 24, 32, 3, 11, BF16X3), (24, 256, 16, 40, 6, TF32X3), (140, 300, 64, 2, 5, BF16X3),
-    (300, 40, 64, 1, 8, BF16)])
+    (300, 40, 64, 1, 8, BF16), (136, 24, 16, 1, 90, TF32X3)])
 def test_multi_step_launch_matches_two_launches_per_step(nx, ny, M, groups, steps, prec):
     from paper_2202_09421_gb300 import binding as B
     from paper_2202_09421_gb300.solver import FCDOMSolver
@@ -30,7 +31,7 @@ def test_multi_step_launch_matches_two_launches_per_step(nx, ny, M, groups, step
     for two_launches in (False, True):
         s = FCDOMSolver(wl.grid, wl.optics, torch.tensor(wl.mua, dtype=torch.float32, device=dev),
                         torch.tensor(wl.mus, dtype=torch.float32, device=dev), wl.c, wl.dt, precision=prec,
-                        ckpt_interval=4)
+                        ckpt_interval=4 if steps < 40 else 40)
         B.rte_set_pass_variant(s.ctx, 1)
         if two_launches:
             B.rte_set_kernel_timing(s.ctx, True)
