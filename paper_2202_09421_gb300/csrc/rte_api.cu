@@ -53,7 +53,7 @@ struct rte_ctx {
   bool inject_expire = false;
   // item counters of the multi-step launches
   DevBuf ctl;
-  DevBuf mseg;                       // adjoint levels of one launch (kDualSteps at most)
+  DevBuf mseg;                       // states of one launch: adjoint levels, or steps with the photon balance
   // photon balance of the last rte_forward (RTE_FLAG_PHOTON_BALANCE):
   // [G][n_steps][3] FP64 terms, block partials, per-group tickets, and the
   // FP64 cos / sin of the ordinates
@@ -283,6 +283,9 @@ rte_status snapshot(rte_ctx* c, const float* u, int G, const std::vector<int>& s
 // Steps of a multi-step launch, at most: 36 ms at 16 groups of 256^2, so that
 // work on other streams gets its turn (a launch costs about 0.1 ms of ramp).
 constexpr int kMarchSteps = 128;
+// The same with the photon balance of every step (16 groups of 256^2: 0.1 ms
+// of ramp over four steps; the buffer holds twice as many states).
+constexpr int kBalanceSteps = 4;
 // The same for the adjoint beside a recompute: the adjoint levels of a launch
 // are kept for its gradient terms.
 constexpr int kDualSteps = 32;
@@ -308,8 +311,19 @@ rte_status march(rte_ctx* c, DevBuf& U, DevBuf& R, DevBuf* L, int& hl, int G, in
   // recompute stream: a launch that keeps every SM for a whole segment leaves
   // nothing to overlap with the passes of the other stream.
   const bool overlapped = c->astream && c->stream == c->astream;
-  if (!fused && !balance_out && !c->timing && !overlapped && rte_kern::tc_march_supported(a)) {
-    if (!seg_out && ((s_end - s_begin) & 1)) {
+  // The photon balance takes the state of every step: runs of kBalanceSteps
+  // into slots, one half of the buffer after the other (a run starts from the
+  // last slot of the run before); without the buffer, single passes.
+  const bool marched = !fused && !c->timing && !overlapped && rte_kern::tc_march_supported(a) &&
+                       (!balance_out || c->mseg.bytes >= 2 * kBalanceSteps * gbytes);
+  auto balance = [&](const float* u, int step) {
+    return cuda_status(rte_kern::launch_balance(
+        u, c->plane, c->nx, c->ny, c->M, G, F(c->mua), D(c->trig), c->dx, c->dy, 2.0 * kPi / c->M, c->opt.c,
+        D(c->bal_partial), static_cast<unsigned*>(c->bal_ticket.p), balance_out, step, c->n_steps, c->stream,
+        &c->launches));
+  };
+  if (marched) {
+    if (!seg_out && !balance_out && ((s_end - s_begin) & 1)) {
       RTE_TRY(cuda_status(cudaMemcpyAsync(oth, cur, gbytes, cudaMemcpyDeviceToDevice, c->stream)));
       std::swap(cur, oth);
     }
@@ -321,10 +335,12 @@ rte_status march(rte_ctx* c, DevBuf& U, DevBuf& R, DevBuf* L, int& hl, int G, in
     ma.dstep = 1;
     ma.ctl = static_cast<int*>(c->ctl.p);
     for (int q = 0; q < 3; ++q) ma.L[q] = F(L[q]);
-    for (int s = s_begin; s < s_end;) {
+    const size_t gfloats = static_cast<size_t>(G) * c->plane;
+    const int longest = balance_out ? kBalanceSteps : kMarchSteps;
+    for (int s = s_begin, run = 0; s < s_end; ++run) {
       if (save_ckpt && I > 0 && s % I == 0) RTE_TRY(copy_checkpoint(c, cur, L, hl, G, s));
       int e = s + 1;                                   // the run [s, e)
-      while (e < s_end && e - s < kMarchSteps && !(save_ckpt && I > 0 && e % I == 0) && !(fluence_out && snap_index[e - 1] >= 0)) ++e;
+      while (e < s_end && e - s < longest && !(save_ckpt && I > 0 && e % I == 0) && !(fluence_out && snap_index[e - 1] >= 0)) ++e;
       ma.u0 = cur;
       ma.u1 = oth;
       ma.hl = hl;
@@ -332,16 +348,25 @@ rte_status march(rte_ctx* c, DevBuf& U, DevBuf& R, DevBuf* L, int& hl, int G, in
       ma.n_steps = e - s;
       if (seg_out) {
         ma.slots = (*seg_out)[s - s_begin];
-        ma.slot_floats = static_cast<size_t>(G) * c->plane;
+        ma.slot_floats = gfloats;
+      }
+      if (balance_out) {
+        ma.slots = F(c->mseg) + static_cast<size_t>(run % 2) * kBalanceSteps * gfloats;
+        ma.slot_floats = gfloats;
       }
       RTE_TRY(cuda_status(rte_kern::launch_march_tc(ma, c->stream, &c->launches)));
       hl = (hl + 2 * (e - s)) % 3;
+      if (balance_out)
+        for (int q = s; q < e; ++q) RTE_TRY(balance(ma.slots + static_cast<size_t>(q - s) * gfloats, q));
       if (seg_out) cur = (*seg_out)[e - 1 - s_begin];
+      else if (balance_out) cur = ma.slots + static_cast<size_t>(e - 1 - s) * gfloats;
       else if ((e - s) & 1) std::swap(cur, oth);
       if (fluence_out && snap_index[e - 1] >= 0)
         RTE_TRY(snapshot(c, cur, G, snap_index, e - 1, fluence_out));
       s = e;
     }
+    if (balance_out)
+      RTE_TRY(cuda_status(cudaMemcpyAsync(U.p, cur, gbytes, cudaMemcpyDeviceToDevice, c->stream)));
     return RTE_OK;
   }
   for (int s = s_begin; s < s_end; ++s) {
@@ -372,11 +397,7 @@ rte_status march(rte_ctx* c, DevBuf& U, DevBuf& R, DevBuf* L, int& hl, int G, in
     if (seg_out)
       RTE_TRY(cuda_status(cudaMemcpyAsync((*seg_out)[s - s_begin], cur, gbytes,
                                           cudaMemcpyDeviceToDevice, c->stream)));
-    if (balance_out)
-      RTE_TRY(cuda_status(rte_kern::launch_balance(
-          cur, c->plane, c->nx, c->ny, c->M, G, F(c->mua), D(c->trig), c->dx, c->dy, 2.0 * kPi / c->M,
-          c->opt.c, D(c->bal_partial), static_cast<unsigned*>(c->bal_ticket.p), balance_out, s, c->n_steps,
-          c->stream, &c->launches)));
+    if (balance_out) RTE_TRY(balance(cur, s));
   }
   if (cur != F(U))
     RTE_TRY(cuda_status(cudaMemcpyAsync(U.p, cur, gbytes, cudaMemcpyDeviceToDevice, c->stream)));
@@ -587,7 +608,7 @@ unsigned long long key_ptr(const void* p) { return static_cast<unsigned long lon
 // Key of the buffers a forward march of context c touches.
 void append_forward_key(const rte_ctx* c, std::vector<unsigned long long>& key) {
   const void* ptrs[] = {c->U.p, c->R.p, c->L[0].p, c->L[1].p, c->L[2].p, c->ring.p, c->S.p, c->A.p,
-                        c->T.p, c->ckpt.p, c->mua.p, c->mus.p, c->ctl.p};
+                        c->T.p, c->ckpt.p, c->mua.p, c->mus.p, c->ctl.p, c->mseg.p};
   key.push_back(static_cast<unsigned long long>(c->n_steps));
   key.push_back(static_cast<unsigned long long>(c->G));
   key.push_back(static_cast<unsigned long long>(c->kmax));
@@ -994,6 +1015,9 @@ rte_status rte_forward(rte_ctx* c, const rte_source_group* groups, int n_groups,
     RTE_TRY(ensure(c->bal_ticket, static_cast<size_t>(G) * sizeof(unsigned)));
     RTE_TRY(cuda_status(cudaMemsetAsync(c->bal_ticket.p, 0, static_cast<size_t>(G) * sizeof(unsigned), c->stream)));
     balance = D(c->bal);
+    // states for the multi-step launches (single passes without the memory)
+    if (rte_kern::tc_march_supported(step_args(c, G)))
+      ensure(c->mseg, 2 * kBalanceSteps * static_cast<size_t>(G) * c->plane * sizeof(float));
   }
   const rte_kern::BoundaryArgs b = forward_bargs(c);
   std::vector<unsigned long long> key;

@@ -53,6 +53,33 @@ def test_multi_step_launch_matches_two_launches_per_step(nx, ny, M, groups, step
         assert np.linalg.norm(a[k] - b[k]) <= 1e-7 * np.linalg.norm(b[k])
 
 
+@pytest.mark.parametrize("steps,ckpt", [(13, 0), (9, 1), (10, 3)])
+def test_photon_balance_of_a_multi_step_launch(steps, ckpt):
+    """The balance of every step, from states in slots, against single passes;
+    runs of one step (a checkpoint at each) and of four."""
+    from paper_2202_09421_gb300 import binding as B
+    from paper_2202_09421_gb300.solver import FCDOMSolver
+    wl = workload_custom(150, 40, 32, steps, 0.02, L=149 / 66, mus=80.0, n_groups=2, t_s=0.1, sigma_t=0.1)
+    dev = torch.device("cuda:0")
+    out = []
+    for two_launches in (False, True):
+        s = FCDOMSolver(wl.grid, wl.optics, torch.tensor(wl.mua, dtype=torch.float32, device=dev),
+                        torch.tensor(wl.mus, dtype=torch.float32, device=dev), wl.c, wl.dt, precision=TF32X3,
+                        ckpt_interval=ckpt, flags=B.RTE_FLAG_PHOTON_BALANCE)
+        B.rte_set_pass_variant(s.ctx, 1)
+        if two_launches:
+            B.rte_set_kernel_timing(s.ctx, True)
+        before = B.rte_kernel_launches(s.ctx)
+        s.forward(wl.groups, steps)
+        launches = B.rte_kernel_launches(s.ctx) - before
+        out.append((s.photon_balance().cpu().numpy(), s.state(1).cpu().numpy(), s.readout(wl.detectors).cpu().numpy(),
+                    launches))
+        s.close()
+    a, b = out
+    assert a[3] < b[3] and np.abs(a[0]).max() > 0
+    assert all(np.array_equal(x, y) for x, y in zip(a[:3], b[:3]))
+
+
 @pytest.mark.parametrize("M,prec,steps,sizes", [
     (32, TF32X3, 7, [(200, 140, 2), (48, 64, 1), (129, 40, 3), (300, 260, 1)]),
     (16, BF16X3, 6, [(24, 260, 1), (257, 129, 2)]), (64, TF32, 5, [(140, 36, 1), (40, 300, 2)])])
