@@ -114,12 +114,8 @@ __global__ void __launch_bounds__(kFT, 2)
   extern __shared__ __align__(1024) unsigned char smraw[];
   __shared__ __align__(8) uint64_t bars[3];          // operator images, hi slot, lo slot
   __shared__ uint32_t tmem_slot;
-  __shared__ int skip;
-  // A launch after a timed-out one does nothing (one read, so that the whole
-  // CTA takes the same branch).
-  if (threadIdx.x == 0) skip = *static_cast<volatile int*>(a.err);
-  __syncthreads();
-  if (skip) return;
+  // A launch after a timed-out one does nothing.
+  if (cta_timed_out(a.err)) return;
 
   unsigned char* sm = smraw + ((1024 - (smem_u32(smraw) & 1023)) & 1023);
   float* box = reinterpret_cast<float*>(sm + kBoxOff);

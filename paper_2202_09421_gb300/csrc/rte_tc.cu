@@ -96,8 +96,14 @@ __device__ __forceinline__ void tc_pass_body(const StepArgs& a, const BoundaryAr
   const float* scale = XPASS ? a.xi : a.eta;
   const int n_lines = XPASS ? ny : nx;        // rows (x) / columns (y) of the grid
 
-  // A launch after a timed-out one does nothing (the march reports the error).
-  if (*static_cast<volatile int*>(a.err)) return;
+  // A launch after a timed-out one does nothing (the march reports the error),
+  // but ends only after the launch that it depends on: a CTA of that one may
+  // still be in a bounded wait, and the march reads and clears the word when
+  // the last launch has ended.
+  if (cta_timed_out(a.err)) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    return;
+  }
   unsigned char* sm = smraw + ((1024 - (smem_u32(smraw) & 1023)) & 1023);
   unsigned char* Psm = sm + L.stage_bytes;    // P~ image (x-pass, TC scattering)
   const uint32_t bar_full = smem_u32(&bars[0]), bar_done = smem_u32(&bars[1]);
@@ -130,6 +136,7 @@ __device__ __forceinline__ void tc_pass_body(const StepArgs& a, const BoundaryAr
     if (gave_up) {
       if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(L.tmem_cols));
+      asm volatile("griddepcontrol.wait;" ::: "memory");
       return;
     }
   }

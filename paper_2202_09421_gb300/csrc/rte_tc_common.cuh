@@ -23,6 +23,15 @@ __device__ __forceinline__ unsigned long long global_ns() {
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
 }
+// Whether the context's timeout word is set, the same answer in every thread
+// of the CTA: one thread reads it.  (Read by every thread, the word could
+// change between two warps' reads; the warps that stayed would then wait at
+// the kernels' counted barriers for the ones that left.)  Every thread calls
+// it, before anything else.
+__device__ __forceinline__ bool cta_timed_out(const int* err) {
+  return __syncthreads_or(threadIdx.x == 0 ? *static_cast<const volatile int*>(err) : 0) != 0;
+}
+
 constexpr float kAB0 = 55.0f / 24.0f, kAB1 = -59.0f / 24.0f, kAB2 = 37.0f / 24.0f,
                 kAB3 = -9.0f / 24.0f;
 

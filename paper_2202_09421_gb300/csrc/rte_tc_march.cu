@@ -665,7 +665,7 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
   const StepArgs& a = ma.a;
   // A launch after a timed-out one does nothing (the march reports the error;
   // BATCH: the items of the medium whose word is set).
-  if (!BATCH && *static_cast<volatile int*>(a.err)) return;
+  if (!BATCH && cta_timed_out(a.err)) return;
   const MarchItems it(a, ma.rt, ma.lag);         // (DUAL: a.G is doubled by the launcher)
   const int total = BATCH ? ma.items : it.per_step() * ma.n_steps;
   auto item_of = [&](int t) {

@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1)
   const int tiles_per_group = (nx + per_tile - 1) / per_tile;
   const int total = tiles_per_group * a.G;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (*static_cast<volatile int*>(a.err)) return;
+  if (cta_timed_out(a.err)) return;
   const int acc_cols = L.nrows_img;
   unsigned char* sm = smraw + ((1024 - (smem_u32(smraw) & 1023)) & 1023);
   float* epi = reinterpret_cast<float*>(sm + L.stage_bytes);

@@ -109,7 +109,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
   const int total = tiles_per_group * a.G;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // A launch after a timed-out one does nothing (the march reports the error).
-  if (*static_cast<volatile int*>(a.err)) return;
+  if (cta_timed_out(a.err)) return;
   const int acc_cols = L.nrows_img;                    // one accumulator buffer (n_mt * 128)
   unsigned char* sm = smraw + ((1024 - (smem_u32(smraw) & 1023)) & 1023);
   auto bar = [&](int k) { return smem_u32(&bars[k]); };
