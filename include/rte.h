@@ -399,8 +399,7 @@ long long rte_graph_captures(const rte_ctx* ctx);
  * Schedules 4 and 5 give the one-tile-per-CTA passes' results bit for bit.
  * rte_discrete_adjoint_gradient, rte_forward_batch and
  * rte_adjoint_gradient_batch run the one-tile-per-CTA passes under every
- * schedule (rte_forward_batch, with a line of more than 128 positions among
- * the media, their tiles as items of one persistent launch per pass).
+ * schedule.
  * Unsupported sizes run the one-tile-per-CTA passes (the plain FP32 passes
  * in RTE_PREC_FP32).  Errors: INVALID_ARG. */
 rte_status rte_set_pass_variant(rte_ctx* ctx, int variant);

@@ -549,10 +549,10 @@ rte_kern::BoundaryArgs forward_bargs(rte_ctx* c) {
 }
 
 // Checkpoint of the march state before step s (every ckpt_interval steps).
-rte_status save_checkpoint(rte_ctx* c, int s, int hl, bool in_r) {
+rte_status save_checkpoint(rte_ctx* c, int s, int hl) {
   const int I = c->par.ckpt_interval;
   if (I <= 0 || s % I != 0) return RTE_OK;
-  return copy_checkpoint(c, F(in_r ? c->R : c->U), c->L, hl, c->G, s);
+  return copy_checkpoint(c, F(c->U), c->L, hl, c->G, s);
 }
 
 // Runs `enqueue` (which puts the whole march on c->stream) directly, or, in
@@ -1095,7 +1095,6 @@ rte_status rte_forward_batch(rte_ctx* const* ctxs, int n_ctx, const rte_source_g
     }
     int ctas_x = 0, ctas_y = 0;
     rte_kern::tc_batch_layout(tab.data(), n_ctx, &ctas_x, &ctas_y);
-    const bool persistent = rte_kern::launch_step_batch_march_layout(tab.data(), n_ctx);
     RTE_TRY(upload(c0->batch_tab, tab, c0->stream));
     // the table must reach the device before the host vector goes away
     RTE_TRY(cuda_status(cudaStreamSynchronize(c0->stream)));
@@ -1103,30 +1102,17 @@ rte_status rte_forward_batch(rte_ctx* const* ctxs, int n_ctx, const rte_source_g
     const auto* dev = static_cast<const rte_kern::BatchProblem*>(c0->batch_tab.p);
     RTE_TRY(run_march(c0, key, [&]() {
       int hl = 0;
-      // The persistent form alternates between U and R and ends in U (an odd
-      // number of steps starts from the zero state in R).
-      bool flip = persistent && (n_steps & 1);
-      if (flip)
-        for (int i = 0; i < n_ctx; ++i)
-          RTE_TRY(cuda_status(cudaMemsetAsync(
-              ctxs[i]->R.p, 0, static_cast<size_t>(ctxs[i]->G) * ctxs[i]->plane * sizeof(float), c0->stream)));
       for (int s = 0; s < n_steps; ++s) {
         for (int i = 0; i < n_ctx; ++i) {
           rte_ctx* c = ctxs[i];
           const cudaStream_t keep = c->stream;
           c->stream = c0->stream;
-          const rte_status st = save_checkpoint(c, s, hl, flip);
+          const rte_status st = save_checkpoint(c, s, hl);
           c->stream = keep;
           if (st != RTE_OK) return st;
         }
-        if (persistent) {
-          RTE_TRY(cuda_status(rte_kern::launch_step_batch_march(tab.data(), dev, n_ctx, s, hl, flip, c0->stream,
-                                                                &c0->launches)));
-          flip = !flip;
-        } else {
-          RTE_TRY(cuda_status(rte_kern::launch_step_tc_batched(tab.data(), dev, n_ctx, s, hl, c0->stream,
-                                                                &c0->launches)));
-        }
+        RTE_TRY(cuda_status(rte_kern::launch_step_tc_batched(tab.data(), dev, n_ctx, s, hl, c0->stream,
+                                                              &c0->launches)));
         hl = (hl + 2) % 3;
       }
       return RTE_OK;

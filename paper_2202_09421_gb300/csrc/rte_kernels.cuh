@@ -116,7 +116,6 @@ struct BatchProblem {
   float* R;
   float* L[3];
   int tile0_x, tiles_x, tile0_y, tiles_y;
-  int item0_x, item0_y;             // of launch_step_batch_march
 };
 
 // tcgen05 form of launch_step (a.tc_mode != 0); see rte_tc.cu.
@@ -166,23 +165,12 @@ struct MarchArgs {
   // beside those of the first, on the same steps of the launch.
   int dual;
   MarchSide two;
-  // batched form (launch_step_batch_march)
-  const BatchProblem* probs;        // device
-  int n_probs, xpass, items, flip;
 };
 bool tc_march_supported(const StepArgs& a);
 // Whether two marches of a.G groups are faster side by side than in turn.
 bool tc_march_dual(const StepArgs& a);
 size_t tc_march_ctl_bytes(int G);
 cudaError_t launch_march_tc(MarchArgs ma, cudaStream_t s, long long* launches);
-
-// launch_step_tc_batched with the tiles of every medium as items of one
-// persistent x-pass and one y-pass launch.  The step goes from U to R (flip:
-// from R to U).  launch_step_batch_march_layout sets the item ranges of the
-// table (host) and says whether the media take this form.
-bool launch_step_batch_march_layout(BatchProblem* probs, int n);
-cudaError_t launch_step_batch_march(const BatchProblem* probs, const BatchProblem* probs_dev, int n, int step,
-                                    int hl, bool flip, cudaStream_t s, long long* launches);
 
 // Persistent warp-specialised passes (rte_tc_ws.cu): nx, ny <= 256, M in
 // {16, 32}, without the tensor-core scattering flag.

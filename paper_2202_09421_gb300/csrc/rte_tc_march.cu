@@ -63,9 +63,6 @@ constexpr int kItemRing = 16;
 // groups: 278 us a step with 5, 280 with 3, 295 with 1).
 constexpr int kMarchLag = 5;
 
-// Forms of the kernel.
-enum { kSingle, kBatch, kDual };
-
 constexpr int kMaxM = 64;
 constexpr int kMaxD = 4;                                       // ring slots, at most
 // y-pass epilogue: per warp a ring of two pairs of rows of 5 arrays, per CTA
@@ -508,7 +505,6 @@ struct MarchItems {
 struct Item {
   bool xpass;
   int s, g, tile, rt0, nrt, n, n_kc;
-  int p;                             // batched form: the problem
   // step order: x(0), .., x(lag - 1); x(lag), y(0); ..; x(G - 1), y(G - 1 -
   // lag); y(G - lag), .., y(G - 1)
   __device__ __forceinline__ Item(const MarchItems& it, const StepArgs& a, int kc, int ticket) {
@@ -533,27 +529,7 @@ struct Item {
       idx = r - g * it.nyi;
       g += it.G - it.lag;
     }
-    p = 0;
-    place(it, a, kc, idx);
-  }
-  // batched form: item t of one pass over the problems, in table order
-  __device__ __forceinline__ Item(const BatchProblem* probs, int n_probs, bool x, int rt, int kc, int t) {
-    xpass = x;
-    s = 0;
-    int lo = 0, hi = n_probs - 1;                  // the last problem that starts at or before t
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) / 2;
-      if ((x ? probs[mid].item0_x : probs[mid].item0_y) <= t) lo = mid;
-      else hi = mid - 1;
-    }
-    p = lo;
-    const BatchProblem& P = probs[p];
-    const MarchItems it(P.a, rt, 0);
-    const int r = t - (x ? P.item0_x : P.item0_y), per_g = x ? it.nxi : it.nyi;
-    g = r / per_g;
-    place(it, P.a, kc, r - g * per_g);
-  }
-  __device__ __forceinline__ void place(const MarchItems& it, const StepArgs& a, int kc, int idx) {
+
     const int parts = xpass ? it.px : it.py;
     tile = idx / parts;
     rt0 = (idx - tile * parts) * it.rt;
@@ -573,8 +549,7 @@ struct MarchShared {
   uint32_t tmem_slot;
   int abort_flag;
   float pcs[kMaxM];
-  StepArgs pa;                       // batched form: of the epilogue's problem
-  BoundaryArgs pb, pb2;              // (dual: of the two marches)
+  BoundaryArgs pb, pb2;              // DUAL: of the two marches
 };
 
 // Bounded wait on an mbarrier; false when it, or any other wait of the CTA,
@@ -646,14 +621,9 @@ struct MarchRing {
 };
 
 // DUAL: two marches of one medium, a.G counting the groups of both, which
-// alternate.  BATCH: one pass of one step of several media
-// (launch_step_batch_march): the
-// items are dealt out in order, no item waits for another, and the epilogue
-// warps take a problem's arguments and tables into shared memory when they
-// come to its first item.
-template <int PREC, int MM, int MODE>
+// alternate.
+template <int PREC, int MM, bool DUAL>
 __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma) {
-  constexpr bool BATCH = MODE == kBatch, DUAL = MODE == kDual;
   using K = Kind<PREC>;
   constexpr bool X3 = K::X3, BF = K::BF;
   constexpr int KC = K::KC, GV = K::GV, M = MM;
@@ -663,19 +633,10 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
   extern __shared__ __align__(1024) unsigned char smraw[];
   __shared__ __align__(8) MarchShared sh;
   const StepArgs& a = ma.a;
-  // A launch after a timed-out one does nothing (the march reports the error;
-  // BATCH: the items of the medium whose word is set).
-  if (!BATCH && cta_timed_out(a.err)) return;
+  // A launch after a timed-out one does nothing (the march reports the error).
+  if (cta_timed_out(a.err)) return;
   const MarchItems it(a, ma.rt, ma.lag);         // (DUAL: a.G is doubled by the launcher)
-  const int total = BATCH ? ma.items : it.per_step() * ma.n_steps;
-  auto item_of = [&](int t) {
-    if constexpr (BATCH) return Item(ma.probs, ma.n_probs, ma.xpass != 0, ma.rt, KC, t);
-    else return Item(it, a, KC, t);
-  };
-  auto args_of = [&](const Item& im) -> const StepArgs& {
-    if constexpr (BATCH) return ma.probs[im.p].a;
-    else return a;
-  };
+  const int total = it.per_step() * ma.n_steps;
   const int acc_cols = it.rt * kMT, tmem_cols = 2 * acc_cols;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   unsigned char* sm = smraw + ((1024 - (smem_u32(smraw) & 1023)) & 1023);
@@ -708,10 +669,8 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
       sh.pb2 = ma.two.b;
     }
   }
-  if constexpr (!BATCH) {
-    for (int k = tid; k < M; k += kMarchThreads) sh.pcs[k] = __ldg(a.PT + k);
-    BcTables(sm_epi, M).fill(ma.b, M, tid, kMarchThreads);
-  }
+  for (int k = tid; k < M; k += kMarchThreads) sh.pcs[k] = __ldg(a.PT + k);
+  BcTables(sm_epi, M).fill(ma.b, M, tid, kMarchThreads);
   if (warp == kWarpCopy) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem_slot)),
                  "r"(tmem_cols));
@@ -721,11 +680,6 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = sh.tmem_slot;
-  // dependent launches: each pass waits here, set up, for the one before
-  if constexpr (BATCH) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  }
   volatile int* abrt = &sh.abort_flag;
   int* xdone = ma.ctl + 32;                    // [G]
   int* ydone = xdone + it.G;
@@ -755,12 +709,12 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
       int n = 0;
       bool fine = true;
       for (int k = 0; fine; ++k) {
-        const int t = BATCH ? static_cast<int>(blockIdx.x + k * gridDim.x) : atomicAdd(ma.ctl, 1);
+        const int t = atomicAdd(ma.ctl, 1);
         sh.item[k % kItemRing] = t < total ? t : -1;
         m_arrive(&sh.item_full[k % kItemRing]);
         if (t >= total) break;
-        const Item im = item_of(t);
-        const unsigned char* Dimg = static_cast<const unsigned char*>(im.xpass ? args_of(im).DxImg : args_of(im).DyImg);
+        const Item im = Item(it, a, KC, t);
+        const unsigned char* Dimg = static_cast<const unsigned char*>(im.xpass ? a.DxImg : a.DyImg);
         const size_t lo_off = static_cast<size_t>((im.n + kMT - 1) / kMT) * kTileBytes;   // lo rows of a chunk
         for (int q = 0; q < im.n_kc && fine; ++q)
           for (int u = 0; u < im.nrt; ++u, ++n) {
@@ -789,7 +743,7 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
       for (int k = 0; fine; ++k) {
         const int t = next_item(k);
         if (t < 0) break;
-        const Item im = item_of(t);
+        const Item im = Item(it, a, KC, t);
         const int b2 = k & 1;
         if (!m_wait(&sh.acc_empty[b2], ((k >> 1) & 1) ^ 1, abrt, a.err)) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -827,11 +781,11 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
     // ---------------- completion counts ----------------
     // (two barriers in turn; the epilogue waits for the count of item k - 2
     // before it arrives for item k, see there)
-    if (!BATCH && lane == 0)
+    if (lane == 0)
       for (int k = 0;; ++k) {
         const int t = next_item(k);
         if (t < 0) break;
-        const Item im = item_of(t);
+        const Item im = Item(it, a, KC, t);
         if (!m_wait(&sh.epi_done[k & 1], (k >> 1) & 1, abrt, a.err)) break;
         m_arrive(&sh.sig_done[k & 1]);
         __threadfence();
@@ -850,14 +804,11 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
     const int c0 = (ct >> 2) * 4, kg = ct & 3;
     const int m = c0 % M;
     float scx[4], scy[4];
-    auto load_scales = [&](const StepArgs& q) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        scx[j] = -__ldg(q.xi + m + j);
-        scy[j] = -__ldg(q.eta + m + j);
-      }
-    };
-    if constexpr (!BATCH) load_scales(a);
+    for (int j = 0; j < 4; ++j) {
+      scx[j] = -__ldg(a.xi + m + j);
+      scy[j] = -__ldg(a.eta + m + j);
+    }
     constexpr int kPieces = BF ? 2 : 1;                  // pieces per chunk
     constexpr int kGrp = 8 / GV;                         // groups per piece: 2 of 4 positions, 1 of 8
     const uint64_t pol_keep = policy_evict_last();
@@ -865,18 +816,14 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
     for (int k = 0;; ++k) {
       const int t = __shfl_sync(0xffffffffu, next_item(k), 0);
       if (t < 0) break;
-      const Item im = item_of(t);
+      const Item im = Item(it, a, KC, t);
       // u^s is complete once every y item of the step before is
-      if (!BATCH && im.s > 0 && !dep_wait(ydone + im.g, im.s * it.nyi, lane, abrt, a.err)) break;
+      if (im.s > 0 && !dep_wait(ydone + im.g, im.s * it.nyi, lane, abrt, a.err)) break;
       const int line = im.tile * per_tile + c0 / M;
-      const StepArgs& ca = args_of(im);
-      if constexpr (BATCH) load_scales(ca);
-      const float* u_in = ubuf(im.g, im.s);
-      if constexpr (BATCH) u_in = ma.flip ? ma.probs[im.p].R : ma.probs[im.p].U;
-      const bool col_ok = line < (im.xpass ? ca.ny : ca.nx);
-      const size_t kstride = im.xpass ? M : static_cast<size_t>(ca.nx) * M;
-      const float* src = u_in + static_cast<size_t>(group_of(im.g)) * ca.plane +
-                         static_cast<size_t>(line) * (im.xpass ? static_cast<size_t>(ca.nx) * M : M) + m;
+      const bool col_ok = line < (im.xpass ? a.ny : a.nx);
+      const size_t kstride = im.xpass ? M : static_cast<size_t>(a.nx) * M;
+      const float* src = ubuf(im.g, im.s) + static_cast<size_t>(group_of(im.g)) * a.plane +
+                         static_cast<size_t>(line) * (im.xpass ? static_cast<size_t>(a.nx) * M : M) + m;
       float sc[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) sc[j] = im.xpass ? scx[j] : scy[j];
@@ -948,57 +895,24 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
     // ---------------- epilogue ----------------
     // The eight warps decide together (epi_all) whether to go on, so that
     // none is left waiting at the barriers of the y epilogue.
-    int cur_p = -1;
-    auto epi_args = [&]() -> const StepArgs& {
-      if constexpr (BATCH) return sh.pa;
-      else return a;
-    };
-    auto epi_bargs = [&]() -> const BoundaryArgs& {
-      if constexpr (BATCH) return sh.pb;
-      else return ma.b;
-    };
-    auto epi_side = [&](int side) -> const BoundaryArgs& {
+    auto epi_bargs = [&](int side) -> const BoundaryArgs& {
       if constexpr (DUAL) return side ? sh.pb2 : sh.pb;
-      else return epi_bargs();
+      else return ma.b;
     };
     for (int k = 0;; ++k) {
       const int t = __shfl_sync(0xffffffffu, next_item(k), 0);
       if (!epi_all(t >= 0)) break;
-      const Item im = item_of(t);
+      const Item im = Item(it, a, KC, t);
       const int b2 = k & 1;
-      if constexpr (BATCH) {
-        if (im.p != cur_p) {                                   // (the same in all eight warps)
-          const BatchProblem* P = ma.probs + im.p;
-          const int* sa = reinterpret_cast<const int*>(&P->a);
-          const int* sb = reinterpret_cast<const int*>(&P->b);
-          for (int w = tid; w < static_cast<int>(sizeof(StepArgs) / 4); w += kEpiWarps * 32)
-            reinterpret_cast<int*>(&sh.pa)[w] = sa[w];
-          for (int w = tid; w < static_cast<int>(sizeof(BoundaryArgs) / 4); w += kEpiWarps * 32)
-            reinterpret_cast<int*>(&sh.pb)[w] = sb[w];
-          epi_all(true);
-          for (int w = tid; w < M; w += kEpiWarps * 32) sh.pcs[w] = __ldg(sh.pa.PT + w);
-          BcTables(sm_epi, M).fill(sh.pb, M, tid, kEpiWarps * 32);
-          epi_all(true);
-          cur_p = im.p;
-        }
-      }
-      const StepArgs& ea = epi_args();
       const int side = side_of(im.g), lg = group_of(im.g);
-      const BoundaryArgs& eb = epi_side(side);
-      const size_t goff = static_cast<size_t>(lg) * ea.plane;
+      const size_t goff = static_cast<size_t>(lg) * a.plane;
       const float* U = ubuf(im.g, im.s);
       float* R = ubuf(im.g, im.s + 1);
-      if constexpr (BATCH) {
-        const BatchProblem* P = ma.probs + im.p;
-        U = ma.flip ? P->R : P->U;
-        R = ma.flip ? P->U : P->R;
-      }
       const uint32_t acc = tmem + b2 * acc_cols;
       const int t0 = im.tile * per_tile, row0 = im.rt0 * kMT;
       const int hl = ((DUAL && side ? ma.two.hl : ma.hl) + 2 * im.s) % 3;
       auto hist = [&](int q) {
-        if constexpr (BATCH) return ma.probs[im.p].L[q];
-        else if constexpr (DUAL) return side ? ma.two.L[q] : ma.L[q];
+        if constexpr (DUAL) return side ? ma.two.L[q] : ma.L[q];
         else return ma.L[q];
       };
       const float *L1 = hist(hl), *L2 = hist((hl + 1) % 3);
@@ -1006,7 +920,7 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
       bool ok = m_wait(&sh.acc_full[b2], (k >> 1) & 1, abrt, a.err);
       __syncwarp();
       // y: R of this step is complete once every x item of the group is
-      if (!BATCH && !im.xpass) ok = dep_wait(xdone + im.g, (im.s + 1) * it.nxi, lane, abrt, a.err) && ok;
+      if (!im.xpass) ok = dep_wait(xdone + im.g, (im.s + 1) * it.nxi, lane, abrt, a.err) && ok;
       if (!epi_all(ok)) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       auto released = [&] {
@@ -1014,21 +928,17 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
         __syncwarp();
         if (lane == 0) m_arrive(&sh.acc_empty[b2]);
       };
-      if (BATCH && !epi_all(*static_cast<volatile int*>(ea.err) == 0)) {
-        released();                                            // the medium's march has timed out
-      } else if (im.xpass) {
-        x_epilogue<MM>(ea, U, R, goff, t0, row0, im.nrt, sh.pcs, acc, sm_epi, warp, lane, released);
+      if (im.xpass) {
+        x_epilogue<MM>(a, U, R, goff, t0, row0, im.nrt, sh.pcs, acc, sm_epi, warp, lane, released);
       } else {
         const int step = DUAL && side ? ma.two.step0 + im.s * ma.two.dstep : ma.step0 + im.s * ma.dstep;
-        y_epilogue<MM>(ea, eb, U, R, L1, L2, L3, goff, step, lg, t0, row0, im.nrt, acc,
+        y_epilogue<MM>(a, epi_bargs(side), U, R, L1, L2, L3, goff, step, lg, t0, row0, im.nrt, acc,
                        sm_epi, warp, lane, [] { asm volatile("bar.sync 1, 256;" ::: "memory"); }, released);
       }
-      if constexpr (!BATCH) {
-        // handed to the signal warp, which has taken item k - 2's phase
-        if (k >= 2) ok = m_wait(&sh.sig_done[b2], ((k >> 1) - 1) & 1, abrt, a.err);
-        if (!__all_sync(0xffffffffu, ok)) ok = false;            // the next epi_all ends the loop (abort flag set)
-        if (lane == 0) m_arrive(&sh.epi_done[b2]);
-      }
+      // handed to the signal warp, which has taken item k - 2's phase
+      if (k >= 2) ok = m_wait(&sh.sig_done[b2], ((k >> 1) - 1) & 1, abrt, a.err);
+      if (!__all_sync(0xffffffffu, ok)) ok = false;            // the next epi_all ends the loop (abort flag set)
+      if (lane == 0) m_arrive(&sh.epi_done[b2]);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -1037,43 +947,34 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(tmem_cols));
 }
 
-template <int PREC, int MM, int MODE>
+template <int PREC, int MM, bool DUAL>
 cudaError_t launch_march_t(const MarchArgs& ma, int sms, cudaStream_t s) {
   constexpr size_t smem = 1024 + MarchRing<Kind<PREC>::X3>::kStage + kEpiBytes;
   static const cudaError_t attr = cudaFuncSetAttribute(
-      tc_march_kernel<PREC, MM, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+      tc_march_kernel<PREC, MM, DUAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (attr != cudaSuccess) return attr;
-  const long long items =
-      MODE == kBatch ? ma.items : static_cast<long long>(MarchItems(ma.a, ma.rt, ma.lag).per_step()) * ma.n_steps;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(items < sms ? static_cast<unsigned>(items) : static_cast<unsigned>(sms));
-  cfg.blockDim = dim3(kMarchThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = MODE == kBatch ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, tc_march_kernel<PREC, MM, MODE>, ma);
+  const long long items = static_cast<long long>(MarchItems(ma.a, ma.rt, ma.lag).per_step()) * ma.n_steps;
+  const int grid = items < sms ? static_cast<int>(items) : sms;
+  tc_march_kernel<PREC, MM, DUAL><<<grid, kMarchThreads, smem, s>>>(ma);
+  return cudaGetLastError();
 }
 
-template <int PREC, int MODE>
+template <int PREC, bool DUAL>
 cudaError_t launch_march_m(const MarchArgs& ma, int sms, cudaStream_t s) {
   switch (ma.a.M) {
-    case 16: return launch_march_t<PREC, 16, MODE>(ma, sms, s);
-    case 32: return launch_march_t<PREC, 32, MODE>(ma, sms, s);
-    default: return launch_march_t<PREC, 64, MODE>(ma, sms, s);
+    case 16: return launch_march_t<PREC, 16, DUAL>(ma, sms, s);
+    case 32: return launch_march_t<PREC, 32, DUAL>(ma, sms, s);
+    default: return launch_march_t<PREC, 64, DUAL>(ma, sms, s);
   }
 }
 
-template <int MODE>
+template <bool DUAL>
 cudaError_t launch_march_p(const MarchArgs& ma, int sms, cudaStream_t s) {
   switch (ma.a.tc_mode) {
-    case 1: return launch_march_m<1, MODE>(ma, sms, s);
-    case 2: return launch_march_m<2, MODE>(ma, sms, s);
-    case 3: return launch_march_m<3, MODE>(ma, sms, s);
-    default: return launch_march_m<4, MODE>(ma, sms, s);
+    case 1: return launch_march_m<1, DUAL>(ma, sms, s);
+    case 2: return launch_march_m<2, DUAL>(ma, sms, s);
+    case 3: return launch_march_m<3, DUAL>(ma, sms, s);
+    default: return launch_march_m<4, DUAL>(ma, sms, s);
   }
 }
 
@@ -1124,53 +1025,8 @@ cudaError_t launch_march_tc(MarchArgs ma, cudaStream_t s, long long* launches) {
   if (ma.a.G * static_cast<long long>(one.nxi > one.nyi ? one.nxi : one.nyi) > sms) ma.rt = 2;
   cudaError_t e = cudaMemsetAsync(ma.ctl, 0, tc_march_ctl_bytes(ma.a.G), s);
   if (e != cudaSuccess) return e;
-  e = ma.dual ? launch_march_p<kDual>(ma, sms, s) : launch_march_p<kSingle>(ma, sms, s);
+  e = ma.dual ? launch_march_p<true>(ma, sms, s) : launch_march_p<false>(ma, sms, s);
   if (launches) *launches += 1;
-  return e;
-}
-
-// Media with a line of more than 128 positions (as tc_march_supported): the
-// one-tile passes size every CTA of a launch for the longest line of the
-// batch, so that one 384-line medium leaves a single CTA per SM to all.
-// Twelve media of 128^2 to 384^2, M = 32, 3xTF32: 406 us a step there, 381
-// here (x 167, y 232 by themselves, the epilogues bound).
-bool launch_step_batch_march_layout(BatchProblem* probs, int n) {
-  int cx = 0, cy = 0;
-  bool rows = false;
-  for (int p = 0; p < n; ++p) {
-    const StepArgs& a = probs[p].a;
-    const MarchItems it(a, 2, 0);
-    probs[p].item0_x = cx;
-    probs[p].item0_y = cy;
-    cx += a.G * it.nxi;
-    cy += a.G * it.nyi;
-    if (a.test_expire || a.tc_scatter) return false;
-    rows = rows || a.nx > kMT || a.ny > kMT;
-  }
-  return rows;                                  // as tc_march_supported
-}
-
-cudaError_t launch_step_batch_march(const BatchProblem* probs, const BatchProblem* probs_dev, int n, int step,
-                                    int hl, bool flip, cudaStream_t s, long long* launches) {
-  MarchArgs ma{};
-  ma.a = probs[0].a;
-  ma.hl = hl;
-  ma.step0 = step;
-  ma.n_steps = 1;
-  ma.rt = 2;
-  ma.probs = probs_dev;
-  ma.n_probs = n;
-  ma.flip = flip ? 1 : 0;
-  const BatchProblem& last = probs[n - 1];
-  const MarchItems it(last.a, 2, 0);
-  ma.xpass = 1;
-  ma.items = last.item0_x + last.a.G * it.nxi;
-  cudaError_t e = launch_march_p<kBatch>(ma, sm_count(), s);
-  if (e != cudaSuccess) return e;
-  ma.xpass = 0;
-  ma.items = last.item0_y + last.a.G * it.nyi;
-  e = launch_march_p<kBatch>(ma, sm_count(), s);
-  if (launches) *launches += 2;
   return e;
 }
 
