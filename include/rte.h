@@ -411,7 +411,8 @@ rte_status rte_set_pass_variant(rte_ctx* ctx, int variant);
  *                           launches tensor-core passes that return at once
  *                           and reports RTE_ERR_TIMEOUT (clearing the word);
  *   RTE_FAULT_EXPIRE_WAIT   the next march's first one-tile-per-CTA
- *                           tensor-core pass (rte_set_pass_variant 1) has one
+ *                           tensor-core pass or multi-step launch
+ *                           (rte_set_pass_variant 1) has one
  *                           CTA wait on a barrier that nothing arrives on,
  *                           before it issues any copy or MMA; the bounded
  *                           wait runs out after about 2 s and the march

@@ -710,6 +710,10 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
       bool fine = true;
       for (int k = 0; fine; ++k) {
         const int t = atomicAdd(ma.ctl, 1);
+        // Failure injection (tests): the CTA of the first item waits on a
+        // barrier that nothing arrives on, before it has issued any copy or
+        // MMA; the bounded wait runs out and every role of every CTA leaves.
+        if (a.test_expire && t == 0 && !m_wait(&sh.d_full[0], 0, abrt, a.err)) break;
         sh.item[k % kItemRing] = t < total ? t : -1;
         m_arrive(&sh.item_full[k % kItemRing]);
         if (t >= total) break;
@@ -899,9 +903,10 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
       if constexpr (DUAL) return side ? sh.pb2 : sh.pb;
       else return ma.b;
     };
+    bool ok = true;
     for (int k = 0;; ++k) {
       const int t = __shfl_sync(0xffffffffu, next_item(k), 0);
-      if (!epi_all(t >= 0)) break;
+      if (!epi_all(t >= 0 && ok)) break;
       const Item im = Item(it, a, KC, t);
       const int b2 = k & 1;
       const int side = side_of(im.g), lg = group_of(im.g);
@@ -917,7 +922,7 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
       };
       const float *L1 = hist(hl), *L2 = hist((hl + 1) % 3);
       float* L3 = hist((hl + 2) % 3);
-      bool ok = m_wait(&sh.acc_full[b2], (k >> 1) & 1, abrt, a.err);
+      ok = m_wait(&sh.acc_full[b2], (k >> 1) & 1, abrt, a.err);
       __syncwarp();
       // y: R of this step is complete once every x item of the group is
       if (!im.xpass) ok = dep_wait(xdone + im.g, (im.s + 1) * it.nxi, lane, abrt, a.err) && ok;
@@ -937,8 +942,8 @@ __global__ void __launch_bounds__(kMarchThreads, 1) tc_march_kernel(MarchArgs ma
       }
       // handed to the signal warp, which has taken item k - 2's phase
       if (k >= 2) ok = m_wait(&sh.sig_done[b2], ((k >> 1) - 1) & 1, abrt, a.err);
-      if (!__all_sync(0xffffffffu, ok)) ok = false;            // the next epi_all ends the loop (abort flag set)
-      if (lane == 0) m_arrive(&sh.epi_done[b2]);
+      ok = __all_sync(0xffffffffu, ok);                        // false: the next epi_all ends the loop
+      if (ok && lane == 0) m_arrive(&sh.epi_done[b2]);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -997,7 +1002,7 @@ bool tc_march_supported(const StepArgs& a) {
   // 64^2, M = 32, four groups 25 us a step against 29 here, sixteen
   // groups 36 against 45.
   const bool rows = a.nx > kMT || a.ny > kMT;
-  return rows && a.tc_mode != 0 && a.tc_scatter == 0 && a.x_variant == 1 && !a.test_expire;
+  return rows && a.tc_mode != 0 && a.tc_scatter == 0 && a.x_variant == 1;
 }
 
 bool tc_march_dual(const StepArgs& a) {

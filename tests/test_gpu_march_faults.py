@@ -90,3 +90,40 @@ def test_timeout_word_of_one_medium_of_a_batch():
                 assert torch.equal(curves, fresh[0]) and torch.equal(u, fresh[1])
             assert float(fresh[1].abs().max()) > 0
             s.close()
+
+
+@pytest.mark.parametrize("groups,balance", [(1, False), (2, True), (12, False)])
+def test_expiring_wait_of_a_multi_step_launch(groups, balance):
+    """One CTA's wait runs out (about 2 s) while the others copy, multiply and
+    wait for its item: every role gives up, what is in flight is drained, the
+    call reports TIMEOUT after one launch's work, and the next is right."""
+    from paper_2202_09421_gb300 import binding as B
+    wl = _wl(150, 140, groups, steps=12)
+    flags = B.RTE_FLAG_PHOTON_BALANCE if balance else 0
+    s, clean = _solver(wl, flags=flags), _solver(wl, flags=flags)
+    B.rte_set_pass_variant(s.ctx, 1)
+    B.rte_inject_fault(s.ctx, B.RTE_FAULT_EXPIRE_WAIT)
+    before = B.rte_kernel_launches(s.ctx)
+    _timeout(s.forward, wl.groups, wl.n_steps)
+    assert B.rte_kernel_launches(s.ctx) - before < (3 if balance else 2) * wl.n_steps      # not the single passes
+    assert all(torch.equal(x, y) for x, y in zip(_results(s, wl), _results(clean, wl)))
+    s.close()
+    clean.close()
+
+
+def test_expiring_wait_of_the_marched_adjoint():
+    from paper_2202_09421_gb300 import binding as B
+    wl = _wl(160, 136, 2, steps=9)
+    s = _solver(wl, ckpt_interval=4)
+    B.rte_set_pass_variant(s.ctx, 1)
+    s.forward(wl.groups, wl.n_steps)
+    meas = 0.5 * s.readout(wl.detectors)
+    good = s.adjoint_gradient(wl.detectors, meas)
+    s.forward(wl.groups, wl.n_steps)
+    B.rte_inject_fault(s.ctx, B.RTE_FAULT_EXPIRE_WAIT)
+    _timeout(s.adjoint_gradient, wl.detectors, meas)
+    s.forward(wl.groups, wl.n_steps)
+    again = s.adjoint_gradient(wl.detectors, meas)
+    assert good[0] == again[0] > 0
+    assert torch.equal(good[1], again[1]) and torch.equal(good[2], again[2])
+    s.close()
