@@ -99,6 +99,16 @@ __device__ __forceinline__ void cp_async16(float* dst, const float* src, bool va
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(valid ? 16 : 0) : "memory");
 }
 
+// 16 bytes that the launch before may still be writing when this one begins
+// (dependent launches): a plain load, behind the wait.  A const __restrict__
+// pointer would allow read-only loads, which hold only for memory that nobody
+// writes while the kernel lives, and would let them move above the wait.
+__device__ __forceinline__ float4 ld_plain4(const float* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+
 // acc[r][c] = sum_k AT[k][row(r)] slab[k][col(c)], k ascending.  copy_slab(k0)
 // starts the copies of slab rows k0 .. k0 + kKC - 1 (zeros past the line).
 template <int T, class CopySlab>
@@ -161,7 +171,7 @@ __device__ __forceinline__ void tile_gemm(const float* __restrict__ AT, int n, c
 }
 
 template <int T>
-__global__ void __launch_bounds__(kMaxThreads) xpass_kernel(StepArgs a, TileShape ts, const float* __restrict__ U,
+__global__ void __launch_bounds__(kMaxThreads) xpass_kernel(StepArgs a, TileShape ts, const float* U,
                                                             float* __restrict__ R) {
   extern __shared__ __align__(16) float smem[];
   const int n = a.nx, M = a.M, ldb = ts.BN + kSlabPad;
@@ -266,7 +276,7 @@ __global__ void __launch_bounds__(kMaxThreads) xpass_kernel(StepArgs a, TileShap
 // a separate instance, so that the forward step compiles without it.
 template <int T, bool TR>
 __global__ void __launch_bounds__(kMaxThreads) ypass_kernel(StepArgs a, BoundaryArgs b, TileShape ts,
-                                                            float* __restrict__ U, const float* __restrict__ R,
+                                                            float* __restrict__ U, const float* R,
                                                             const float* __restrict__ L1,
                                                             const float* __restrict__ L2, float* __restrict__ L3,
                                                             int src_step, int ring_step) {
@@ -356,7 +366,7 @@ __global__ void __launch_bounds__(kMaxThreads) ypass_kernel(StepArgs a, Boundary
       if (i >= nx || j >= n) continue;
       float* ac = &acc[jj][4 * v];
       const size_t base = base0 + static_cast<size_t>(j) * nx * M;
-      const float4 r4 = ld4(R + base), p4 = ld4(L1 + base), q4 = ld4(L2 + base), s4 = ld4(L3 + base);
+      const float4 r4 = ld_plain4(R + base), p4 = ld4(L1 + base), q4 = ld4(L2 + base), s4 = ld4(L3 + base);
       if constexpr (TR) {
         // transposed step: ubar = w^{k+1} + L^T v
         ac[0] = r4.x - eta.x * ac[0] + p4.x;

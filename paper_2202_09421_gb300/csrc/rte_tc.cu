@@ -309,7 +309,7 @@ __device__ __forceinline__ void tc_pass_body(const StepArgs& a, const BoundaryAr
         const int i = t * kMT + row, j = t0 + r, m0 = grp * 4;
         if (i < nx && j < ny && m0 < M) {
           const size_t cell = static_cast<size_t>(j) * nx + i;
-          val[h] = *reinterpret_cast<const float4*>(U + goff + cell * M + m0);
+          val[h] = ld4_plain(U + goff + cell * M + m0);
           bv[h] = __ldg(a.mus + cell);
         }
       }
@@ -381,7 +381,7 @@ __device__ __forceinline__ void tc_pass_body(const StepArgs& a, const BoundaryAr
 #pragma unroll
         for (int k = 0; k < MM / 4; ++k) {
           float4 u4 = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (valid) u4 = reinterpret_cast<const float4*>(U + goff + cell * M)[k];
+          if (valid) u4 = ld4_plain(U + goff + cell * M + 4 * k);
           uu[4 * k] = u4.x; uu[4 * k + 1] = u4.y; uu[4 * k + 2] = u4.z; uu[4 * k + 3] = u4.w;
         }
         if (valid) {
@@ -429,9 +429,9 @@ __device__ __forceinline__ void tc_pass_body(const StepArgs& a, const BoundaryAr
         const size_t cell = static_cast<size_t>(j) * nx + i;
         bv = __ldg(a.mus + cell);
         ab = __ldg(a.mua + cell) + bv;
-        const float4* up = reinterpret_cast<const float4*>(U + goff + cell * M);
+        const float* up = U + goff + cell * M;
 #pragma unroll
-        for (int k = 0; k < MM / 4; ++k) u4[k] = up[k];
+        for (int k = 0; k < MM / 4; ++k) u4[k] = ld4_plain(up + 4 * k);
       };
       load_pair(half, ucur, abcur, bcur);
       for (int p = half; p < n_pairs; p += 2) {

@@ -223,6 +223,15 @@ __device__ __forceinline__ float4 ld4_hint(const float* ptr, uint64_t pol) {
   return v;
 }
 
+// 16 bytes that the launch before may still be writing when this one begins
+// (dependent launches): a plain load, behind the wait, that the compiler
+// neither turns into a read-only one nor moves over the wait.
+__device__ __forceinline__ float4 ld4_plain(const float* ptr) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(ptr));
+  return v;
+}
+
 // 32-byte global accesses (sm_100 and later): whole 32-byte sectors per
 // thread, so a warp that walks 32 nodes of 128 B leaves no half-written
 // sectors for L2 to merge.  Addresses are 32-byte aligned.
