@@ -61,6 +61,21 @@ __device__ __forceinline__ float exitance_sum_node(const float* w, const float* 
   return p[0];
 }
 
+// sum_m w_m v_m of a node whose M ordinates are adjacent lanes (w_m v_m of
+// ordinate m on lane m), in the order of exitance_sum_node.  The sum is in the
+// node's lanes with m % 4 == 0.
+template <int M>
+__device__ __forceinline__ float lane_exitance(float w, float v, int lane) {
+  const int q = lane & ~3;
+  float ex = __shfl_sync(0xffffffffu, w, q) * __shfl_sync(0xffffffffu, v, q);
+#pragma unroll
+  for (int e = 1; e < 4; ++e)
+    ex = fmaf(__shfl_sync(0xffffffffu, w, q + e), __shfl_sync(0xffffffffu, v, q + e), ex);
+#pragma unroll
+  for (int o = 4; o < M; o <<= 1) ex += __shfl_xor_sync(0xffffffffu, ex, o);
+  return ex;
+}
+
 // Operand kinds of the precision modes (rte.h): 1 3xTF32, 2 TF32, 3 bf16x3,
 // 4 BF16.  KC = K positions per 128-byte row, GV = values per 16-byte group.
 template <int PREC>

@@ -396,8 +396,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1)
               if (fy == 1 && !(bt || tp)) continue;
               const int F = fy == 0 ? (lf ? 0 : 1) : (bt ? 2 : 3);
               const float* val = bc_s + t * kNC + w * M;
-              float ex = 0.f;
-              for (int m = 0; m < M; ++m) ex = fmaf(bc_wexit[F * M + m], val[m], ex);
+              const float ex = exitance_sum_node<M>(bc_wexit + F * M, val);
               ro[fy == 0 ? (lf ? j : ny + j) : (bt ? 2 * ny + i : 2 * ny + nx + i)] = ex;
             }
           }

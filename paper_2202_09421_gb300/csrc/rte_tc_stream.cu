@@ -109,21 +109,6 @@ __host__ __device__ inline int stream_stages(int stage_bytes) {
   return s > kMaxStages ? kMaxStages : s;
 }
 
-// sum_m w_m v_m of a node whose M ordinates are adjacent lanes (w_m v_m of
-// ordinate m on lane m), in the order of the one-tile y-pass: four ordinates
-// in order, then pairwise.  The sum in the node's lanes with m % 4 == 0.
-template <int M>
-__device__ __forceinline__ float lane_exitance(float w, float v, int lane) {
-  const int q = lane & ~3;
-  float ex = __shfl_sync(0xffffffffu, w, q) * __shfl_sync(0xffffffffu, v, q);
-#pragma unroll
-  for (int e = 1; e < 4; ++e)
-    ex = fmaf(__shfl_sync(0xffffffffu, w, q + e), __shfl_sync(0xffffffffu, v, q + e), ex);
-#pragma unroll
-  for (int o = 4; o < M; o <<= 1) ex += __shfl_xor_sync(0xffffffffu, ex, o);
-  return ex;
-}
-
 // The y epilogue's rows per accumulator load: all loads of a chunk are
 // issued before any is used.
 constexpr int kRowsY = 16;

@@ -464,16 +464,12 @@ __global__ void __launch_bounds__(kWsThreads, 1)
             if (ro) {
               if (__any_sync(kFull, bnd && (lf || rt))) {
                 const int F = lf ? 0 : 1;
-                float ex = 0.f;
-                for (int mm = 0; mm < M; ++mm)
-                  ex = fmaf(bc_wexit[F * M + mm], __shfl_sync(kFull, val, base + mm), ex);
+                const float ex = lane_exitance<M>(bc_wexit[F * M + m], val, lane);
                 if (bnd && (lf || rt) && m == 0) ro[lf ? j : ny + j] = ex;
               }
               if (__any_sync(kFull, bnd && (bt || tp))) {
                 const int F = bt ? 2 : 3;
-                float ex = 0.f;
-                for (int mm = 0; mm < M; ++mm)
-                  ex = fmaf(bc_wexit[F * M + mm], __shfl_sync(kFull, val, base + mm), ex);
+                const float ex = lane_exitance<M>(bc_wexit[F * M + m], val, lane);
                 if (bnd && (bt || tp) && m == 0) ro[bt ? 2 * ny + i : 2 * ny + nx + i] = ex;
               }
             }
