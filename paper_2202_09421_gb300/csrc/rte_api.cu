@@ -53,7 +53,6 @@ struct rte_ctx {
   bool inject_expire = false;
   // item counters of the multi-step launches
   DevBuf ctl;
-  DevBuf mseg;                       // states of one launch: adjoint levels, or steps with the photon balance
   // photon balance of the last rte_forward (RTE_FLAG_PHOTON_BALANCE):
   // [G][n_steps][3] FP64 terms, block partials, per-group tickets, and the
   // FP64 cos / sin of the ordinates
@@ -283,12 +282,17 @@ rte_status snapshot(rte_ctx* c, const float* u, int G, const std::vector<int>& s
 // Steps of a multi-step launch, at most: 36 ms at 16 groups of 256^2, so that
 // work on other streams gets its turn (a launch costs about 0.1 ms of ramp).
 constexpr int kMarchSteps = 128;
-// The same with the photon balance of every step (16 groups of 256^2: 0.1 ms
-// of ramp over four steps; the buffer holds twice as many states).
-constexpr int kBalanceSteps = 4;
+// The same with the photon balance of every step: the states of the last two
+// steps of a launch are in U and R.
+constexpr int kBalanceSteps = 2;
 // The same for the adjoint beside a recompute: the adjoint levels of a launch
 // are kept for its gradient terms.
 constexpr int kDualSteps = 32;
+// Checkpoint interval from which the two march side by side (a launch takes at
+// most half of it; 256^2, two groups, single passes on two streams against
+// them: an interval of 3 226 us against 241, of 5 218 against 216, of 6 217
+// against 205, of 20 222 against 193).
+constexpr int kDualInterval = 6;
 
 // Runs steps [s_begin, s_end) of the forward march on (U, R, L), starting
 // from whatever state they hold; records checkpoints/exitance/fluence when
@@ -311,11 +315,7 @@ rte_status march(rte_ctx* c, DevBuf& U, DevBuf& R, DevBuf* L, int& hl, int G, in
   // recompute stream: a launch that keeps every SM for a whole segment leaves
   // nothing to overlap with the passes of the other stream.
   const bool overlapped = c->astream && c->stream == c->astream;
-  // The photon balance takes the state of every step: runs of kBalanceSteps
-  // into slots, one half of the buffer after the other (a run starts from the
-  // last slot of the run before); without the buffer, single passes.
-  const bool marched = !fused && !c->timing && !overlapped && rte_kern::tc_march_supported(a) &&
-                       (!balance_out || c->mseg.bytes >= 2 * kBalanceSteps * gbytes);
+  const bool marched = !fused && !c->timing && !overlapped && rte_kern::tc_march_supported(a);
   auto balance = [&](const float* u, int step) {
     return cuda_status(rte_kern::launch_balance(
         u, c->plane, c->nx, c->ny, c->M, G, F(c->mua), D(c->trig), c->dx, c->dy, 2.0 * kPi / c->M, c->opt.c,
@@ -323,7 +323,7 @@ rte_status march(rte_ctx* c, DevBuf& U, DevBuf& R, DevBuf* L, int& hl, int G, in
         &c->launches));
   };
   if (marched) {
-    if (!seg_out && !balance_out && ((s_end - s_begin) & 1)) {
+    if (!seg_out && ((s_end - s_begin) & 1)) {
       RTE_TRY(cuda_status(cudaMemcpyAsync(oth, cur, gbytes, cudaMemcpyDeviceToDevice, c->stream)));
       std::swap(cur, oth);
     }
@@ -337,7 +337,7 @@ rte_status march(rte_ctx* c, DevBuf& U, DevBuf& R, DevBuf* L, int& hl, int G, in
     for (int q = 0; q < 3; ++q) ma.L[q] = F(L[q]);
     const size_t gfloats = static_cast<size_t>(G) * c->plane;
     const int longest = balance_out ? kBalanceSteps : kMarchSteps;
-    for (int s = s_begin, run = 0; s < s_end; ++run) {
+    for (int s = s_begin; s < s_end;) {
       if (save_ckpt && I > 0 && s % I == 0) RTE_TRY(copy_checkpoint(c, cur, L, hl, G, s));
       int e = s + 1;                                   // the run [s, e)
       while (e < s_end && e - s < longest && !(save_ckpt && I > 0 && e % I == 0) && !(fluence_out && snap_index[e - 1] >= 0)) ++e;
@@ -350,23 +350,16 @@ rte_status march(rte_ctx* c, DevBuf& U, DevBuf& R, DevBuf* L, int& hl, int G, in
         ma.slots = (*seg_out)[s - s_begin];
         ma.slot_floats = gfloats;
       }
-      if (balance_out) {
-        ma.slots = F(c->mseg) + static_cast<size_t>(run % 2) * kBalanceSteps * gfloats;
-        ma.slot_floats = gfloats;
-      }
       RTE_TRY(cuda_status(rte_kern::launch_march_tc(ma, c->stream, &c->launches)));
       hl = (hl + 2 * (e - s)) % 3;
       if (balance_out)
-        for (int q = s; q < e; ++q) RTE_TRY(balance(ma.slots + static_cast<size_t>(q - s) * gfloats, q));
+        for (int q = s; q < e; ++q) RTE_TRY(balance((q - s) & 1 ? cur : oth, q));
       if (seg_out) cur = (*seg_out)[e - 1 - s_begin];
-      else if (balance_out) cur = ma.slots + static_cast<size_t>(e - 1 - s) * gfloats;
       else if ((e - s) & 1) std::swap(cur, oth);
       if (fluence_out && snap_index[e - 1] >= 0)
         RTE_TRY(snapshot(c, cur, G, snap_index, e - 1, fluence_out));
       s = e;
     }
-    if (balance_out)
-      RTE_TRY(cuda_status(cudaMemcpyAsync(U.p, cur, gbytes, cudaMemcpyDeviceToDevice, c->stream)));
     return RTE_OK;
   }
   for (int s = s_begin; s < s_end; ++s) {
@@ -608,7 +601,7 @@ unsigned long long key_ptr(const void* p) { return static_cast<unsigned long lon
 // Key of the buffers a forward march of context c touches.
 void append_forward_key(const rte_ctx* c, std::vector<unsigned long long>& key) {
   const void* ptrs[] = {c->U.p, c->R.p, c->L[0].p, c->L[1].p, c->L[2].p, c->ring.p, c->S.p, c->A.p,
-                        c->T.p, c->ckpt.p, c->mua.p, c->mus.p, c->ctl.p, c->mseg.p};
+                        c->T.p, c->ckpt.p, c->mua.p, c->mus.p, c->ctl.p};
   key.push_back(static_cast<unsigned long long>(c->n_steps));
   key.push_back(static_cast<unsigned long long>(c->G));
   key.push_back(static_cast<unsigned long long>(c->kmax));
@@ -815,7 +808,6 @@ rte_status rte_destroy(rte_ctx* c) {
   release(c->batch_jobs);
   release(c->err);
   release(c->ctl);
-  release(c->mseg);
   release(c->bal);
   release(c->bal_partial);
   release(c->bal_ticket);
@@ -1015,9 +1007,6 @@ rte_status rte_forward(rte_ctx* c, const rte_source_group* groups, int n_groups,
     RTE_TRY(ensure(c->bal_ticket, static_cast<size_t>(G) * sizeof(unsigned)));
     RTE_TRY(cuda_status(cudaMemsetAsync(c->bal_ticket.p, 0, static_cast<size_t>(G) * sizeof(unsigned), c->stream)));
     balance = D(c->bal);
-    // states for the multi-step launches (single passes without the memory)
-    if (rte_kern::tc_march_supported(step_args(c, G)))
-      ensure(c->mseg, 2 * kBalanceSteps * static_cast<size_t>(G) * c->plane * sizeof(float));
   }
   const rte_kern::BoundaryArgs b = forward_bargs(c);
   std::vector<unsigned long long> key;
@@ -1265,14 +1254,15 @@ static rte_status adjoint_impl(rte_ctx* c, const rte_detector* dets, int n_det, 
   // Continuous form with multi-step launches, all on the context's stream.
   // With few groups (tc_march_dual) the adjoint levels of a segment march
   // beside the recompute of the next one, in launches of up to kDualSteps
-  // levels of both, each followed by its gradient terms; the adjoint levels
-  // of a launch take a buffer of their own.  With more groups, or without
-  // the memory for that buffer, recompute, adjoint and gradient of a segment
-  // follow one another, with the adjoint levels in the second segment buffer.
-  const bool marched = !discrete && !fused_adj && !c->timing && rte_kern::tc_march_supported(sa);
-  const int chunk = std::min(I, kDualSteps);
-  const bool dual = marched && rte_kern::tc_march_dual(sa) &&
-                    ensure(c->mseg, static_cast<size_t>(chunk) * gbytes) == RTE_OK;
+  // levels of both, each followed by its gradient terms.  With more groups,
+  // recompute, adjoint and gradient of a segment follow one another, with the
+  // adjoint levels in the second segment buffer.  Short segments take single
+  // passes on two streams.
+  const bool few = rte_kern::tc_march_dual(sa);
+  const bool marched =
+      !discrete && !fused_adj && !c->timing && rte_kern::tc_march_supported(sa) && I >= (few ? kDualInterval : 2);
+  const bool dual = marched && few;
+  const int chunk = std::min(I / 2, kDualSteps);
   // Levels needed: forward steps 0 .. N-2 (the adjoint vanishes at the last).
   const int last = N - 2;
   // Segments in reverse order.  The forward recompute of a segment (second
@@ -1348,7 +1338,6 @@ static rte_status adjoint_impl(rte_ctx* c, const rte_detector* dets, int n_det, 
         rte_kern::MarchSide adj{}, rec{};
         adj.b = ba;
         adj.u0 = adj.u1 = mcur;
-        adj.slots = F(c->mseg);
         adj.hl = hl_adj;
         adj.step0 = s_end - 1 - d;
         adj.dstep = -1;
@@ -1365,6 +1354,12 @@ static rte_status adjoint_impl(rte_ctx* c, const rte_detector* dets, int n_det, 
         }
         const bool has_adj = d < n, has_rec = d2 < n2;
         ma.n_steps = std::min(has_adj ? std::min(chunk, n - d) : kMarchSteps, has_rec ? n2 - d2 : n);
+        // The adjoint levels go where no forward level is kept: the first
+        // launch's at the end of the next segment's half, of which it writes
+        // no more than the first half, the others' over levels of this segment
+        // whose gradient terms are formed.
+        if (has_adj && d > 0) ma.n_steps = std::min(ma.n_steps, d);
+        adj.slots = d == 0 ? nxt + static_cast<size_t>(I - ma.n_steps) * gfloats : fwd + static_cast<size_t>(n - d) * gfloats;
         ma.dual = has_adj && has_rec ? 1 : 0;
         const rte_kern::MarchSide& one = has_adj ? adj : rec;
         ma.b = one.b;

@@ -127,3 +127,30 @@ def test_expiring_wait_of_the_marched_adjoint():
     assert good[0] == again[0] > 0
     assert torch.equal(good[1], again[1]) and torch.equal(good[2], again[2])
     s.close()
+
+
+def _taken(fn):
+    """Device memory that a call leaves allocated."""
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    fn()
+    torch.cuda.synchronize()
+    return free - torch.cuda.mem_get_info()[0]
+
+
+@pytest.mark.parametrize("balance,ckpt", [(False, 20), (True, 0)])
+def test_multi_step_launches_take_no_states_of_their_own(balance, ckpt):
+    """A forward keeps the state, its scratch, three histories and four states
+    per checkpoint; a gradient two segments, the adjoint state, its scratch
+    and three histories.  The multi-step launches add none (a few MB of tables
+    and the allocator's granules aside)."""
+    from paper_2202_09421_gb300 import binding as B
+    wl = _wl(256, 256, 3, steps=41)
+    s = _solver(wl, ckpt_interval=ckpt, flags=B.RTE_FLAG_PHOTON_BALANCE if balance else 0)
+    state = 3 * 256 * 256 * 32 * 4
+    n_ckpt = 3 if ckpt else 0
+    assert _taken(lambda: s.forward(wl.groups, wl.n_steps)) <= (5 + 4 * n_ckpt) * state + state
+    if ckpt:
+        meas = torch.zeros_like(s.readout(wl.detectors))
+        assert _taken(lambda: s.adjoint_gradient(wl.detectors, meas)) <= (2 * ckpt + 5) * state + state
+    s.close()
