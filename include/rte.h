@@ -375,7 +375,10 @@ long long rte_graph_captures(const rte_ctx* ctx);
  *      without RTE_FLAG_TC_SCATTER and with a line of more than 128
  *      positions, the same tiles as items of a persistent launch of up to
  *      128 steps (between checkpoints and snapshots), bit for bit the same
- *      results, also in the segments of rte_adjoint_gradient;
+ *      results, also in the segments of rte_adjoint_gradient.  A context on
+ *      which no schedule was set, or whose schedule the autotuner set, takes
+ *      these launches at the sizes and runs of steps where they are faster
+ *      than two passes a step; schedule 1 set here, wherever supported;
  *   2  one-tile-per-CTA x-pass and the pipelined persistent y-pass (the main
  *      loop of one tile and the epilogue of the previous one on two warp
  *      groups of one CTA per SM) where supported (tensor-core precisions,

@@ -59,6 +59,7 @@ struct rte_ctx {
   DevBuf bal, bal_partial, bal_ticket, trig;
   bool bal_valid = false;
   int x_variant = 1;               // pass kernels: 0 persistent warp-specialised, 1 one tile per CTA, 2 pipelined y-pass
+  bool march_all = false;          // schedule 1 by the caller: multi-step launches wherever supported
   // state of the last forward
   int G = 0, n_steps = -1, kmax = 0;
   int hl = 0;                      // history rotation index
@@ -181,6 +182,7 @@ rte_kern::StepArgs step_args(rte_ctx* c, int G) {
   a.tc_mode = c->tc_mode;
   a.tc_scatter = (c->par.flags & RTE_FLAG_TC_SCATTER) ? 1 : 0;
   a.x_variant = c->x_variant;
+  a.march_all = c->march_all ? 1 : 0;
   a.DxImg = c->DxImg.p;
   a.DyImg = c->DyImg.p;
   a.PImg = F(c->PImg);
@@ -310,63 +312,71 @@ rte_status march(rte_ctx* c, DevBuf& U, DevBuf& R, DevBuf* L, int& hl, int G, in
   float* cur = F(U);
   float* oth = F(R);
   // Multi-step launches: runs of steps between checkpoints and snapshots.
-  // Without slots the state alternates between U and R, so that it ends in U
-  // (an odd number of steps starts from a copy in R).  Not on the adjoint's
+  // Without slots the state alternates between U and R.  Not on the adjoint's
   // recompute stream: a launch that keeps every SM for a whole segment leaves
   // nothing to overlap with the passes of the other stream.
   const bool overlapped = c->astream && c->stream == c->astream;
   const bool marched = !fused && !c->timing && !overlapped && rte_kern::tc_march_supported(a);
+  const int longest = balance_out ? kBalanceSteps : kMarchSteps;
+  const int shortest = marched ? rte_kern::tc_march_min_run(a) : 0;
+  auto run_end = [&](int s) {                          // the run [s, e)
+    int e = s + 1;
+    while (marched && e < s_end && e - s < longest && !(save_ckpt && I > 0 && e % I == 0) &&
+           !(fluence_out && snap_index[e - 1] >= 0))
+      ++e;
+    return e;
+  };
+  if (marched && !seg_out) {
+    // start in R where the launches would otherwise end there
+    int odd = 0;
+    for (int s = s_begin, e; s < s_end; s = e) {
+      e = run_end(s);
+      if (e - s >= shortest) odd ^= (e - s) & 1;
+    }
+    if (odd) {
+      RTE_TRY(cuda_status(cudaMemcpyAsync(oth, cur, gbytes, cudaMemcpyDeviceToDevice, c->stream)));
+      std::swap(cur, oth);
+    }
+  }
+  // The photon balance takes the state of every step.
   auto balance = [&](const float* u, int step) {
     return cuda_status(rte_kern::launch_balance(
         u, c->plane, c->nx, c->ny, c->M, G, F(c->mua), D(c->trig), c->dx, c->dy, 2.0 * kPi / c->M, c->opt.c,
         D(c->bal_partial), static_cast<unsigned*>(c->bal_ticket.p), balance_out, step, c->n_steps, c->stream,
         &c->launches));
   };
-  if (marched) {
-    if (!seg_out && ((s_end - s_begin) & 1)) {
-      RTE_TRY(cuda_status(cudaMemcpyAsync(oth, cur, gbytes, cudaMemcpyDeviceToDevice, c->stream)));
-      std::swap(cur, oth);
-    }
+  // steps [s, e) in one launch
+  auto march_run = [&](int s, int e) -> rte_status {
     rte_kern::MarchArgs ma{};
     ma.a = a;
     ma.b = b;
-    ma.slots = nullptr;
-    ma.slot_floats = 0;
+    ma.slots = seg_out ? (*seg_out)[s - s_begin] : nullptr;
+    ma.slot_floats = seg_out ? static_cast<size_t>(G) * c->plane : 0;
     ma.dstep = 1;
     ma.ctl = static_cast<int*>(c->ctl.p);
     for (int q = 0; q < 3; ++q) ma.L[q] = F(L[q]);
-    const size_t gfloats = static_cast<size_t>(G) * c->plane;
-    const int longest = balance_out ? kBalanceSteps : kMarchSteps;
-    for (int s = s_begin; s < s_end;) {
-      if (save_ckpt && I > 0 && s % I == 0) RTE_TRY(copy_checkpoint(c, cur, L, hl, G, s));
-      int e = s + 1;                                   // the run [s, e)
-      while (e < s_end && e - s < longest && !(save_ckpt && I > 0 && e % I == 0) && !(fluence_out && snap_index[e - 1] >= 0)) ++e;
-      ma.u0 = cur;
-      ma.u1 = oth;
-      ma.hl = hl;
-      ma.step0 = s;
-      ma.n_steps = e - s;
-      if (seg_out) {
-        ma.slots = (*seg_out)[s - s_begin];
-        ma.slot_floats = gfloats;
-      }
-      RTE_TRY(cuda_status(rte_kern::launch_march_tc(ma, c->stream, &c->launches)));
-      hl = (hl + 2 * (e - s)) % 3;
-      if (balance_out)
-        for (int q = s; q < e; ++q) RTE_TRY(balance((q - s) & 1 ? cur : oth, q));
-      if (seg_out) cur = (*seg_out)[e - 1 - s_begin];
-      else if ((e - s) & 1) std::swap(cur, oth);
-      if (fluence_out && snap_index[e - 1] >= 0)
-        RTE_TRY(snapshot(c, cur, G, snap_index, e - 1, fluence_out));
-      s = e;
-    }
+    ma.u0 = cur;
+    ma.u1 = oth;
+    ma.hl = hl;
+    ma.step0 = s;
+    ma.n_steps = e - s;
+    RTE_TRY(cuda_status(rte_kern::launch_march_tc(ma, c->stream, &c->launches)));
+    hl = (hl + 2 * (e - s)) % 3;
+    if (balance_out)
+      for (int q = s; q < e; ++q) RTE_TRY(balance((q - s) & 1 ? cur : oth, q));
+    if (seg_out) cur = (*seg_out)[e - 1 - s_begin];
+    else if ((e - s) & 1) std::swap(cur, oth);
     return RTE_OK;
-  }
-  for (int s = s_begin; s < s_end; ++s) {
+  };
+  // step s by itself
+  auto pass_step = [&](int s) -> rte_status {
+    if (cur != F(U) && cur != F(R)) {                  // a slot keeps its state
+      RTE_TRY(cuda_status(cudaMemcpyAsync(U.p, cur, gbytes, cudaMemcpyDeviceToDevice, c->stream)));
+      cur = F(U);
+    }
     float* L1 = F(L[hl]);
     float* L2 = F(L[(hl + 1) % 3]);
     float* L3 = F(L[(hl + 2) % 3]);
-    if (save_ckpt && I > 0 && s % I == 0) RTE_TRY(copy_checkpoint(c, cur, L, hl, G, s));
     cudaEvent_t* ev = nullptr;
     if (c->timing) {
       while (c->events.size() < 3 * (c->n_timed + 1)) {
@@ -382,17 +392,26 @@ rte_status march(rte_ctx* c, DevBuf& U, DevBuf& R, DevBuf* L, int& hl, int G, in
       RTE_TRY(cuda_status(step_fn(a, b, cur, oth, L1, L2, L3, s, c->stream, &c->launches, ev)));
       std::swap(cur, oth);
     } else {
-      RTE_TRY(cuda_status(rte_kern::launch_step(a, b, cur, F(R), L1, L2, L3, s, c->stream,
+      RTE_TRY(cuda_status(rte_kern::launch_step(a, b, cur, oth, L1, L2, L3, s, c->stream,
                                                 &c->launches, ev)));
     }
     hl = (hl + 2) % 3;
-    if (fluence_out && snap_index[s] >= 0) RTE_TRY(snapshot(c, cur, G, snap_index, s, fluence_out));
     if (seg_out)
       RTE_TRY(cuda_status(cudaMemcpyAsync((*seg_out)[s - s_begin], cur, gbytes,
                                           cudaMemcpyDeviceToDevice, c->stream)));
-    if (balance_out) RTE_TRY(balance(cur, s));
+    return balance_out ? balance(cur, s) : RTE_OK;
+  };
+  for (int s = s_begin, e; s < s_end; s = e) {
+    if (save_ckpt && I > 0 && s % I == 0) RTE_TRY(copy_checkpoint(c, cur, L, hl, G, s));
+    e = run_end(s);
+    if (marched && e - s >= shortest) {
+      RTE_TRY(march_run(s, e));
+    } else {
+      for (int q = s; q < e; ++q) RTE_TRY(pass_step(q));
+    }
+    if (fluence_out && snap_index[e - 1] >= 0) RTE_TRY(snapshot(c, cur, G, snap_index, e - 1, fluence_out));
   }
-  if (cur != F(U))
+  if (cur != F(U) && !(seg_out && marched))
     RTE_TRY(cuda_status(cudaMemcpyAsync(U.p, cur, gbytes, cudaMemcpyDeviceToDevice, c->stream)));
   return RTE_OK;
 }
@@ -605,7 +624,7 @@ void append_forward_key(const rte_ctx* c, std::vector<unsigned long long>& key) 
   key.push_back(static_cast<unsigned long long>(c->n_steps));
   key.push_back(static_cast<unsigned long long>(c->G));
   key.push_back(static_cast<unsigned long long>(c->kmax));
-  key.push_back(static_cast<unsigned long long>(c->x_variant));
+  key.push_back(static_cast<unsigned long long>(c->x_variant) + (c->march_all ? 16 : 0));
   key.push_back(static_cast<unsigned long long>(c->par.flags));
   key.push_back(static_cast<unsigned long long>(c->inject_expire));
   for (const void* p : ptrs) key.push_back(key_ptr(p));
@@ -640,6 +659,7 @@ long long rte_graph_captures(const rte_ctx* ctx) { return ctx ? ctx->graph_captu
 rte_status rte_set_pass_variant(rte_ctx* c, int variant) {
   if (!c || variant < 0 || variant > 5) return RTE_ERR_INVALID_ARG;
   c->x_variant = variant;
+  c->march_all = true;
   return RTE_OK;
 }
 
@@ -673,6 +693,8 @@ rte_status rte_autotune(rte_ctx* c, const rte_source_group* groups, int n_groups
     cands.push_back(choice);
   }
   const int keep_variant = c->x_variant, keep_flags = c->par.flags;
+  const bool keep_march_all = c->march_all;
+  c->march_all = false;                                   // multi-step launches by size, in the trials and from now on
   const bool keep_timing = c->timing;
   c->timing = false;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -705,6 +727,7 @@ rte_status rte_autotune(rte_ctx* c, const rte_source_group* groups, int n_groups
   if (st != RTE_OK || best_choice < 0) {
     c->x_variant = keep_variant;
     c->par.flags = keep_flags;
+    c->march_all = keep_march_all;
     return st != RTE_OK ? st : RTE_ERR_STATE;
   }
   c->x_variant = best_choice % 6;

@@ -63,6 +63,7 @@ struct StepArgs {
   int x_variant;                    // 0 persistent warp-specialised passes, 1 one tile per CTA, 2 pipelined y-pass,
                                     // 3 tile-local fused step, 4 TMA-fed persistent x-pass + one-tile y-pass,
                                     // 5 TMA-fed persistent x- and y-passes
+  int march_all;                    // multi-step launches wherever supported, not only where they are faster
   const void* DxImg;
   const void* DyImg;
   const float* PImg;                // phase matrix as the scattering operand
@@ -133,7 +134,7 @@ cudaError_t launch_step_tc_batched(const BatchProblem* probs, const BatchProblem
 
 // Several steps of every group in one launch (rte_tc_march.cu): schedule 1
 // with a line of more than 128 positions, without the tensor-core scattering
-// flag.  State buffers: u0 and u1
+// flag, where it is the faster form (or march_all).  State buffers: u0 and u1
 // alternate (the state before step k of the launch is in u0 for even k, u1
 // for odd k), or, with slots, u^{k} of step k > 0 is written to slot k - 1
 // (slot_floats apart) and u0 holds the state before the first.  L[hl] is
@@ -166,7 +167,9 @@ struct MarchArgs {
   int dual;
   MarchSide two;
 };
+// Whether steps take this form, and the shortest run of steps that does.
 bool tc_march_supported(const StepArgs& a);
+int tc_march_min_run(const StepArgs& a);
 // Whether two marches of a.G groups are faster side by side than in turn.
 bool tc_march_dual(const StepArgs& a);
 size_t tc_march_ctl_bytes(int G);

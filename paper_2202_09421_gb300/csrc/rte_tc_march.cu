@@ -996,13 +996,78 @@ int sm_count() {
 
 }  // namespace
 
+namespace {
+
+// What a pass of all groups has to work off.
+struct PassTiles {
+  long long most, shorter;           // slab tiles: of either pass at most, of the pass along the shorter axis
+  int lo, hi;                        // positions of the shorter and the longer axis
+  bool pairs;                        // the one-tile passes hold two CTAs on an SM
+  explicit PassTiles(const StepArgs& a) {
+    const int per_tile = kNC / a.M;
+    const long long tx = static_cast<long long>(a.G) * ((a.ny + per_tile - 1) / per_tile),
+                    ty = static_cast<long long>(a.G) * ((a.nx + per_tile - 1) / per_tile);
+    most = tx > ty ? tx : ty;
+    shorter = a.nx < a.ny ? tx : ty;
+    lo = a.nx < a.ny ? a.nx : a.ny;
+    hi = a.nx < a.ny ? a.ny : a.nx;
+    pairs = a.M < 64 && hi <= 256;
+  }
+};
+
+// Whether the multi-step launches are faster than two one-tile passes a step.
+// They gain where a pass is a chain (few tiles, many K chunks: the split
+// products of 3xTF32) or holds one CTA per SM; they lose where the passes fill
+// every SM with two CTAs and have little to do per tile: a short axis (its
+// items are mostly latency, here one at a time per SM), a second row tile of a
+// few rows, tiles that fit one wave of two per SM but not one of one.  The
+// lines are drawn through times at 1010 random sizes (16 to 512 positions, 1
+// to 24 groups, every precision and M), 40 steps in one run; the speed of the
+// passes is 1:
+//   taken: 620 sizes, geometric mean 1.24, 6 below 0.97 (the worst 0.90);
+//   left:  0.42 to 1.5 (206 x 21, M = 32, 22 groups, BF16 66 us a step in the
+//   passes, 130 here; 24 x 256, M = 16, 40 groups, 3xTF32 88 against 150;
+//   260 x 24, M = 32, 16 groups, TF32 60 against 113; 130 x 130, M = 16, 16
+//   groups, TF32 51 against 69), geometric mean 0.97.
+bool march_pays(const StepArgs& a) {
+  const PassTiles t(a);
+  const int sms = sm_count();
+  const bool x3tf32 = a.tc_mode == 1, bf16 = a.tc_mode == 4;
+  if (a.M == 16 && t.pairs && t.most > 2 * sms) return false;
+  if (a.M == 64 && t.lo >= 96 && t.most > sms) return true;
+  if (x3tf32) {
+    if (t.hi > 400) return t.shorter <= 8 * sms || t.lo >= 40;
+    if (t.lo >= 64 || (t.lo >= 40 && t.shorter <= 8 * sms)) return t.hi >= 152 || 2 * t.most <= sms;
+    return t.shorter <= sms && t.hi > 207;
+  }
+  if (t.hi < 152) return false;
+  if (t.hi > 432) return t.lo >= 32 && (!bf16 || a.nx < a.ny);
+  if (t.lo > 160) return !(t.pairs && t.most > sms && t.most <= 2 * sms);
+  if (a.nx < a.ny && t.hi > 256) return t.lo >= 56 || t.shorter <= sms;
+  if (bf16) return false;
+  if (a.M == 64) return t.lo >= 56;
+  return a.tc_mode == 2 && t.lo > kMT && t.hi >= 160 && t.most <= sms;
+}
+
+}  // namespace
+
 bool tc_march_supported(const StepArgs& a) {
-  // A grid of one tile per line has nothing to split over rows, and the two
-  // passes of rte_tc.cu, whose CTAs share an SM by twos, serve it better:
-  // 64^2, M = 32, four groups 25 us a step against 29 here, sixteen
-  // groups 36 against 45.
-  const bool rows = a.nx > kMT || a.ny > kMT;
-  return rows && a.tc_mode != 0 && a.tc_scatter == 0 && a.x_variant == 1;
+  if (a.tc_mode == 0 || a.tc_scatter != 0 || a.x_variant != 1 || (a.nx <= kMT && a.ny <= kMT)) return false;
+  return a.march_all || march_pays(a);
+}
+
+int tc_march_min_run(const StepArgs& a) {
+  // A launch's ramp is 6 to 40 us (its first x items and last y items by
+  // themselves).  A run of one step pays where a pass leaves half of the SMs
+  // idle anyway (256^2, one group, a snapshot at every step: 58 us a step
+  // against 90 in the passes) or the passes hold one CTA per SM (512^2, M =
+  // 64: 329 against 458); runs of two do in 3xTF32 (120 sizes: 1.23 of the
+  // passes' speed on average), in the other precisions those of four.
+  if (a.march_all) return 1;
+  const PassTiles t(a);
+  if (2 * t.most <= sm_count()) return 1;
+  if (a.tc_mode == 1) return t.pairs ? 2 : 1;
+  return t.pairs ? 4 : 2;
 }
 
 bool tc_march_dual(const StepArgs& a) {
