@@ -903,6 +903,16 @@ __global__ void __launch_bounds__(kBalThreads)
 
 }  // namespace
 
+int device_sms() {
+  static const int n = [] {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    return v > 0 ? v : 1;
+  }();
+  return n;
+}
+
 namespace {
 
 struct TilePlan {
@@ -922,13 +932,12 @@ struct TilePlan {
 // and 128 CTAs, 22 with 32 and 256), and otherwise in the narrowest of at
 // least four warps (64^2, M = 16, one group: 12.2 with 32, 13.3 with 64).
 TilePlan plan_tile(int n, int lines, int M, int G, bool xpass) {
-  constexpr int kSms = 152;
   TilePlan p{};
   const long long outputs = static_cast<long long>(n) * lines * M * G;
   auto tiles = [&](int per) { return (lines + per - 1) / per; };
   auto threads4 = [&](int per) { return simt_ld(n) / 4 * (per * M / 4); };
   int per = 1;
-  if (outputs >= 64LL * 256 * kSms || threads4(1) > kMaxThreads) {
+  if (outputs >= 64LL * 256 * device_sms() || threads4(1) > kMaxThreads) {
     p.T = 8;
     per = M < 32 ? 32 / M : 1;
   } else {
@@ -1061,7 +1070,7 @@ cudaError_t launch_grad_batch(const GradJob* jobs_dev, int n_jobs, int max_ncell
 }
 
 cudaError_t launch_save_batch(const SaveJob* jobs_dev, int n_jobs, int slot, cudaStream_t s, long long* launches) {
-  dim3 grid(4 * 152, n_jobs);
+  dim3 grid(4 * device_sms(), n_jobs);
   save_batch_kernel<<<grid, 256, 0, s>>>(jobs_dev, slot);
   if (launches) *launches += 1;
   return cudaGetLastError();

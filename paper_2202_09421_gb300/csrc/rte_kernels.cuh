@@ -10,6 +10,9 @@ constexpr int kKC = 16;
 __host__ __device__ constexpr int simt_ld(int n) { return (n + 15) / 16 * 16; }
 __host__ __device__ constexpr int simt_rows(int n) { return (n + kKC - 1) / kKC * kKC; }
 
+// SMs of the current device (one GPU per process).
+int device_sms();
+
 // Boundary/source description shared by the y-pass epilogue.
 struct BoundaryArgs {
   const int* face_refl;             // [4][M]

@@ -983,21 +983,6 @@ cudaError_t launch_march_p(const MarchArgs& ma, int sms, cudaStream_t s) {
   }
 }
 
-int sm_count() {
-  static int n = 0;                             // one GPU per process
-  if (n == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (n <= 0) n = 1;
-  }
-  return n;
-}
-
-}  // namespace
-
-namespace {
-
 // What a pass of all groups has to work off.
 struct PassTiles {
   long long most, shorter;           // slab tiles: of either pass at most, of the pass along the shorter axis
@@ -1031,7 +1016,7 @@ struct PassTiles {
 //   groups, TF32 51 against 69), geometric mean 0.97.
 bool march_pays(const StepArgs& a) {
   const PassTiles t(a);
-  const int sms = sm_count();
+  const int sms = device_sms();
   const bool x3tf32 = a.tc_mode == 1, bf16 = a.tc_mode == 4;
   if (a.M == 16 && t.pairs && t.most > 2 * sms) return false;
   if (a.M == 64 && t.lo >= 96 && t.most > sms) return true;
@@ -1065,7 +1050,7 @@ int tc_march_min_run(const StepArgs& a) {
   // passes' speed on average), in the other precisions those of four.
   if (a.march_all) return 1;
   const PassTiles t(a);
-  if (2 * t.most <= sm_count()) return 1;
+  if (2 * t.most <= device_sms()) return 1;
   if (a.tc_mode == 1) return t.pairs ? 2 : 1;
   return t.pairs ? 4 : 2;
 }
@@ -1077,13 +1062,13 @@ bool tc_march_dual(const StepArgs& a) {
   // against 134, two 188 against 208, four 302 against 316, eight 472 against
   // 448, sixteen 925 against 878 (twice the state between two uses in L2).
   const MarchItems it(a, 2, 0);
-  return a.G * static_cast<long long>(it.nxi > it.nyi ? it.nxi : it.nyi) < 2 * sm_count();
+  return a.G * static_cast<long long>(it.nxi > it.nyi ? it.nxi : it.nyi) < 2 * device_sms();
 }
 
 size_t tc_march_ctl_bytes(int G) { return (32 + 2 * static_cast<size_t>(G)) * sizeof(int); }
 
 cudaError_t launch_march_tc(MarchArgs ma, cudaStream_t s, long long* launches) {
-  const int sms = sm_count();
+  const int sms = device_sms();
   if (ma.dual) ma.a.G *= 2;
   // Row tiles per item: two output tiles share a conversion of the slab, one
   // makes twice the items.  One where a pass has no more items than SMs that

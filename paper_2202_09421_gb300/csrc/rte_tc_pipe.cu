@@ -28,7 +28,6 @@
 
 namespace rte_kern {
 
-
 namespace {
 
 using namespace tc;
@@ -417,17 +416,6 @@ __global__ void __launch_bounds__(kPipeThreads, 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * acc_cols));
 }
 
-int pipe_sm_count() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (n <= 0) n = 1;
-  }
-  return n;
-}
-
 template <int PREC, int MM>
 cudaError_t launch_pipe(const StepArgs& a, const BoundaryArgs& b, float* U, const float* R, const float* L1,
                         const float* L2, float* L3, int src_step, int ring_step, cudaStream_t s) {
@@ -447,7 +435,7 @@ cudaError_t launch_pipe(const StepArgs& a, const BoundaryArgs& b, float* U, cons
   }
   const int per_tile = kNC / MM;
   const int total = (a.nx + per_tile - 1) / per_tile * a.G;
-  const int grid = total < pipe_sm_count() ? total : pipe_sm_count();
+  const int grid = total < device_sms() ? total : device_sms();
   tc_ypass_pipe<PREC, MM><<<grid, kPipeThreads, smem, s>>>(a, b, U, R, L1, L2, L3, src_step, ring_step);
   return cudaGetLastError();
 }
@@ -475,6 +463,5 @@ cudaError_t launch_ypass_pipe(const StepArgs& a, const BoundaryArgs& b, float* U
     default: return launch_pipe_m<4>(a, b, U, R, L1, L2, L3, src_step, ring_step, s);
   }
 }
-
 
 }  // namespace rte_kern

@@ -34,7 +34,6 @@
 
 namespace rte_kern {
 
-
 namespace {
 
 using namespace tc;
@@ -488,17 +487,6 @@ __global__ void __launch_bounds__(kWsThreads, 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * acc_cols));
 }
 
-int sm_count() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    if (n <= 0) n = 1;
-  }
-  return n;
-}
-
 template <bool XPASS, int PREC, int MM>
 cudaError_t launch_ws(const StepArgs& a, const BoundaryArgs& b, float* U, float* R, const float* L1,
                       const float* L2, float* L3, int src_step, int ring_step, cudaStream_t s) {
@@ -520,7 +508,7 @@ cudaError_t launch_ws(const StepArgs& a, const BoundaryArgs& b, float* U, float*
   const int per_tile = kNC / MM;
   const int lines = XPASS ? a.ny : a.nx;
   const int total = (lines + per_tile - 1) / per_tile * a.G;
-  const int grid = total < sm_count() ? total : sm_count();
+  const int grid = total < device_sms() ? total : device_sms();
   tc_pass_ws<XPASS, PREC, MM><<<grid, kWsThreads, smem, s>>>(a, b, U, R, L1, L2, L3, src_step, ring_step);
   return cudaGetLastError();
 }
@@ -556,6 +544,5 @@ cudaError_t launch_pass_ws(bool xpass, const StepArgs& a, const BoundaryArgs& b,
   return xpass ? launch_ws_pass<true>(a, b, U, R, L1, L2, L3, src_step, ring_step, s)
                : launch_ws_pass<false>(a, b, U, R, L1, L2, L3, src_step, ring_step, s);
 }
-
 
 }  // namespace rte_kern
