@@ -895,6 +895,20 @@ bool tc_supported(int nx, int ny, int M, int precision, int flags) {
   return true;
 }
 
+// Whether the x-pass is launched as a dependent of the y-pass before it.  It
+// gains up to a fifth where launches count (32^2, one group 15.4 -> 13.0 us a
+// step; 64^2, 16 groups 37.0 -> 32.3; 128^2, 12 groups 83.5 -> 80.8) and
+// nothing, within 1 %, on large grids, but for many x tiles of two row tiles
+// whose MMAs are few (TF32, BF16): there the early CTAs stand where the last
+// ones of the y-pass could work off faster (160^2, M = 32, 16 groups, TF32
+// 146.1 -> 149.3; 256^2, 8 groups, BF16 159.7 -> 162.6; in 3xTF32 176.7 ->
+// 174.7 and 193.8 -> 192.3).
+static bool xpass_dependent(const StepArgs& a) {
+  const int per_tile = kNC / a.M;
+  const long long tiles = static_cast<long long>(a.G) * ((a.ny + per_tile - 1) / per_tile);
+  return a.tc_mode == 1 || a.M == 64 || a.nx <= kMT || a.nx > 2 * kMT || tiles <= 2 * device_sms();
+}
+
 cudaError_t launch_step_tc(const StepArgs& a, const BoundaryArgs& b, float* U, float* R, const float* L1,
                            const float* L2, float* L3, int step, cudaStream_t s, long long* launches,
                            cudaEvent_t* ev) {
@@ -911,7 +925,7 @@ cudaError_t launch_step_tc(const StepArgs& a, const BoundaryArgs& b, float* U, f
   const bool ystream = tma && a.x_variant == 5 && tc_ystream_supported(a);
   e = ws       ? launch_pass_ws(true, a, b, U, R, L1, L2, L3, step, ring_step, s)
       : stream ? launch_xpass_stream(a, b, U, R, s)
-               : launch_mode<true>(a, b, U, R, L1, L2, L3, step, ring_step, s, !ev);
+               : launch_mode<true>(a, b, U, R, L1, L2, L3, step, ring_step, s, !ev && xpass_dependent(a));
   if (e != cudaSuccess) return e;
   if (ev) cudaEventRecord(ev[1], s);
   e = ws        ? launch_pass_ws(false, a, b, U, R, L1, L2, L3, step, ring_step, s)
