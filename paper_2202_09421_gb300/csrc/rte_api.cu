@@ -2,9 +2,11 @@
 // time-march driver, detector readout and the checkpointed adjoint gradient.
 #include <algorithm>
 #include <atomic>
+#include <chrono>
 #include <cstdint>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <utility>
 #include <vector>
@@ -51,8 +53,11 @@ struct rte_ctx {
   // and the test-only request that the next march's first pass time out
   DevBuf err;
   bool inject_expire = false;
-  // item counters of the multi-step launches
+  // item counters of the multi-step launches, and the events that keep the
+  // host at most two launches ahead (Pace)
   DevBuf ctl;
+  cudaEvent_t pace[2] = {nullptr, nullptr};
+  cudaEvent_t fp32_end = nullptr;  // behind the last FP32 forward (Marching)
   // photon balance of the last rte_forward (RTE_FLAG_PHOTON_BALANCE):
   // [G][n_steps][3] FP64 terms, block partials, per-group tickets, and the
   // FP64 cos / sin of the ordinates
@@ -183,6 +188,7 @@ rte_kern::StepArgs step_args(rte_ctx* c, int G) {
   a.tc_scatter = (c->par.flags & RTE_FLAG_TC_SCATTER) ? 1 : 0;
   a.x_variant = c->x_variant;
   a.march_all = c->march_all ? 1 : 0;
+  a.beside = 0;
   a.DxImg = c->DxImg.p;
   a.DyImg = c->DyImg.p;
   a.PImg = F(c->PImg);
@@ -281,29 +287,127 @@ rte_status snapshot(rte_ctx* c, const float* u, int G, const std::vector<int>& s
                                               static_cast<float>(2.0 * kPi / c->M), c->stream, &c->launches));
 }
 
-// Steps of a multi-step launch, at most: 36 ms at 16 groups of 256^2, so that
-// work on other streams gets its turn (a launch costs about 0.1 ms of ramp).
-constexpr int kMarchSteps = 128;
-// The same with the photon balance of every step: the states of the last two
-// steps of a launch are in U and R.
+// Marches of this process that may be on the GPU side by side.  A multi-step
+// launch keeps every SM, so solves of several streams that take them follow
+// one another, while the two passes a step of several small solves fill the
+// SMs together (256^2, one group, 3xTF32, on one, two, four, eight streams:
+// 79, 92, 107, 158 us for a step of all in the passes, 46, 90, 179, 357 in
+// multi-step launches).  So a march takes them, run by run, while no other
+// stream has a march under way, nor had one lately (threads that solve again
+// and again are each alone for a moment now and then), and the passes
+// otherwise, unless it fills the SMs by itself (tc_march_shares).  Calls in
+// progress are known by their streams; an FP32 forward returns before its
+// work is done and leaves an event behind it.
+constexpr std::chrono::milliseconds kLately{50};
+struct Marches {
+  using Clock = std::chrono::steady_clock;
+  std::mutex lock;
+  Clock::time_point together = Clock::now() - 2 * kLately;   // two streams were last seen marching
+  std::vector<cudaStream_t> calls;                           // one entry per call in progress
+  std::vector<std::pair<cudaEvent_t, cudaStream_t>> fp32;    // one entry per FP32 context that has marched
+};
+Marches& marches() {
+  static Marches* const all = new Marches;                   // contexts may be destroyed after static objects
+  return *all;
+}
+
+// A call that marches on stream s, from its construction on.
+class Marching {
+ public:
+  explicit Marching(cudaStream_t s) : stream_(s) {
+    std::lock_guard<std::mutex> hold(marches().lock);
+    marches().calls.push_back(s);
+    if (beside()) marches().together = Marches::Clock::now();
+  }
+  ~Marching() {
+    std::lock_guard<std::mutex> hold(marches().lock);
+    std::vector<cudaStream_t>& c = marches().calls;
+    c.erase(std::find(c.begin(), c.end(), stream_));
+  }
+  Marching(const Marching&) = delete;
+  Marching& operator=(const Marching&) = delete;
+  bool alone() const {
+    std::lock_guard<std::mutex> hold(marches().lock);
+    const auto now = Marches::Clock::now();
+    if (beside()) marches().together = now;
+    return now - marches().together > kLately;
+  }
+
+ private:
+  bool beside() const {                                      // the lock is held
+    for (cudaStream_t s : marches().calls)
+      if (s != stream_) return true;
+    for (const auto& e : marches().fp32)
+      if (e.second != stream_ && cudaEventQuery(e.first) == cudaErrorNotReady) {
+        cudaGetLastError();
+        return true;
+      }
+    return false;
+  }
+  cudaStream_t stream_;
+};
+
+// Leaves the event behind an FP32 forward of context c.
+rte_status mark_fp32_end(rte_ctx* c) {
+  if (!c->fp32_end) {
+    RTE_TRY(cuda_status(cudaEventCreateWithFlags(&c->fp32_end, cudaEventDisableTiming)));
+    RTE_TRY(cuda_status(cudaEventRecord(c->fp32_end, c->stream)));
+    std::lock_guard<std::mutex> hold(marches().lock);
+    marches().fp32.emplace_back(c->fp32_end, c->stream);
+    return RTE_OK;
+  }
+  return cuda_status(cudaEventRecord(c->fp32_end, c->stream));
+}
+
+// Steps of a multi-step launch, at most: 4.4 ms at 16 groups of 256^2, 1.4 ms
+// at one, so that other work gets its turn and a march learns soon that it is
+// no longer alone.  The ramp of a launch costs little of that: 256^2, 16
+// groups 276.3 us a step in launches of 128 steps, 277.9 of 16, 283.9 of 4;
+// one group 44.1, 44.9, 45.1; 200 x 131, three groups 43.3, 44.3, 49.1.
+int march_limit(const rte_kern::StepArgs& a) {
+  const long long values = static_cast<long long>(a.G) * static_cast<long long>(a.plane);
+  return static_cast<int>(std::max<long long>(2, std::min<long long>(32, (1LL << 29) / values)));
+}
+
+// Keeps the host at most two launches of `limit` steps ahead of the GPU, so
+// that the choice between launches and passes is made near the time it is for.
+class Pace {
+ public:
+  Pace(rte_ctx* c, int limit) : c_(c), limit_(limit) {}
+  rte_status after(int steps) {
+    if ((steps_ += steps) < limit_) return RTE_OK;
+    steps_ = 0;
+    for (cudaEvent_t& e : c_->pace)
+      if (!e) RTE_TRY(cuda_status(cudaEventCreateWithFlags(&e, cudaEventDisableTiming)));
+    RTE_TRY(cuda_status(cudaEventRecord(c_->pace[n_ & 1], c_->stream)));
+    if (n_++ > 0) RTE_TRY(cuda_status(cudaEventSynchronize(c_->pace[n_ & 1])));
+    return RTE_OK;
+  }
+
+ private:
+  rte_ctx* c_;
+  int limit_, steps_ = 0, n_ = 0;
+};
+
+// Steps of a launch with the photon balance of every step: the states of the
+// last two are in U and R.
 constexpr int kBalanceSteps = 2;
-// The same for the adjoint beside a recompute: the adjoint levels of a launch
-// are kept for its gradient terms.
-constexpr int kDualSteps = 32;
-// Checkpoint interval from which the two march side by side (a launch takes at
-// most half of it; 256^2, two groups, single passes on two streams against
+// Checkpoint interval from which an adjoint and a recompute march side by side
+// (a launch takes at most half of it; 256^2, two groups, single passes on two streams against
 // them: an interval of 3 226 us against 241, of 5 218 against 216, of 6 217
 // against 205, of 20 222 against 193).
 constexpr int kDualInterval = 6;
 
 // Runs steps [s_begin, s_end) of the forward march on (U, R, L), starting
 // from whatever state they hold; records checkpoints/exitance/fluence when
-// asked.
+// asked.  Whether other marches are under way is asked run by run of `live`,
+// or, without it (a graph's capture), told by `beside`.
 rte_status march(rte_ctx* c, DevBuf& U, DevBuf& R, DevBuf* L, int& hl, int G, int s_begin,
                  int s_end, const rte_kern::BoundaryArgs& b, bool save_ckpt,
                  const std::vector<int>& snap_index, float* fluence_out,
-                 std::vector<float*>* seg_out, double* balance_out = nullptr) {
-  const rte_kern::StepArgs a = step_args(c, G);
+                 std::vector<float*>* seg_out, const Marching* live, bool beside = false,
+                 double* balance_out = nullptr) {
+  rte_kern::StepArgs a = step_args(c, G);
   const size_t gbytes = static_cast<size_t>(G) * c->plane * sizeof(float);
   const int I = c->par.ckpt_interval;
   // The tile-local fused step reads u^k from one buffer and writes u^{k+1}
@@ -317,7 +421,10 @@ rte_status march(rte_ctx* c, DevBuf& U, DevBuf& R, DevBuf* L, int& hl, int G, in
   // nothing to overlap with the passes of the other stream.
   const bool overlapped = c->astream && c->stream == c->astream;
   const bool marched = !fused && !c->timing && !overlapped && rte_kern::tc_march_supported(a);
-  const int longest = balance_out ? kBalanceSteps : kMarchSteps;
+  const bool shares = marched && rte_kern::tc_march_shares(a);
+  a.beside = beside;
+  const int limit = march_limit(a), longest = balance_out ? std::min(limit, kBalanceSteps) : limit;
+  Pace pace(c, limit);
   const int shortest = marched ? rte_kern::tc_march_min_run(a) : 0;
   auto run_end = [&](int s) {                          // the run [s, e)
     int e = s + 1;
@@ -404,12 +511,14 @@ rte_status march(rte_ctx* c, DevBuf& U, DevBuf& R, DevBuf* L, int& hl, int G, in
   for (int s = s_begin, e; s < s_end; s = e) {
     if (save_ckpt && I > 0 && s % I == 0) RTE_TRY(copy_checkpoint(c, cur, L, hl, G, s));
     e = run_end(s);
-    if (marched && e - s >= shortest) {
+    if (live && (marched || (s - s_begin) % limit == 0)) a.beside = !live->alone();
+    if (marched && e - s >= shortest && (shares || !a.beside)) {
       RTE_TRY(march_run(s, e));
     } else {
       for (int q = s; q < e; ++q) RTE_TRY(pass_step(q));
     }
     if (fluence_out && snap_index[e - 1] >= 0) RTE_TRY(snapshot(c, cur, G, snap_index, e - 1, fluence_out));
+    if (marched && live) RTE_TRY(pace.after(e - s));
   }
   if (cur != F(U) && !(seg_out && marched))
     RTE_TRY(cuda_status(cudaMemcpyAsync(U.p, cur, gbytes, cudaMemcpyDeviceToDevice, c->stream)));
@@ -845,6 +954,16 @@ rte_status rte_destroy(rte_ctx* c) {
   }
   for (cudaEvent_t e : c->aev)
     if (e) cudaEventDestroy(e);
+  for (cudaEvent_t e : c->pace)
+    if (e) cudaEventDestroy(e);
+  if (c->fp32_end) {
+    {
+      std::lock_guard<std::mutex> hold(marches().lock);
+      auto& ends = marches().fp32;
+      ends.erase(std::find_if(ends.begin(), ends.end(), [&](const auto& e) { return e.first == c->fp32_end; }));
+    }
+    cudaEventDestroy(c->fp32_end);
+  }
   if (c->astream) {
     cudaStreamSynchronize(c->astream);
     cudaStreamDestroy(c->astream);
@@ -1020,6 +1139,7 @@ rte_status rte_forward(rte_ctx* c, const rte_source_group* groups, int n_groups,
       return RTE_ERR_INVALID_ARG;
     snap_index[snap_steps[k]] = k;
   }
+  const Marching live(c->stream);
   RTE_TRY(prepare_forward(c, groups, n_groups, n_steps));
   double* balance = nullptr;
   if (c->par.flags & RTE_FLAG_PHOTON_BALANCE) {
@@ -1038,11 +1158,17 @@ rte_status rte_forward(rte_ctx* c, const rte_source_group* groups, int n_groups,
   key.push_back(key_ptr(balance));
   key.push_back(key_ptr(c->bal_partial.p));
   for (int k = 0; k < n_snaps; ++k) key.push_back(static_cast<unsigned long long>(snap_steps[k]));
+  // a graph goes by what is under way at the call; the plain FP32 form, whose
+  // launches do not depend on it, does not ask
+  const bool graph = (c->par.flags & RTE_FLAG_CUDA_GRAPH) && !c->timing;
+  const bool beside = graph && c->tc_mode != 0 && !live.alone();
+  key.push_back(beside);
   RTE_TRY(run_march(c, key, [&]() {
     int hl = 0;
     return march(c, c->U, c->R, c->L, hl, c->G, 0, n_steps, b, true, snap_index, fluence_out, nullptr,
-                 balance);
+                 graph || c->tc_mode == 0 ? nullptr : &live, beside, balance);
   }));
+  if (c->tc_mode == 0) RTE_TRY(mark_fp32_end(c));
   c->hl = (2 * n_steps) % 3;
   const rte_status st = tc_check(c);
   if (st == RTE_OK && balance) c->bal_valid = true;
@@ -1062,6 +1188,7 @@ rte_status rte_forward_batch(rte_ctx* const* ctxs, int n_ctx, const rte_source_g
     for (int k = 0; k < i; ++k)
       if (ctxs[k] == c) return RTE_ERR_INVALID_ARG;
   }
+  const Marching live(c0->stream);
   for (int i = 0; i < n_ctx; ++i) RTE_TRY(prepare_forward(ctxs[i], groups[i], n_groups[i], n_steps));
   std::vector<unsigned long long> key{static_cast<unsigned long long>(n_ctx)};
   for (int i = 0; i < n_ctx; ++i) {
@@ -1081,12 +1208,13 @@ rte_status rte_forward_batch(rte_ctx* const* ctxs, int n_ctx, const rte_source_g
           const cudaStream_t keep = c->stream;
           c->stream = c0->stream;              // the capture stream while a graph is recorded
           const rte_status st = march(c, c->U, c->R, c->L, hl[i], c->G, s, s + 1, bargs[i], true, no_snaps,
-                                      nullptr, nullptr);
+                                      nullptr, nullptr, nullptr);
           c->stream = keep;
           if (st != RTE_OK) return st;
         }
       return RTE_OK;
     }));
+    RTE_TRY(mark_fp32_end(c0));
   } else {
     // Tensor-core form: one x-pass and one y-pass launch per step over the
     // tiles of every medium, the media with the longest lines first.
@@ -1105,6 +1233,9 @@ rte_status rte_forward_batch(rte_ctx* const* ctxs, int n_ctx, const rte_source_g
       P.R = F(c->R);
       for (int q = 0; q < 3; ++q) P.L[q] = F(c->L[q]);
     }
+    const bool beside = !live.alone();
+    for (rte_kern::BatchProblem& P : tab) P.a.beside = beside;
+    key.push_back(beside);
     int ctas_x = 0, ctas_y = 0;
     rte_kern::tc_batch_layout(tab.data(), n_ctx, &ctas_x, &ctas_y);
     RTE_TRY(upload(c0->batch_tab, tab, c0->stream));
@@ -1206,6 +1337,7 @@ static rte_status adjoint_impl(rte_ctx* c, const rte_detector* dets, int n_det, 
   if (c->n_steps <= 0 || c->par.ckpt_interval <= 0) return RTE_ERR_STATE;
   for (int d = 0; d < n_det; ++d)
     if (!(dets[d].sigma_d > 0)) return RTE_ERR_INVALID_ARG;
+  const Marching live(c->stream);
   if (discrete) RTE_TRY(ensure_transposed(c));
   const int G = c->G, N = c->n_steps, I = c->par.ckpt_interval;
   const size_t gfloats = static_cast<size_t>(G) * c->plane, gbytes = gfloats * sizeof(float);
@@ -1276,16 +1408,23 @@ static rte_status adjoint_impl(rte_ctx* c, const rte_detector* dets, int n_det, 
   std::vector<int> no_snaps(N, -1);
   // Continuous form with multi-step launches, all on the context's stream.
   // With few groups (tc_march_dual) the adjoint levels of a segment march
-  // beside the recompute of the next one, in launches of up to kDualSteps
-  // levels of both, each followed by its gradient terms.  With more groups,
+  // beside the recompute of the next one, in launches of at most half a
+  // segment of both, each followed by its gradient terms.  With more groups,
   // recompute, adjoint and gradient of a segment follow one another, with the
   // adjoint levels in the second segment buffer.  Short segments take single
   // passes on two streams.
-  const bool few = rte_kern::tc_march_dual(sa);
-  const bool marched =
-      !discrete && !fused_adj && !c->timing && rte_kern::tc_march_supported(sa) && I >= (few ? kDualInterval : 2);
+  // They go by the other marches under way: beside others the call takes
+  // single passes on two streams from the start, or single passes in turn for
+  // the levels during which another one came.
+  const bool few = rte_kern::tc_march_dual(sa), shares = rte_kern::tc_march_shares(sa);
+  sa.beside = c->tc_mode != 0 && !live.alone();
+  const bool marched = !discrete && !fused_adj && !c->timing && rte_kern::tc_march_supported(sa) &&
+                       I >= (few ? kDualInterval : 2) && (shares || !sa.beside);
   const bool dual = marched && few;
-  const int chunk = std::min(I / 2, kDualSteps);
+  rte_kern::StepArgs s2 = sa;
+  if (dual) s2.G *= 2;
+  const int limit = march_limit(s2), chunk = dual ? std::min(I / 2, limit) : limit;
+  Pace pace(c, limit);
   // Levels needed: forward steps 0 .. N-2 (the adjoint vanishes at the last).
   const int last = N - 2;
   // Segments in reverse order.  The forward recompute of a segment (second
@@ -1328,7 +1467,7 @@ static rte_status adjoint_impl(rte_ctx* c, const rte_detector* dets, int n_det, 
     rte_status st = restore(seg);
     int hl = 0;
     std::vector<float*> segp = seg_ptrs(k, s0, s_end);
-    if (st == RTE_OK) st = march(c, c->U, c->R, c->L, hl, G, s0, s_end, bf, false, no_snaps, nullptr, &segp);
+    if (st == RTE_OK) st = march(c, c->U, c->R, c->L, hl, G, s0, s_end, bf, false, no_snaps, nullptr, &segp, &live);
     if (st == RTE_OK) st = cuda_status(cudaEventRecord(done_fwd[k % 2], c->stream));
     c->stream = keep;
     c->timing = keep_timing;
@@ -1345,103 +1484,102 @@ static rte_status adjoint_impl(rte_ctx* c, const rte_detector* dets, int n_det, 
   for (size_t k = 0; k < segs.size(); ++k) {
     const int seg = segs[k];
     const int s0 = seg * I, s_end = std::min(s0 + I, last + 1);
-    if (dual) {
-      const bool more = k + 1 < segs.size();
-      const int t0 = more ? segs[k + 1] * I : 0, n = s_end - s0, n2 = more ? std::min(t0 + I, last + 1) - t0 : 0;
-      if (more) RTE_TRY(restore(segs[k + 1]));
-      float* fwd = F(c->seg) + static_cast<size_t>(k % 2) * I * gfloats;          // this segment's levels
-      float* nxt = F(c->seg) + static_cast<size_t>((k + 1) % 2) * I * gfloats;    // the next one's
-      const long long step = static_cast<long long>(gfloats);
-      int hl_fwd = 0;
-      for (int d = 0, d2 = 0; d < n || d2 < n2;) {
-        rte_kern::MarchArgs ma{};
-        ma.a = sa;
-        ma.ctl = static_cast<int*>(c->ctl.p);
-        // adjoint levels s_end - 1 - d .., recomputed levels t0 + d2 ..
-        rte_kern::MarchSide adj{}, rec{};
-        adj.b = ba;
-        adj.u0 = adj.u1 = mcur;
-        adj.hl = hl_adj;
-        adj.step0 = s_end - 1 - d;
-        adj.dstep = -1;
-        rec.b = bf;
-        rec.slots = nxt + static_cast<size_t>(d2) * gfloats;
-        rec.u0 = rec.u1 = d2 == 0 ? F(c->U) : rec.slots - gfloats;
-        rec.hl = hl_fwd;
-        rec.step0 = t0 + d2;
-        rec.dstep = 1;
-        adj.slot_floats = rec.slot_floats = gfloats;
-        for (int q = 0; q < 3; ++q) {
-          adj.L[q] = F(c->LA[q]);
-          rec.L[q] = F(c->L[q]);
-        }
-        const bool has_adj = d < n, has_rec = d2 < n2;
-        ma.n_steps = std::min(has_adj ? std::min(chunk, n - d) : kMarchSteps, has_rec ? n2 - d2 : n);
-        // The adjoint levels go where no forward level is kept: the first
-        // launch's at the end of the next segment's half, of which it writes
-        // no more than the first half, the others' over levels of this segment
-        // whose gradient terms are formed.
-        if (has_adj && d > 0) ma.n_steps = std::min(ma.n_steps, d);
-        adj.slots = d == 0 ? nxt + static_cast<size_t>(I - ma.n_steps) * gfloats : fwd + static_cast<size_t>(n - d) * gfloats;
-        ma.dual = has_adj && has_rec ? 1 : 0;
-        const rte_kern::MarchSide& one = has_adj ? adj : rec;
-        ma.b = one.b;
-        ma.u0 = one.u0;
-        ma.u1 = one.u1;
-        ma.slots = one.slots;
-        ma.slot_floats = gfloats;
-        for (int q = 0; q < 3; ++q) ma.L[q] = one.L[q];
-        ma.hl = one.hl;
-        ma.step0 = one.step0;
-        ma.dstep = one.dstep;
-        ma.two = rec;
-        RTE_TRY(cuda_status(rte_kern::launch_march_tc(ma, c->stream, &c->launches)));
-        const int m = ma.n_steps;
-        if (has_rec) {
-          hl_fwd = (hl_fwd + 2 * m) % 3;
-          d2 += m;
-        }
-        if (!has_adj) continue;
-        hl_adj = (hl_adj + 2 * m) % 3;
-        // slot l of the launch is level s_end - 1 - d - l
-        RTE_TRY(cuda_status(rte_kern::launch_grad(
-            adj.slots, fwd + static_cast<size_t>(n - 1 - d) * gfloats, F(c->PT), F(c->area), c->nx, c->ny, c->M, G,
-            c->plane, c->plane, scale, 1, {m, step, -step}, dJ_dmua ? D(c->grad_a) : nullptr,
-            dJ_dmus ? D(c->grad_b) : nullptr, c->stream, &c->launches)));
-        RTE_TRY(cuda_status(cudaMemcpyAsync(mcur, adj.slots + static_cast<size_t>(m - 1) * gfloats, gbytes,
-                                            cudaMemcpyDeviceToDevice, c->stream)));
-        d += m;
-      }
-      continue;
-    }
     if (marched) {
-      const int n = s_end - s0;
-      RTE_TRY(recompute(static_cast<int>(k)));
-      rte_kern::MarchArgs ma{};
-      ma.a = sa;
-      ma.b = ba;
-      for (int q = 0; q < 3; ++q) ma.L[q] = F(c->LA[q]);
-      ma.dstep = -1;
-      ma.ctl = static_cast<int*>(c->ctl.p);
-      ma.slot_floats = gfloats;
-      float* mslots = F(c->seg) + static_cast<size_t>(I) * gfloats;
-      for (int o = 0; o < n; o += kMarchSteps) {
-        ma.slots = mslots + static_cast<size_t>(o) * gfloats;
-        ma.u0 = ma.u1 = o == 0 ? mcur : ma.slots - gfloats;
-        ma.hl = hl_adj;
-        ma.step0 = s_end - 1 - o;
-        ma.n_steps = std::min(kMarchSteps, n - o);
-        RTE_TRY(cuda_status(rte_kern::launch_march_tc(ma, c->stream, &c->launches)));
-        hl_adj = (hl_adj + 2 * ma.n_steps) % 3;
-      }
-      // adjoint slot l is level s_end - 1 - l
+      const bool more = dual && k + 1 < segs.size();
+      const int t0 = more ? segs[k + 1] * I : 0, n = s_end - s0, n2 = more ? std::min(t0 + I, last + 1) - t0 : 0;
+      if (!dual) RTE_TRY(recompute(static_cast<int>(k)));
+      if (more) RTE_TRY(restore(segs[k + 1]));
+      float* fwd = F(c->seg) + (dual ? static_cast<size_t>(k % 2) * I * gfloats : 0);   // this segment's levels
+      // the next one's (dual), or the adjoint levels of this one
+      float* nxt = F(c->seg) + (dual ? static_cast<size_t>((k + 1) % 2) : 1) * I * gfloats;
       const long long step = static_cast<long long>(gfloats);
-      RTE_TRY(cuda_status(rte_kern::launch_grad(
-          mslots, seg_ptrs(static_cast<int>(k), s0, s_end)[n - 1], F(c->PT), F(c->area), c->nx, c->ny, c->M, G,
-          c->plane, c->plane, scale, 1, {n, step, -step}, dJ_dmua ? D(c->grad_a) : nullptr,
-          dJ_dmus ? D(c->grad_b) : nullptr, c->stream, &c->launches)));
-      RTE_TRY(cuda_status(cudaMemcpyAsync(mcur, mslots + static_cast<size_t>(n - 1) * gfloats, gbytes,
-                                          cudaMemcpyDeviceToDevice, c->stream)));
+      float* rcur = F(c->U);                             // state of the recompute
+      int hl_fwd = 0;
+      for (int d = 0, d2 = 0, m; d < n || d2 < n2;) {
+        // adjoint levels s_end - 1 - d .., recomputed levels t0 + d2 ..
+        const bool has_adj = d < n, has_rec = d2 < n2;
+        float* gradient_of = F(c->MU);                   // the first of this turn's adjoint levels
+        sa.beside = !live.alone();
+        if (!shares && sa.beside) {
+          m = 1;
+          DevBuf* H = has_adj ? c->LA : c->L;
+          int& h = has_adj ? hl_adj : hl_fwd;
+          if (!has_adj && rcur != F(c->U))
+            RTE_TRY(cuda_status(cudaMemcpyAsync(c->U.p, rcur, gbytes, cudaMemcpyDeviceToDevice, c->stream)));
+          RTE_TRY(cuda_status(rte_kern::launch_step(
+              sa, has_adj ? ba : bf, has_adj ? F(c->MU) : F(c->U), has_adj ? F(c->RA) : F(c->R), F(H[h]),
+              F(H[(h + 1) % 3]), F(H[(h + 2) % 3]), has_adj ? s_end - 1 - d : t0 + d2, c->stream, &c->launches)));
+          h = (h + 2) % 3;
+          if (!has_adj) {
+            rcur = F(c->U);
+            RTE_TRY(cuda_status(cudaMemcpyAsync(nxt + static_cast<size_t>(d2++) * gfloats, rcur, gbytes,
+                                                cudaMemcpyDeviceToDevice, c->stream)));
+          }
+        } else {
+          m = std::min(has_adj ? std::min(chunk, n - d) : limit, has_rec ? n2 - d2 : n);
+          // With a recompute the adjoint levels go where no forward level is
+          // kept: the first launch's at the end of the next segment's half, of
+          // which it writes no more than the first half, the others' over
+          // levels of this segment whose gradient terms are formed.
+          if (dual && has_adj && d > 0) m = std::min(m, d);
+          rte_kern::MarchSide adj{}, rec{};
+          adj.b = ba;
+          adj.u0 = adj.u1 = F(c->MU);
+          adj.slots = !dual   ? nxt + static_cast<size_t>(d) * gfloats
+                      : d == 0 ? nxt + static_cast<size_t>(I - m) * gfloats
+                               : fwd + static_cast<size_t>(n - d) * gfloats;
+          adj.hl = hl_adj;
+          adj.step0 = s_end - 1 - d;
+          adj.dstep = -1;
+          rec.b = bf;
+          rec.slots = nxt + static_cast<size_t>(d2) * gfloats;
+          rec.u0 = rec.u1 = rcur;
+          rec.hl = hl_fwd;
+          rec.step0 = t0 + d2;
+          rec.dstep = 1;
+          adj.slot_floats = rec.slot_floats = gfloats;
+          for (int q = 0; q < 3; ++q) {
+            adj.L[q] = F(c->LA[q]);
+            rec.L[q] = F(c->L[q]);
+          }
+          rte_kern::MarchArgs ma{};
+          ma.a = sa;
+          ma.ctl = static_cast<int*>(c->ctl.p);
+          ma.n_steps = m;
+          ma.dual = has_adj && has_rec ? 1 : 0;
+          const rte_kern::MarchSide& one = has_adj ? adj : rec;
+          ma.b = one.b;
+          ma.u0 = one.u0;
+          ma.u1 = one.u1;
+          ma.slots = one.slots;
+          ma.slot_floats = gfloats;
+          for (int q = 0; q < 3; ++q) ma.L[q] = one.L[q];
+          ma.hl = one.hl;
+          ma.step0 = one.step0;
+          ma.dstep = one.dstep;
+          ma.two = rec;
+          RTE_TRY(cuda_status(rte_kern::launch_march_tc(ma, c->stream, &c->launches)));
+          if (has_rec) {
+            hl_fwd = (hl_fwd + 2 * m) % 3;
+            d2 += m;
+            rcur = nxt + static_cast<size_t>(d2 - 1) * gfloats;
+          }
+          if (has_adj) hl_adj = (hl_adj + 2 * m) % 3;
+          gradient_of = adj.slots;
+        }
+        if (has_adj) {
+          // adjoint level l of this turn is forward level s_end - 1 - d - l
+          RTE_TRY(cuda_status(rte_kern::launch_grad(
+              gradient_of, fwd + static_cast<size_t>(n - 1 - d) * gfloats, F(c->PT), F(c->area), c->nx, c->ny, c->M, G,
+              c->plane, c->plane, scale, 1, {m, step, -step}, dJ_dmua ? D(c->grad_a) : nullptr,
+              dJ_dmus ? D(c->grad_b) : nullptr, c->stream, &c->launches)));
+          if (gradient_of != F(c->MU))
+            RTE_TRY(cuda_status(cudaMemcpyAsync(c->MU.p, gradient_of + static_cast<size_t>(m - 1) * gfloats, gbytes,
+                                                cudaMemcpyDeviceToDevice, c->stream)));
+          d += m;
+        }
+        RTE_TRY(pace.after(m));
+      }
       continue;
     }
     // next segment's recompute may start once the adjoint that read its
@@ -1532,6 +1670,7 @@ rte_status rte_adjoint_gradient_batch(rte_ctx* const* ctxs, int n_ctx, const rte
                            dJ_dmus ? dJ_dmus[i] : nullptr, false));
     return RTE_OK;
   }
+  const Marching live(c0->stream);
   const int N = c0->n_steps, I = c0->par.ckpt_interval;
   const cudaStream_t st = c0->stream;
   // Per medium: detector curves, objective, adjoint boundary data rho of eq.
@@ -1626,6 +1765,8 @@ rte_status rte_adjoint_gradient_batch(rte_ctx* const* ctxs, int n_ctx, const rte
     for (int q = 0; q < 3; ++q) Q.L[q] = F(c->LA[q]);
   }
   int cx = 0, cy = 0;
+  const bool beside = !live.alone();
+  for (int r = 0; r < n_ctx; ++r) tf[r].a.beside = ta[r].a.beside = beside;
   rte_kern::tc_batch_layout(tf.data(), n_ctx, &cx, &cy);
   rte_kern::tc_batch_layout(ta.data(), n_ctx, &cx, &cy);
   RTE_TRY(upload(c0->batch_tab, tf, st));
@@ -1738,8 +1879,6 @@ rte_status rte_adjoint_gradient_batch(rte_ctx* const* ctxs, int n_ctx, const rte
 // needs first; calls that overlap on the GPU (other streams, other threads,
 // other contexts on the same device) race on it.
 // ---------------------------------------------------------------------------
-#include <mutex>
-
 namespace {
 
 constexpr size_t kStaticScratchBytes = 64ull << 20;
@@ -1810,6 +1949,7 @@ extern "C" rte_status rte_forward_static(rte_ctx* c, const rte_source_group* gro
   const size_t need = 5 * gbytes + ring_b + S_b + A_b + T_b + W_b + lh_b;
   if (need > kStaticScratchBytes) return RTE_ERR_UNSUPPORTED;
 
+  const Marching live(c->stream);
   void* base = nullptr;
   RTE_TRY(static_scratch_address(&base));
   char* p = static_cast<char*>(base);

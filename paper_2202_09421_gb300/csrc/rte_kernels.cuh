@@ -66,6 +66,7 @@ struct StepArgs {
   int x_variant;                    // 0 persistent warp-specialised passes, 1 one tile per CTA, 2 pipelined y-pass,
                                     // 3 tile-local fused step, 4 TMA-fed persistent x-pass + one-tile y-pass,
                                     // 5 TMA-fed persistent x- and y-passes
+  int beside;                       // marches on other streams are under way
   int march_all;                    // multi-step launches wherever supported, not only where they are faster
   const void* DxImg;
   const void* DyImg;
@@ -173,6 +174,8 @@ struct MarchArgs {
 // Whether steps take this form, and the shortest run of steps that does.
 bool tc_march_supported(const StepArgs& a);
 int tc_march_min_run(const StepArgs& a);
+// Whether it is the faster form beside other marches too.
+bool tc_march_shares(const StepArgs& a);
 // Whether two marches of a.G groups are faster side by side than in turn.
 bool tc_march_dual(const StepArgs& a);
 size_t tc_march_ctl_bytes(int G);

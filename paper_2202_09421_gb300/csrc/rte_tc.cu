@@ -830,7 +830,7 @@ cudaError_t launch_batched_one(const BatchProblem* probs, const BatchProblem* de
   attr_pdl[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr_pdl[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr_pdl;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = XPASS && probs[0].a.beside && 3 * ctas > device_sms() ? 0 : 1;   // as xpass_dependent
   return cudaLaunchKernelEx(&cfg, tc_pass_batched<XPASS, PREC, MM, SCAT_TC>, dev, n, step, hl);
 }
 
@@ -902,10 +902,15 @@ bool tc_supported(int nx, int ny, int M, int precision, int flags) {
 // whose MMAs are few (TF32, BF16): there the early CTAs stand where the last
 // ones of the y-pass could work off faster (160^2, M = 32, 16 groups, TF32
 // 146.1 -> 149.3; 256^2, 8 groups, BF16 159.7 -> 162.6; in 3xTF32 176.7 ->
-// 174.7 and 193.8 -> 192.3).
+// 174.7 and 193.8 -> 192.3).  Beside other marches the early CTAs stand in the
+// way of those, unless they are few (four solves on streams of their own,
+// 3xTF32: 64^2, M = 16, one group 27.6 us a step as an ordinary launch, 24.0
+// as a dependent one, 128^2, M = 32 49.2 and 46.5; but 64^2, M = 32, four
+// groups 34.6 and 36.3, 24 x 256, M = 16, eight groups 74.5 and 97.1).
 static bool xpass_dependent(const StepArgs& a) {
   const int per_tile = kNC / a.M;
   const long long tiles = static_cast<long long>(a.G) * ((a.ny + per_tile - 1) / per_tile);
+  if (a.beside) return 3 * tiles <= device_sms();
   return a.tc_mode == 1 || a.M == 64 || a.nx <= kMT || a.nx > 2 * kMT || tiles <= 2 * device_sms();
 }
 

@@ -1055,6 +1055,17 @@ int tc_march_min_run(const StepArgs& a) {
   return t.pairs ? 4 : 2;
 }
 
+bool tc_march_shares(const StepArgs& a) {
+  // Three waves of 3xTF32 items: two and four solves on streams of their own,
+  // us for a step of all, in the passes and in multi-step launches, 256^2, M =
+  // 32: four groups 168, 306 and 189, 374; six 250, 457 and 238, 472; eight
+  // 324, 607 and 284, 564; sixteen 605, 1205 and 553, 1101; 512^2, M = 32, two
+  // groups 502, 982 and 442, 879; but 300^2, M = 64, four groups, bf16x3 654,
+  // 1321 and 776, 1546, and 160^2, M = 32, sixteen groups 276, 515 and 285, 564.
+  const PassTiles t(a);
+  return a.tc_mode == 1 && a.M < 64 && t.lo > 192 && 2 * t.most >= (t.pairs ? 6 : 3) * device_sms();
+}
+
 bool tc_march_dual(const StepArgs& a) {
   // Where one march leaves SMs without an item now and then, fewer than two
   // items of a pass for each.  256^2, M = 32, a gradient's step (forward,
