@@ -374,12 +374,12 @@ long long rte_graph_captures(const rte_ctx* ctx);
  *   1  (default) one-tile-per-CTA passes; in the tensor-core precisions,
  *      without RTE_FLAG_TC_SCATTER and with a line of more than 128
  *      positions, the same tiles as items of a persistent launch of up to
- *      32 steps (between checkpoints and snapshots), bit for bit the same
+ *      64 steps (between checkpoints and snapshots), bit for bit the same
  *      results, also in the segments of rte_adjoint_gradient.  A context on
  *      which no schedule was set, or whose schedule the autotuner set, takes
  *      these launches at the sizes and runs of steps where they are faster
  *      than two passes a step; schedule 1 set here, wherever supported.
- *      Such a launch keeps every SM (for up to about 5 ms; other work on the
+ *      Such a launch keeps every SM (for up to about 9 ms; other work on the
  *      GPU waits so long), so marches that do not fill the GPU by themselves
  *      take the passes while a march of this library is under way on another
  *      stream of the process, and for 50 ms after;

@@ -359,14 +359,16 @@ rte_status mark_fp32_end(rte_ctx* c) {
   return cuda_status(cudaEventRecord(c->fp32_end, c->stream));
 }
 
-// Steps of a multi-step launch, at most: 4.4 ms at 16 groups of 256^2, 1.4 ms
-// at one, so that other work gets its turn and a march learns soon that it is
-// no longer alone.  The ramp of a launch costs little of that: 256^2, 16
-// groups 276.3 us a step in launches of 128 steps, 277.9 of 16, 283.9 of 4;
-// one group 44.1, 44.9, 45.1; 200 x 131, three groups 43.3, 44.3, 49.1.
+// Steps of a multi-step launch, at most: 9 ms at 16 groups of 256^2, 3 ms at
+// one, so that other work gets its turn and a march learns soon that it is no
+// longer alone.  The ramp of a launch costs little of that: 256^2, 16 groups
+// 276.3 us a step in launches of 128 steps, 277.7 of 32, 277.9 of 16, 283.9 of
+// 4; one group 44.1, 44.9, 44.9, 45.1; 200 x 131, three groups 43.3, 43.7,
+// 44.3, 49.1 (80 steps in runs of 41 and 39 3723 us a call, of 32, 9, 32 and
+// 7 3773).
 int march_limit(const rte_kern::StepArgs& a) {
   const long long values = static_cast<long long>(a.G) * static_cast<long long>(a.plane);
-  return static_cast<int>(std::max<long long>(2, std::min<long long>(32, (1LL << 29) / values)));
+  return static_cast<int>(std::max<long long>(2, std::min<long long>(64, (1LL << 30) / values)));
 }
 
 // Keeps the host at most two launches of `limit` steps ahead of the GPU, so
