@@ -61,13 +61,13 @@ NCU_TRAFFIC = {
     # whose sources changed since its capture no longer matches.
     # multi-step march (csrc/rte_tc_march.cu + rte_tc_common.cuh), one launch
     # of 8 steps, per step: profiles/march_tomo256_ncu.md
-    ("tc_march_kernel", "25c766fede07c72f"): (6604.819200e6 + 3142.840320e6) / 8,
+    ("tc_march_kernel", "c475e751ecedc186"): (6603.971328e6 + 3144.515584e6) / 8,
     # tile-local fused step (csrc/rte_fused.cu), 16 x 16 parts:
     # profiles/fused_step_tomo256_ncu.md
     ("fused_step_kernel", "0a3a711e2bec192f"): 539.476224e6 + 230.795264e6,
     # its tensor-core form (csrc/rte_fused_tc.cu + rte_tc_common.cuh):
     # profiles/fused_step_tc_tomo256_ncu.md
-    ("fused_step_tc_kernel", "3bafd3fcf47785d7"): 539.331328e6 + 230.892800e6,
+    ("fused_step_tc_kernel", "97a3d4ea316cc6cb"): 539.561984e6 + 231.317248e6,
 }
 
 

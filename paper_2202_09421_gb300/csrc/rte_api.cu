@@ -54,9 +54,10 @@ struct rte_ctx {
   DevBuf err;
   bool inject_expire = false;
   // item counters of the multi-step launches, and the events that keep the
-  // host at most two launches ahead (Pace)
+  // host from running too far ahead (Pace)
   DevBuf ctl;
-  cudaEvent_t pace[2] = {nullptr, nullptr};
+  static constexpr int kAhead = 16;
+  cudaEvent_t pace[kAhead] = {};
   cudaEvent_t fp32_end = nullptr;  // behind the last FP32 forward (Marching)
   // photon balance of the last rte_forward (RTE_FLAG_PHOTON_BALANCE):
   // [G][n_steps][3] FP64 terms, block partials, per-group tickets, and the
@@ -322,6 +323,7 @@ class Marching {
   ~Marching() {
     std::lock_guard<std::mutex> hold(marches().lock);
     std::vector<cudaStream_t>& c = marches().calls;
+    if (beside()) marches().together = Marches::Clock::now();
     c.erase(std::find(c.begin(), c.end(), stream_));
   }
   Marching(const Marching&) = delete;
@@ -371,8 +373,12 @@ int march_limit(const rte_kern::StepArgs& a) {
   return static_cast<int>(std::max<long long>(2, std::min<long long>(64, (1LL << 30) / values)));
 }
 
-// Keeps the host at most two launches of `limit` steps ahead of the GPU, so
-// that the choice between launches and passes is made near the time it is for.
+// Keeps the host at most kAhead launches of `limit` steps ahead of the GPU (45
+// ms at one group of 256^2, 140 ms at sixteen), so that the choice between
+// launches and passes is made near the time it is for; far enough for a pause
+// of the host not to be one of the GPU (two launches ahead, one of three runs
+// of the benchmark took 594 ms a solve on a busy host, where all others took
+// 548 to 552).
 class Pace {
  public:
   Pace(rte_ctx* c, int limit) : c_(c), limit_(limit) {}
@@ -381,8 +387,9 @@ class Pace {
     steps_ = 0;
     for (cudaEvent_t& e : c_->pace)
       if (!e) RTE_TRY(cuda_status(cudaEventCreateWithFlags(&e, cudaEventDisableTiming)));
-    RTE_TRY(cuda_status(cudaEventRecord(c_->pace[n_ & 1], c_->stream)));
-    if (n_++ > 0) RTE_TRY(cuda_status(cudaEventSynchronize(c_->pace[n_ & 1])));
+    constexpr int kAhead = rte_ctx::kAhead;
+    RTE_TRY(cuda_status(cudaEventRecord(c_->pace[n_ % kAhead], c_->stream)));
+    if (++n_ >= kAhead) RTE_TRY(cuda_status(cudaEventSynchronize(c_->pace[n_ % kAhead])));
     return RTE_OK;
   }
 

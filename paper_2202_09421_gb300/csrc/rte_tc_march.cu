@@ -23,9 +23,10 @@
 //   warp 13, one lane   takes the tickets and copies the operator units (128
 //                       output positions x one K chunk, hi and lo) into a
 //                       ring;
-//   warps 8-11          convert the slab: a thread owns one slab column,
-//                       loads its values two pieces ahead into registers,
-//                       scales, splits and writes the K-major operand chunk;
+//   warps 8-11          convert the slab: a thread owns four neighbouring
+//                       slab columns, loads their values two pieces ahead
+//                       into registers, scales, splits and writes its part of
+//                       the K-major operand chunk;
 //   warp 12, one lane   issues the MMAs into one of two accumulators in
 //                       tensor memory;
 //   warps 0-7           the epilogue of the item before (x_epilogue,
@@ -70,7 +71,7 @@ constexpr int kMaxD = 4;                                       // ring slots, at
 // x-pass epilogue keeps its 8 KB of node values per warp at the warp's place
 // of that ring, so that a warp may go on to another item on its own.
 constexpr int kYPair = 2 * 5 * 512;                            // bytes of a warp's two rows
-constexpr int kYWarpBytes = 2 * kYPair;                        // 20 KB
+constexpr int kYWarpBytes = 2 * kYPair;                        // 10 KB
 constexpr size_t kYRingBytes = static_cast<size_t>(kEpiWarps) * kYWarpBytes;
 constexpr size_t kYTileBytes = 16 * kNC * 4;
 constexpr size_t kBcTabBytes = kMaxM * (8 * 8 + 4 * 4);

@@ -15,6 +15,12 @@ FP32, TF32X3 = 0, 1
 LATELY = 0.1                  # seconds after which a march beside another is forgotten
 
 
+@pytest.fixture(autouse=True)
+def forgotten():
+    yield
+    time.sleep(LATELY)                                   # other tests count the launches of a march alone
+
+
 def _wl(nx, ny, M, groups, steps):
     return workload_custom(nx, ny, M, steps, 0.02, L=(nx - 1) / 66, mus=80.0, n_groups=groups, t_s=0.1, sigma_t=0.1)
 
