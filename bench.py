@@ -61,7 +61,7 @@ NCU_TRAFFIC = {
     # whose sources changed since its capture no longer matches.
     # multi-step march (csrc/rte_tc_march.cu + rte_tc_common.cuh), one launch
     # of 8 steps, per step: profiles/march_tomo256_ncu.md
-    ("tc_march_kernel", "c475e751ecedc186"): (6603.971328e6 + 3144.515584e6) / 8,
+    ("tc_march_kernel", "384152f4a508eb20"): (6600.705536e6 + 3143.943936e6) / 8,
     # tile-local fused step (csrc/rte_fused.cu), 16 x 16 parts:
     # profiles/fused_step_tomo256_ncu.md
     ("fused_step_kernel", "0a3a711e2bec192f"): 539.476224e6 + 230.795264e6,

@@ -902,16 +902,23 @@ bool tc_supported(int nx, int ny, int M, int precision, int flags) {
 // whose MMAs are few (TF32, BF16): there the early CTAs stand where the last
 // ones of the y-pass could work off faster (160^2, M = 32, 16 groups, TF32
 // 146.1 -> 149.3; 256^2, 8 groups, BF16 159.7 -> 162.6; in 3xTF32 176.7 ->
-// 174.7 and 193.8 -> 192.3).  Beside other marches the early CTAs stand in the
+// 174.7 and 193.8 -> 192.3).  Nor where the x tiles would have an SM each and
+// the y tiles come in waves: the early CTAs crowd by twos on the SMs that are
+// free first (M = 32, 204 x 27, 17 groups, 3xTF32, 119 and 867 tiles 56.5 ->
+// 67.0; 217 x 56, 10 groups, BF16 49.1 -> 56.9; 184 x 45, 6 groups, bf16x3, 72
+// and 276 tiles 36.7 -> 41.3).  Beside other marches the early CTAs stand in the
 // way of those, unless they are few (four solves on streams of their own,
 // 3xTF32: 64^2, M = 16, one group 27.6 us a step as an ordinary launch, 24.0
 // as a dependent one, 128^2, M = 32 49.2 and 46.5; but 64^2, M = 32, four
 // groups 34.6 and 36.3, 24 x 256, M = 16, eight groups 74.5 and 97.1).
 static bool xpass_dependent(const StepArgs& a) {
-  const int per_tile = kNC / a.M;
-  const long long tiles = static_cast<long long>(a.G) * ((a.ny + per_tile - 1) / per_tile);
-  if (a.beside) return 3 * tiles <= device_sms();
-  return a.tc_mode == 1 || a.M == 64 || a.nx <= kMT || a.nx > 2 * kMT || tiles <= 2 * device_sms();
+  const int per_tile = kNC / a.M, sms = device_sms();
+  const long long tiles = static_cast<long long>(a.G) * ((a.ny + per_tile - 1) / per_tile),
+                  tiles_y = static_cast<long long>(a.G) * ((a.nx + per_tile - 1) / per_tile);
+  if (a.beside) return 3 * tiles <= sms;
+  if (a.M == 32 && a.nx > kMT && a.nx <= 2 * kMT && 5 * tiles > 2 * sms && tiles <= sms && 2 * tiles_y > 3 * sms)
+    return false;
+  return a.tc_mode == 1 || a.M == 64 || a.nx <= kMT || a.nx > 2 * kMT || tiles <= 2 * sms;
 }
 
 cudaError_t launch_step_tc(const StepArgs& a, const BoundaryArgs& b, float* U, float* R, const float* L1,

@@ -1010,28 +1010,38 @@ struct PassTiles {
 // lines are drawn through times at 1010 random sizes (16 to 512 positions, 1
 // to 24 groups, every precision and M), 40 steps in one run; the speed of the
 // passes is 1:
-//   taken: 620 sizes, geometric mean 1.24, 6 below 0.97 (the worst 0.90);
-//   left:  0.42 to 1.5 (206 x 21, M = 32, 22 groups, BF16 66 us a step in the
+//   taken: 696 sizes, geometric mean 1.25, 4 below 0.97 (the worst 0.94);
+//   left:  0.41 to 1.36 (206 x 21, M = 32, 22 groups, BF16 66 us a step in the
 //   passes, 130 here; 24 x 256, M = 16, 40 groups, 3xTF32 88 against 150;
 //   260 x 24, M = 32, 16 groups, TF32 60 against 113; 130 x 130, M = 16, 16
-//   groups, TF32 51 against 69), geometric mean 0.97.
+//   groups, TF32 51 against 69), geometric mean 0.94.
 bool march_pays(const StepArgs& a) {
   const PassTiles t(a);
   const int sms = device_sms();
   const bool x3tf32 = a.tc_mode == 1, bf16 = a.tc_mode == 4;
-  if (a.M == 16 && t.pairs && t.most > 2 * sms) return false;
+  const bool x_short = a.nx < a.ny;
+  if (a.M == 16 && t.pairs && t.most > 2 * sms) return x3tf32 && t.lo >= 160;
   if (a.M == 64 && t.lo >= 96 && t.most > sms) return true;
+  if (!bf16 && 4 * t.most <= sms) return true;
   if (x3tf32) {
+    if (a.M == 64 && (t.hi > 256 || (t.lo >= 32 && t.most > sms))) return true;
     if (t.hi > 400) return t.shorter <= 8 * sms || t.lo >= 40;
     if (t.lo >= 64 || (t.lo >= 40 && t.shorter <= 8 * sms)) return t.hi >= 152 || 2 * t.most <= sms;
-    return t.shorter <= sms && t.hi > 207;
+    return (t.shorter <= sms && t.hi >= 160) || (t.shorter <= (x_short ? 6 : 4) * sms && t.hi > 300);
   }
   if (t.hi < 152) return false;
-  if (t.hi > 432) return t.lo >= 32 && (!bf16 || a.nx < a.ny);
-  if (t.lo > 160) return !(t.pairs && t.most > sms && t.most <= 2 * sms);
-  if (a.nx < a.ny && t.hi > 256) return t.lo >= 56 || t.shorter <= sms;
-  if (bf16) return false;
-  if (a.M == 64) return t.lo >= 56;
+  if (!bf16) {
+    if (a.M == 64 && (t.hi > 300 || t.lo >= 40)) return true;
+    if ((x_short && t.hi > 300) || (2 * t.most <= sms && (t.lo > 64 || t.hi > 256))) return true;
+    if (t.hi > 360 && t.shorter <= sms) return true;
+  }
+  if (a.M == 32 && t.lo > kMT && t.most > 2 * sms) return true;
+  if (t.lo >= 152) {
+    const bool one_wave = t.pairs && t.most > sms && t.most <= 2 * sms && (a.M == 16 || bf16);
+    return !one_wave && !(bf16 && a.M < 64 && t.hi > 256 && t.hi <= 300);
+  }
+  if (t.hi > 432 && t.lo >= 32 && (!bf16 || x_short)) return true;
+  if (x_short && t.hi > 256) return t.lo >= 56 || t.shorter <= sms;
   return a.tc_mode == 2 && t.lo > kMT && t.hi >= 160 && t.most <= sms;
 }
 
@@ -1048,12 +1058,15 @@ int tc_march_min_run(const StepArgs& a) {
   // idle anyway (256^2, one group, a snapshot at every step: 58 us a step
   // against 90 in the passes) or the passes hold one CTA per SM (512^2, M =
   // 64: 329 against 458); runs of two do in 3xTF32 (120 sizes: 1.23 of the
-  // passes' speed on average), in the other precisions those of four.
+  // passes' speed on average), in the other precisions those of four (of two
+  // beside passes with one CTA per SM, but not with BF16 operands: 257 x 206, M
+  // = 64, ten groups, the balance of every step 574 us in the passes, 630 in
+  // launches of two steps).
   if (a.march_all) return 1;
   const PassTiles t(a);
   if (2 * t.most <= device_sms()) return 1;
   if (a.tc_mode == 1) return t.pairs ? 2 : 1;
-  return t.pairs ? 4 : 2;
+  return t.pairs || a.tc_mode == 4 ? 4 : 2;
 }
 
 bool tc_march_shares(const StepArgs& a) {
