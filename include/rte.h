@@ -98,7 +98,8 @@ typedef struct rte_optics {
 /* RTE_FLAG_CUDA_GRAPH runs the forward march (rte_forward,
  * rte_forward_batch) as a CUDA graph: captured on the first call, replayed
  * while the step count, groups and buffers stay the same, re-captured when
- * they change.  The graph runs on a private stream ordered after the
+ * they change or, in the tensor-core precisions, when marches on other streams
+ * come or go (rte_set_pass_variant).  The graph runs on a private stream ordered after the
  * context's stream by events, so the call stays asynchronous on that stream.
  * Off while per-kernel timing is on. */
 #define RTE_FLAG_CUDA_GRAPH 2

@@ -59,7 +59,7 @@ def _same(a, b):
     return all(torch.equal(x, y) for x, y in zip(a, b))
 
 
-@pytest.mark.parametrize("busy_steps,steps,graph", [(150, 20, False), (8, 2500, False), (150, 20, True)])
+@pytest.mark.parametrize("busy_steps,steps,graph", [(150, 20, False), (8, 4000, False), (150, 20, True)])
 def test_a_march_beside_another_takes_the_passes(busy_steps, steps, graph):
     """An FP32 forward (which returns before its work is done) under way on
     another stream for all, or for a part, of the march."""
